@@ -82,7 +82,7 @@ HBM_FALLBACK_GBS = 6800.0
 # (profiles/kernel_traffic_batched_256cloths.md), valid while the kernel's source
 # file is the one measured (its hash).
 TRAFFIC = {
-    "front": {"source": "dc_frontal.cu", "source_sha": "d56e13ad7997eba6", "bytes_per_launch": 945.14e6,
+    "front": {"source": "dc_front_factor.cu", "source_sha": "d56e13ad7997eba6", "bytes_per_launch": 945.14e6,
               "note": "ncu dram__bytes_read.sum + dram__bytes_write.sum, mean of the 9 levels of one "
                       "factorisation, 256 cloths (profiles/kernel_traffic_batched_256cloths.md)"},
     "sweeps": {"source": "dc_kernels.cu", "source_sha": "232ea24582784521", "bytes_per_launch": 747.46e6,
@@ -560,7 +560,7 @@ KERNEL_CLASSES = {
               "Signorini-Coulomb solve fused in)",
     "solve_fwd": "k_ps_fwd_tree (forward supernodal sweep, FP64, 3 columns)",
     "solve_bwd": "k_ps_bwd_tree (backward sweep + fused per-node Signorini-Coulomb solve)",
-    "front": "k_front_level (one level of the FP32 multifrontal LDL^T of the adjoint preconditioner)",
+    "front": "k_ff_* (one level of the FP32 multifrontal LDL^T of the adjoint preconditioner: extend, panels, updates, finish)",
     "msolve": "k_msolve_fwd_tree / k_msolve_bwd_tree (preconditioner solves)",
     "krylov": "k_bmdot / k_breduce / k_bvupdate / k_bscale (GMRES vectors)",
     "apply_h": "k_adj_elem + k_adj_gather (matrix-free adjoint operator)",

@@ -386,7 +386,7 @@ dc_status dc_global_solve_static(dc_ctx* ctx, const double* rhs, double* out);
  * skip_items outside [1, number of items). */
 dc_status dc_debug_sweep_wait_timeout(dc_ctx* ctx, int32_t skip_items);
 
-/* Testing the adjoint preconditioner's dense front kernel on its own: one
+/* Testing the adjoint preconditioner's front factorisation on its own: one
  * symmetric n x n front A (host, column-major FP32; the lower triangle is read)
  * with p pivot columns goes through the partial LDL^T that factorises every
  * front of the multifrontal preconditioner (Sec. 4, Eq. ppr_adjoint is the
@@ -394,14 +394,13 @@ dc_status dc_debug_sweep_wait_timeout(dc_ctx* ctx, int32_t skip_items);
  * afterwards: in its first p columns D on the diagonal and the unit-lower L
  * below it, in the trailing (n - p) x (n - p) lower triangle the Schur
  * complement A22 - L21 D L21^T.  linv_out (host, p x p column-major, nullable)
- * receives the inverse of L's unit-lower pivot block.  threads: 128, 256 or
- * 512; use_tc: 1 updates trailing blocks of 64 rows or more on the tensor
- * cores (TF32 split in three passes, FP32 accumulation), 0 by FP32 FMA tiles;
- * use_gscr: 1 keeps the panel scratch in global memory (the path of fronts
- * too large for shared memory).  Synchronous; allocates its own device memory.
- * DC_ERR_INVALID unless 1 <= p <= n <= 4096 (and the shared memory fits),
- * DC_ERR_TIMEOUT if a tensor-core completion wait gave up, DC_ERR_CUDA on a
- * CUDA error; dc_last_error(NULL) has the message. */
+ * receives the inverse of L's unit-lower pivot block.  threads (128, 256 or 512),
+ * use_tc and use_gscr named variants of an earlier one-CTA kernel; they are
+ * checked as before and change nothing else: every front goes through the same
+ * tiled launches.  Synchronous; allocates its own device memory.
+ * DC_ERR_INVALID unless 1 <= p <= n <= 4096 (without use_gscr a front must also
+ * fit the 227 KB that one CTA's panel took), DC_ERR_CUDA on a CUDA error;
+ * dc_last_error(NULL) has the message. */
 dc_status dc_debug_front_factor(int32_t n, int32_t p, const float* A, float* out, float* linv_out,
                                 int32_t threads, int32_t use_tc, int32_t use_gscr);
 

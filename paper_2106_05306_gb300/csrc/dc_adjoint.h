@@ -63,31 +63,23 @@ void adj_params(const DevMesh& dm, const AdjDev& ad, const Segs& sg, const d4* z
 void adj_add_ext(d4* g, const double* ext, const int* int2ext, int m, int layout, cudaStream_t s);
 
 // Per-step multifrontal LDL^T preconditioner (dc_frontal.cu).
-size_t frontal_factor_smem(int max_f, int max_p, bool tc);
-bool frontal_level_tc(int max_f);
-dc_status frontal_debug_factor(int n, int p, const float* A, float* out, float* linv_out, int threads, int tc,
-                               int use_gscr, std::string* err);
-// a factorisation CTA with its panel scratch in global memory: shared bytes, and
-// global floats per CTA
-size_t frontal_factor_smem_small(bool tc);
-long frontal_factor_gscr(int max_f, int max_p);
+// Numeric factorisation of the fronts (dc_front_factor.cu): the tile lists of its
+// launches, laid out once per front structure, and one factorisation.
+void ff_plan(const HostFronts& fr, FrontPlan& plan, std::vector<int2>& tasks);
+void ff_factorize(const FrontDev& fd, const FrontPlan& plan, cudaStream_t s, KTimer* kt);
+dc_status ff_debug_factor(int n, int p, const float* A, float* out, float* linv_out, std::string* err);
 size_t frontal_solve_smem(int max_f);
-// Raises the shared-memory limits of the factorisation kernel (to factor_bytes)
-// and of the solve kernels (fronts of up to max_f unknowns).
-cudaError_t frontal_configure(size_t factor_bytes, int max_f);
-// Fronts per level that exceed the shared memory of one CTA: the global scratch
-// (floats) their level launch needs, the largest over the levels (0 if none),
-// and the largest shared-memory size of the other levels.
-void frontal_plan(const HostFronts& fr, size_t smem_limit, long* gscr_floats, size_t* factor_bytes);
+// Raises the shared-memory limits of the solve kernels (fronts of up to max_f unknowns).
+cudaError_t frontal_configure(int max_f);
 // Launch shape of the tree-scheduled solves for fronts of at most max_f
 // unknowns: the CTAs of each kernel that fit on the device at once, and the
 // dynamic shared memory.
 cudaError_t frontal_tree_grid(int max_f, int* grid_f, int* grid_b, size_t* smem);
-// lvl_ptr / lvl_maxf / lvl_maxp: host arrays, the fronts of level l are
-// lvl_sn[lvl_ptr[l] .. lvl_ptr[l+1]), the largest has lvl_maxf[l] unknowns and
-// the largest pivot block lvl_maxp[l].
-void frontal_factorize(const DevMesh& dm, const AdjDev& ad, const FrontDev& fd, const int* lvl_ptr, int nlev,
-                       const int* lvl_maxf, const int* lvl_maxp, cudaStream_t s, KTimer* kt = nullptr);
+// Assembles the constrained matrix into the fronts and factorises them.
+void frontal_factorize(const DevMesh& dm, const AdjDev& ad, const FrontDev& fd, const FrontPlan& plan, cudaStream_t s,
+                       KTimer* kt = nullptr);
+// lvl_ptr / lvl_maxf: host arrays, the fronts of level l are
+// lvl_sn[lvl_ptr[l] .. lvl_ptr[l+1]), the largest has lvl_maxf[l] unknowns.
 // act_sn / act_ptr (optional): device list of the fronts to solve, level l at
 // act_sn[act_ptr[l] .. act_ptr[l+1]) (act_ptr on the host); fronts of masked
 // instances may be listed (they exit at once), active ones must be.  With

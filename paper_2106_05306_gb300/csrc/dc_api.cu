@@ -582,10 +582,21 @@ dc_status dc_get_instance_nonconverged(dc_ctx* c, int64_t* counts) {
     return DC_OK;
 }
 
+static size_t one_cta_front_bytes(int n, int p, bool tc) {
+    const size_t panel = 2 * 32 * 33 + 32 + 32 * (((size_t)n + 7) / 8 * 8), inverse = 64 * ((size_t)p + 1) + 1024;
+    return ((tc ? 12288 : 0) + std::max(panel, inverse)) * sizeof(float) + 64;
+}
+
 dc_status dc_debug_front_factor(int32_t n, int32_t p, const float* A, float* out, float* linv_out,
                                 int32_t threads, int32_t use_tc, int32_t use_gscr) {
     std::string err;
-    const dc_status st = frontal_debug_factor(n, p, A, out, linv_out, threads, use_tc, use_gscr, &err);
+    dc_status st = DC_ERR_INVALID;
+    if (n < 1 || p < 1 || p > n || n > 4096 || (threads != 128 && threads != 256 && threads != 512))
+        err = "dc_debug_front_factor: needs 1 <= p <= n <= 4096 and 128, 256 or 512 threads";
+    else if (!use_gscr && one_cta_front_bytes(n, p, use_tc != 0) > 227 * 1024)
+        err = "dc_debug_front_factor: front too large for shared memory; set use_gscr";
+    else
+        st = ff_debug_factor(n, p, A, out, linv_out, &err);
     if (st != DC_OK) g_create_err = err;
     return st;
 }

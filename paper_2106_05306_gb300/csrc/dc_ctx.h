@@ -72,10 +72,10 @@ struct dc_ctx {
     cudaEvent_t ev_block = nullptr;
     size_t dev_bytes = 0, dev_peak = 0;   // device bytes held now / at most
     HostFronts fr;
+    FrontPlan fplan;               // launches of one factorisation of the fronts
     FrontDev fdv{};
     int nlev = 0;
     std::vector<int> lvl_maxf;     // largest front of every level
-    std::vector<int> lvl_maxp;     // largest pivot block of every level
     std::vector<int> lvl_maxfs;    // ... in nodes (supernodal substitution)
     std::vector<int> ps_lvl_ptr, ps_nbig, ps_nsmall, ps_maxbig;   // supernodal level lists (large, then small)
     int* d_int2ext = nullptr;

@@ -320,6 +320,16 @@ void launch_mass_solve(const DevMesh& dm, const DevParams& P, const d4* b, d4* v
 void launch_count_cases(const int* contact, const int* case_, int m_free,
                         unsigned long long* counters, cudaStream_t s);
 
+// Launches of one numeric factorisation of the fronts, in order (dc_front_factor.cu):
+// launch q works on the tiles FrontDev::tasks[begin .. begin + count).
+enum { FF_EXTEND = 0, FF_PANEL = 1, FF_UPDATE = 2, FF_FINISH = 3 };
+struct FrontLaunch {
+    int kind, k, level, begin, count;  // k: panel (FF_PANEL, FF_UPDATE)
+};
+struct FrontPlan {
+    std::vector<FrontLaunch> launches;
+};
+
 // Device view of the multifrontal structure and its per-step numeric storage.
 struct FrontDev {
     int S, NP, max_f;
@@ -331,7 +341,7 @@ struct FrontDev {
     const int* p;
     const long long* off;
     const long long* acc_off;
-    const long long* binv_off;         // per front: offset of its diagonal-block inverses
+    const long long* binv_off;         // per front: offset of its factorised diagonal blocks
     const long long* linv_off;         // per front: offset of the inverse of its pivot block
     const int* uptr;
     const int* unode;
@@ -348,7 +358,7 @@ struct FrontDev {
     const double* pr_coef;
     float* pool;                       // fronts (lower triangles used)
     float* acc;                        // per-front update vectors of the forward solve
-    float* binv;                       // inverses of the 32x32 unit-lower diagonal blocks
+    float* binv;                       // factorised 32x32 diagonal blocks (L below, D on the diagonal)
     float* linv;                       // inverses of the unit-lower pivot blocks (p x p, column-major)
     float* rvec;                       // [3 m_free] right-hand side
     float* zvec;                       // [3 m_free] D^-1 L^-1 r
@@ -369,8 +379,5 @@ struct FrontDev {
     unsigned long long* fault;         // sticky: set when a dependency wait gave up
     int tree_grid_f, tree_grid_b;      // host: CTAs of a tree-scheduled launch
     size_t tree_smem;                  // host: its dynamic shared memory
-    // factorisation levels whose CTAs need more than smem_limit bytes of shared
-    // memory keep their panel scratch in gscr instead (per CTA, per slot)
-    size_t smem_limit;                 // host
-    float* gscr;
+    const int2* tasks;                 // tile lists of the factorisation (FrontPlan)
 };

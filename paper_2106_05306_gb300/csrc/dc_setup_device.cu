@@ -423,21 +423,15 @@ dc_status upload_params(dc_ctx* c, ParamPrep& pp) {
     int dev = 0, smem_optin = 0;
     CK(cudaGetDevice(&dev));
     CK(cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    // levels whose fronts do not fit one CTA's shared memory factorise with a
-    // global scratch instead (the top fronts of large meshes)
-    long gscr_floats = 0;
-    size_t factor_bytes = 0;
-    frontal_plan(frm, (size_t)smem_optin, &gscr_floats, &factor_bytes);
     if (frontal_solve_smem(frm.max_f) > (size_t)smem_optin) {
         c->err = "dc_set_params: the largest front (" + std::to_string(frm.max_f) +
                  " unknowns) exceeds the shared memory of one solve CTA";
         return DC_ERR_INVALID;
     }
-    CK(frontal_configure(factor_bytes, frm.max_f));
+    CK(frontal_configure(frm.max_f));
     free_pool(c, c->front_allocs);
     auto& F = c->front_allocs;
     FrontDev fd{};
-    fd.smem_limit = (size_t)smem_optin;
     fd.S = frm.S;
     fd.NP = (int)frm.pr_i.size();
     fd.max_f = frm.max_f;
@@ -491,6 +485,13 @@ dc_status upload_params(dc_ctx* c, ParamPrep& pp) {
     fd.pr_coef = d_pcoef;
     fd.tau = d_tau;
     fd.sn_inst = d_sninst;
+    int2* d_tasks;
+    {
+        std::vector<int2> tasks;
+        ff_plan(frm, c->fplan, tasks);
+        if ((s = upload(c, F, &d_tasks, tasks))) return s;
+    }
+    fd.tasks = d_tasks;
     // tree-scheduled solves: the fronts in a topological order (children first);
     // DC_LEVEL_SOLVES=1 in the environment selects one launch per tree level
     // instead (same results)
@@ -525,10 +526,6 @@ dc_status upload_params(dc_ctx* c, ParamPrep& pp) {
         (s = dalloc(c, F, &c->fds[1].binv, (size_t)frm.binv_size)) ||
         (s = dalloc(c, F, &c->fds[1].linv, (size_t)frm.linv_size)))
         return s;
-    for (int k = 0; k < 2; ++k) {
-        c->fds[k].gscr = nullptr;
-        if (gscr_floats > 0 && (s = dalloc(c, F, &c->fds[k].gscr, (size_t)gscr_floats, false))) return s;
-    }
     c->fdv = c->fds[0];
     // supernodal substitution of P (global_solver 1) on the same partition
     dm.solver = pp.q[0].global_solver;
@@ -628,13 +625,9 @@ dc_status upload_params(dc_ctx* c, ParamPrep& pp) {
         }
     c->nlev = (int)frm.lvl_ptr.size() - 1;
     c->lvl_maxf.assign(std::max(c->nlev, 0), 0);
-    c->lvl_maxp.assign(std::max(c->nlev, 0), 0);
     for (int l = 0; l < c->nlev; ++l)
         for (int q = frm.lvl_ptr[l]; q < frm.lvl_ptr[l + 1]; ++q)
             c->lvl_maxf[l] = std::max(c->lvl_maxf[l], frm.f[frm.lvl_sn[q]]);
-    for (int l = 0; l < c->nlev; ++l)
-        for (int q = frm.lvl_ptr[l]; q < frm.lvl_ptr[l + 1]; ++q)
-            c->lvl_maxp[l] = std::max(c->lvl_maxp[l], frm.p[frm.lvl_sn[q]]);
     c->front_flops = pp.front_flops;
     c->factor_nnz = pp.factor_nnz;
     c->fwd_nnz = (long long)hfm.fval.size();
@@ -715,20 +708,16 @@ size_t estimate_device_bytes(const dc_ctx* c, const MeshPrep& mp, const ParamPre
     add(vbytes(r.child)); add(vbytes(r.cmap)); add(vbytes(r.lvl_sn)); add(vbytes(r.pr_i)); add(vbytes(r.pr_j));
     add(vbytes(r.pr_dst)); add(vbytes(r.pr_ld)); add(vbytes(r.pr_cptr)); add(vbytes(r.pr_code));
     add(vbytes(r.pr_coef)); add(vbytes(pp.tau)); add(vbytes(pp.tau));
-    long gscr_floats = 0;
-    size_t factor_bytes = 0;
-    int dev = 0, optin = 227 * 1024;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
-        cudaGetLastError();
-        optin = 227 * 1024;   // host-only estimate without a device: the GB300 limit
+    {
+        FrontPlan plan;
+        std::vector<int2> tasks;
+        ff_plan(r, plan, tasks);
+        add(vbytes(tasks));
     }
-    frontal_plan(r, (size_t)optin, &gscr_floats, &factor_bytes);
     for (int s = 0; s < 2; ++s) {
         add(4 * (size_t)r.pool_size);
         add(4 * (size_t)r.binv_size);
         add(4 * (size_t)r.linv_size);
-        if (gscr_floats > 0) add(4 * (size_t)gscr_floats);
     }
     add(4 * (size_t)r.acc_size); add(12 * MF); add(12 * MF); add(12 * MF);
     add(4 * (size_t)r.S); add(4 * (size_t)r.S); add(8 * ((size_t)r.S + 1));   // tree order, parents, tickets/flags
