@@ -566,8 +566,8 @@ dc_status dc_debug_sweep_wait_timeout(dc_ctx* c, int32_t skip_items) {
         c->err = "dc_debug_sweep_wait_timeout: needs global_solver 1 with tree-scheduled sweeps";
         return DC_ERR_INVALID;
     }
-    if (skip_items < 1 || skip_items >= c->dm.ps.n_items) {
-        c->err = "dc_debug_sweep_wait_timeout: skip_items outside [1, " + std::to_string(c->dm.ps.n_items) + ")";
+    if (skip_items < 1 || skip_items >= c->dm.ps.n_ftask) {
+        c->err = "dc_debug_sweep_wait_timeout: skip_items outside [1, " + std::to_string(c->dm.ps.n_ftask) + ")";
         return DC_ERR_INVALID;
     }
     launch_solve_fwd_skip(c->dm, c->b, c->y, skip_items, c->stream);

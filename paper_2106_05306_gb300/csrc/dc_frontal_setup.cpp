@@ -311,6 +311,87 @@ void dc_build_tree_items(const HostFronts& fr, std::vector<int>& tq_ptr, std::ve
     }
 }
 
+// Tasks of the tree-scheduled supernodal sweeps, fronts farthest from their root
+// first (backward: nearest first).  Fronts of one depth stay together: half A of the
+// large ones and the small ones, then half B, so that a CTA waiting for a half A seldom
+// holds up a task that is ready.
+// A large front whose two products have at most `target` entries is one task; else
+// each half is cut into row blocks of about that many: 32 tasks per SM and sweep,
+// within [1600, 8192] entries (1600 entries, 4800 FMAs over the three columns, take an
+// SM 1.4 us, about the cost of starting a task; 3200 measured 20% slower on one
+// 100 x 100 cloth).  Small fronts go one to a CTA while there are at most eight of
+// them per SM -- alone on a CTA a small front takes about 1 us of FP64 time instead of
+// 6 us on one of its eight warps -- and in groups of a warp each beyond that, where
+// every SM has other work (200 x 200 nodes, 12 per SM: 24.0 ms in groups, 30.5 alone).
+// No choice here changes a bit of the result.
+void dc_build_ps_tasks(const HostFronts& fr, const std::vector<int>& tq_ptr, const std::vector<int>& tq_sn,
+                       std::vector<int4>& ftask, std::vector<int4>& btask, std::vector<int4>& need, bool& alone) {
+    constexpr int SMS = 152;
+    auto large = [&](int s) { return fr.f[s] / 3 > DC_PS_SMALL; };
+    long long total = 0;
+    int n_small = 0;
+    for (int s = 0; s < fr.S; ++s) {
+        const long long ns = fr.p[s] / 3, nu = fr.f[s] / 3 - ns;
+        total += ns * (ns + 1) / 2 + ns * nu;
+        n_small += !large(s);
+    }
+    const long long target = std::min<long long>(8192, std::max<long long>(1600, total / (SMS * 32)));
+    alone = n_small <= 8 * SMS;
+    need.assign(fr.S, make_int4(1, 0, 1, 0));
+    ftask.clear();
+    btask.clear();
+    // row blocks of a half whose row i has work(i) entries; multiples of 4 rows (a
+    // 32-byte sector of every column)
+    auto blocks = [&](std::vector<int4>& out, int s, int phase, int rows, auto work) {
+        int n = 0;
+        for (int r = 0; r < rows; ++n) {
+            long long w = 0;
+            int e = r;
+            while (e < rows && (w < target || e % 4)) w += work(e++);
+            out.push_back(make_int4(s, phase, r, e));
+            r = e;
+        }
+        return n;
+    };
+    std::vector<int> depth(fr.S, 0);
+    for (int s = fr.S - 1; s >= 0; --s) depth[s] = fr.parent[s] >= 0 ? depth[fr.parent[s]] + 1 : 0;
+    const int n_items = (int)tq_ptr.size() - 1;
+    std::vector<std::pair<int, int>> span;   // items of one depth
+    for (int q = 0; q < n_items;) {
+        int e = q;
+        while (e < n_items && depth[tq_sn[tq_ptr[e]]] == depth[tq_sn[tq_ptr[q]]]) ++e;
+        span.push_back({q, e});
+        q = e;
+    }
+    auto emit = [&](std::vector<int4>& out, const std::pair<int, int>& sp, bool fwd) {
+        for (int second = 0; second < 2; ++second)
+            for (int q = sp.first; q < sp.second; ++q) {
+                const int s = tq_sn[tq_ptr[q]];
+                const long long ns = fr.p[s] / 3, nu = fr.f[s] / 3 - ns;
+                if (!large(s)) {
+                    if (second) continue;
+                    if (alone)
+                        for (int e = tq_ptr[q]; e < tq_ptr[q + 1]; ++e) out.push_back(make_int4(tq_sn[e], PS_FRONT, 0, 0));
+                    else
+                        out.push_back(make_int4(tq_ptr[q], PS_GROUP, tq_ptr[q + 1] - tq_ptr[q], 0));
+                } else if (ns * (ns + 1) / 2 + ns * nu <= target) {
+                    if (!second) out.push_back(make_int4(s, PS_AB, 0, 0));
+                } else if (fwd && !second) {
+                    (nu > 0 ? need[s].y : need[s].x) =
+                        blocks(out, s, PS_A, (int)ns, [&](int i) { return (long long)i + 1; });
+                } else if (fwd && nu > 0) {
+                    need[s].x = blocks(out, s, PS_B, (int)nu, [&](int) { return ns; });
+                } else if (!fwd && !second && nu > 0) {
+                    need[s].w = blocks(out, s, PS_A, (int)ns, [&](int) { return nu; });
+                } else if (!fwd && second) {
+                    need[s].z = blocks(out, s, PS_B, (int)ns, [&](int i) { return ns - i; });
+                }
+            }
+    };
+    for (const auto& sp : span) emit(ftask, sp, true);
+    for (size_t k = span.size(); k-- > 0;) emit(btask, span[k], false);
+}
+
 // For every front s and node position t of s (t < f_s / 3, pivots first): the
 // update-vector entries of s's children that add into t, children in cptr order
 // and entries in ascending order (entry j of child c is aoff[c] + stride j), so that a gather summing them in list order

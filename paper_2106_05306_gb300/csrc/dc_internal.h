@@ -120,8 +120,12 @@ struct HostPSolve {
 // values = false: offsets and sizes only (the GPU factorisation fills the panels)
 void dc_build_psolve(const HostFactor& hf, const HostFronts& fr, HostPSolve& ps, bool values = true);
 void dc_merge_psolve(const std::vector<HostPSolve>& P, HostPSolve& out);
-// Work items of the tree-scheduled sweeps (see PSolveDev::tq_ptr)
+// Work items of the tree-scheduled sweeps, in topological order
 void dc_build_tree_items(const HostFronts& fr, std::vector<int>& tq_ptr, std::vector<int>& tq_sn);
+// Tasks of the tree-scheduled supernodal sweeps from those items (PSolveDev::ftask,
+// btask, need, alone)
+void dc_build_ps_tasks(const HostFronts& fr, const std::vector<int>& tq_ptr, const std::vector<int>& tq_sn,
+                       std::vector<int4>& ftask, std::vector<int4>& btask, std::vector<int4>& need, bool& alone);
 // Pull lists of the forward solves' child gather (see PSolveDev::pull_off and
 // FrontDev::pull_off): entry j of child c's update vector is aoff[c] + stride j
 void dc_build_pull_lists(const HostFronts& fr, const std::vector<int>& aoff, int stride, std::vector<int>& pull_off,
@@ -134,6 +138,10 @@ void dc_build_pull_lists(const HostFronts& fr, const std::vector<int>& aoff, int
 constexpr int DC_PS_SMALL = 64;
 // small fronts solved together by one CTA (one per warp)
 constexpr int DC_PS_WARPS = 8;
+// A task (x, y, z, w) of the tree-scheduled sweeps: y says what it is, PS_GROUP the z
+// small fronts tq_sn[x ..), a warp each; PS_FRONT the small front x on a whole CTA;
+// PS_AB the large front x; PS_A / PS_B rows [z, w) of its first / second half.
+enum { PS_A = 0, PS_B = 1, PS_AB = 2, PS_GROUP = 3, PS_FRONT = 4 };
 
 // Device view of the supernodal substitution (global_solver 1): the front
 // partition (node-level counts are the fronts' DOF counts / 3) and the panels.
@@ -164,23 +172,27 @@ struct PSolveDev {
     const double* xinvt;
     d4* acc;                           // update vectors of the forward sweep (nodes)
     d4* xint;                          // solution of the backward sweep before any per-node update
-    // tree-scheduled sweeps (one launch per sweep): work items in a topological
-    // order, children first; item q is the fronts tq_sn[tq_ptr[q] .. tq_ptr[q+1]),
-    // one large front or up to DC_PS_WARPS small ones of equal depth
+    // tree-scheduled sweeps: tasks in a topological order (forward: children first;
+    // backward: parents first) and, per front, how many tasks end each of its phases
+    // (forward, forward half A, backward, backward half A)
     int tree;                          // 1: tree-scheduled sweeps, 0: one launch per level
-    int S, n_items;
+    int S, n_ftask, n_btask;
+    const int4* ftask;
+    const int4* btask;
+    const int4* need;                  // [S]
+    d4* wbuf;                          // [m_free] w_s between the halves of the backward sweep
     const int* parent;                 // [S] parent front, -1 at a root
-    const int* tq_ptr;
-    const int* tq_sn;
+    const int* tq_sn;                  // small fronts, group by group
     // gather of the children's update vectors into front s: position t < fs/3
     // sums acc[pull_idx[e]] for e in [pull_ptr[pull_off[s] + t], pull_ptr[pull_off[s] + t + 1]),
     // children in cptr order
     const int* pull_off;               // [S]
     const int* pull_ptr;
     const int* pull_idx;
-    int* sched;                        // [2][S + 1]: ticket counter, then per-front done flags (fwd; bwd)
+    int* sched;                        // [2][2 S + 1]: ticket counter, tasks done per front, half-A tasks done (fwd; bwd)
     unsigned long long* fault;         // sticky: set when a dependency wait gave up
-    int tree_grid_f, tree_grid_b;      // host: CTAs of a tree-scheduled launch (fwd, bwd)
+    int alone;                         // host: 1: no PS_GROUP tasks
+    int tree_grid;                     // host: CTAs of a tree-scheduled launch
     size_t tree_smem;                  // host: its dynamic shared memory
     int fused;                         // host: 1: both sweeps of a global step as one launch
 };
@@ -298,9 +310,8 @@ cudaError_t psolve_configure(int max_fs);
 // the launch (testing the bounded waits: those items never run).
 void launch_solve_fwd_skip(const DevMesh& dm, const d4* b, d4* y, int skip, cudaStream_t s);
 // Launch shape of the tree-scheduled sweeps whose largest CTA-path front has
-// max_fs nodes: the CTAs of each kernel that fit on the device at once, and the
-// dynamic shared memory
-cudaError_t psolve_tree_grid(int max_fs, int* grid_f, int* grid_b, size_t* smem);
+// max_fs nodes: the CTAs that fit on the device at once, and the dynamic shared memory
+cudaError_t psolve_tree_grid(int max_fs, bool alone, int* grid, size_t* smem);
 // x_{n+1} = x_n + h v; sets *nonfinite when a state entry is not finite
 void launch_finalize(const DevMesh& dm, const DevParams& P, const d4* x_n, const d4* v,
                      d4* x_np1, unsigned long long* nonfinite, cudaStream_t s);

@@ -342,6 +342,19 @@ __device__ __forceinline__ int coulomb(double mu, double c, const double n[3], d
     return 2;
 }
 
+// The contact update of one node (out of line: few nodes take it, and inlined it sets
+// the register count of every kernel that ends in finish_row).
+__device__ __noinline__ void contact_row(double s0, double s1, double s2, double mu, double c, const d4* nb, d4* f,
+                                         d4* out, int* case_) {
+    const d4 q = ld(nb), fo = ld(f);
+    const double n[3] = {q.x, q.y, q.z};
+    const double vt[3] = {s0 - c * fo.x, s1 - c * fo.y, s2 - c * fo.z};
+    double v[3], fn[3];
+    *case_ = coulomb(mu, c, n, q.w, vt, v, fn);
+    st(f, fn[0], fn[1], fn[2]);
+    st(out, v[0], v[1], v[2]);
+}
+
 // Output of one row of the backward substitution: mode 0 stores it; mode 1
 // applies the node's Signorini-Coulomb update (contact nodes) and stores v; mode 2
 // stores the compliance c_j = h s0.
@@ -354,14 +367,7 @@ __device__ __forceinline__ void finish_row(const DevParams& P, int row, double s
         return;
     }
     if (mode == 1 && contact[row] >= 0) {
-        d4 q = ld(nb + row), fo = ld(f + row);
-        double c = cc[row];
-        double n[3] = {q.x, q.y, q.z};
-        double vt[3] = {s0 - c * fo.x, s1 - c * fo.y, s2 - c * fo.z};
-        double v[3], fn[3];
-        case_[row] = coulomb(P.node_mu[row], c, n, q.w, vt, v, fn);
-        st(f + row, fn[0], fn[1], fn[2]);
-        st(out + row, v[0], v[1], v[2]);
+        contact_row(s0, s1, s2, P.node_mu[row], cc[row], nb + row, f + row, out + row, case_ + row);
         return;
     }
     st(out + row, s0, s1, s2);
@@ -379,170 +385,342 @@ __global__ void k_solve_bwd(DevMesh dm, DevParams P, const d4* __restrict__ y, d
     finish_row(P, row, s0, s1, s2, out, mode, contact, nb, cc, f, case_, c_out);
 }
 
-// Issues L2 prefetches for [p, p + bytes) (128-byte lines, spread over the CTA),
-// so that a front's blocks stream in from HBM while the CTA gathers its inputs.
-__device__ __forceinline__ void prefetch_l2(const void* p, size_t bytes) {
-    const char* c = static_cast<const char*>(p);
-    for (size_t o = (size_t)threadIdx.x * 128; o < bytes; o += (size_t)blockDim.x * 128)
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(c + o));
-}
+// ---- supernodal substitution (global_solver 1): leaves-first for L y = b and
+// root-first for L^T x = y, three right-hand sides.  Per front, with w its gathered
+// right-hand side:
+//   forward   half A  y_s = L_ss^-1 w_s             half B  acc = w_U - L_Us y_s
+//   backward  half A  w_s = y_s - L_Us^T x_U        half B  x_s = L_ss^-T w_s.
 
-// ---- supernodal substitution (global_solver 1): one CTA per supernode, levels
-// leaves-first for L y = b and root-first for L^T x = y, three right-hand sides.
-// Shared memory holds the front's vectors component-major ([3][n]).
-
-// Column-major product on one CTA with three right-hand sides: t_c,i = sum_k
-// A[k * lda + i] v[c * ldv + k] for i < nrows and k < K (tri 1: only k <= i;
-// tri 2: only k >= i).  Rows go in passes of GV_ROWS; the k range is cut into G
-// contiguous chunks with G a function of K alone.  Every (row, chunk) pair with
-// a nonempty k range is one work item -- the pairs are numbered chunk by chunk,
-// so that the triangle's empty pairs take no lanes -- and a row's partial sums
-// are added in chunk order.  The result depends only on (nrows, K), never on the
-// CTA size (a supernode gives the same bits whatever else shares its launch).
-// fin(i, t0, t1, t2) stores (it must not write v).
-constexpr int GV_ROWS = 128;
+// Fronts of at most PS_SMALL nodes sum a row in plain k order, one lane per (row,
+// column of the right-hand side); larger fronts cut the k range of a row into at most
+// GV_MAXG chunks, their number a function of its length K alone, and add the chunks in
+// order.  A row's result depends only on its front, never on which CTA, warp, lane or
+// rows share its task.
+constexpr int PS_SMALL = DC_PS_SMALL;
+constexpr int PS_WARPS = DC_PS_WARPS;      // small fronts per CTA when they go in groups
+constexpr int PS_LD = PS_SMALL + 1;        // shared-memory column stride of a small front (no bank conflicts)
+constexpr int GV_ROWS = 128;               // rows of one pass
 constexpr int GV_MAXG = 8;
+constexpr int PS_CH = 16;                  // entries of an item loaded before a wait
 __host__ __device__ constexpr int gv_groups(int K) { return K <= 8 ? 1 : (K + 7) / 8 < GV_MAXG ? (K + 7) / 8 : GV_MAXG; }
 
-template <class Fin>
-__device__ __forceinline__ void cm_gemv3(const double* __restrict__ A, long lda, int nrows, int K, int tri,
-                                         const double* __restrict__ v, int ldv, double* __restrict__ red, Fin fin) {
-    const int nt = blockDim.x, tid = threadIdx.x;
-    const int G = gv_groups(K);
-    const int C = (K + G - 1) / G;
-    constexpr int RS = GV_ROWS * GV_MAXG;      // stride between the three columns' partial sums
-    for (int i0 = 0; i0 < nrows; i0 += GV_ROWS) {
-        const int R = min(GV_ROWS, nrows - i0);
-        // rows [lo(g), hi(g)) of this pass have a nonempty k range in chunk g
-        auto lo = [&](int g) { return tri == 1 ? min(R, max(0, g * C - i0)) : 0; };
-        auto hi = [&](int g) { return tri == 2 ? max(0, min(R, (g + 1) * C - i0)) : R; };
-        int n_items = 0;
-        for (int g = 0; g < G; ++g) n_items += max(0, hi(g) - lo(g));
-        for (int item = tid; item < n_items; item += nt) {
-            int g = 0, base = 0;
-            for (;; ++g) {
-                const int n = max(0, hi(g) - lo(g));
-                if (item < base + n) break;
-                base += n;
-            }
-            const int r = lo(g) + item - base, i = i0 + r;
-            int k0 = g * C;
-            int k1 = min(K, k0 + C);
-            if (tri == 1) k1 = min(k1, i + 1);
-            if (tri == 2) k0 = max(k0, i);
-            const double* a = A + i;
-            double a0 = 0.0, a1 = 0.0, a2 = 0.0;
-#pragma unroll 4
-            for (int k = k0; k < k1; ++k) {
-                const double x = a[(long)k * lda];
-                a0 += x * v[k];
-                a1 += x * v[ldv + k];
-                a2 += x * v[2 * ldv + k];
-            }
-            red[g * GV_ROWS + r] = a0;
-            red[RS + g * GV_ROWS + r] = a1;
-            red[2 * RS + g * GV_ROWS + r] = a2;
-        }
-        __syncthreads();
-        if (tid < R) {
-            double t0 = 0.0, t1 = 0.0, t2 = 0.0;
-            for (int q = 0; q < G; ++q) {
-                if (tid < lo(q) || tid >= hi(q)) continue;
-                t0 += red[q * GV_ROWS + tid];
-                t1 += red[RS + q * GV_ROWS + tid];
-                t2 += red[2 * RS + q * GV_ROWS + tid];
-            }
-            fin(i0 + tid, t0, t1, t2);
-        }
-        __syncthreads();
-    }
+// The entries of the children's update vectors that add into position t of a front
+// (pull list pp, children in order), then b_t for a pivot (bt not null).  The list is
+// read before the CTA's dependency wait (ps_pull_begin), the vectors after it.  The sums
+// are those of a child-by-child scatter into zeroed storage, in the same order.
+struct PsPull {
+    int e0, e1, i0, i1;
+};
+__device__ __forceinline__ PsPull ps_pull_begin(const PSolveDev& ps, const int* __restrict__ pp, int t) {
+    PsPull q;
+    q.e0 = pp[t];
+    q.e1 = pp[t + 1];
+    q.i0 = q.e0 < q.e1 ? ps.pull_idx[q.e0] : 0;
+    q.i1 = q.e0 + 1 < q.e1 ? ps.pull_idx[q.e0 + 1] : 0;
+    return q;
 }
-
-// Fronts of at most PS_SMALL nodes take the warp path: one warp per front,
-// warp-synchronous, sums in plain k order; larger fronts take the CTA path.  A
-// front's path depends only on its own size, so its bits do not depend on what
-// else shares its level.
-constexpr int PS_SMALL = DC_PS_SMALL;
-constexpr int PS_WARPS = DC_PS_WARPS;    // small fronts per CTA
-constexpr int PS_LD = PS_SMALL + 1;       // shared-memory column stride of the warp path (no bank conflicts)
-
-// Right-hand side of position t of a front: the children's update entries that
-// add into t (pull list pp, children in order), then b_t for a pivot (bt not
-// null); the three columns go to w[0], w[stride], w[2 stride].  The sums are
-// those of a child-by-child scatter into zeroed storage, in the same order.
-__device__ __forceinline__ void ps_gather(const PSolveDev& ps, const int* __restrict__ pp, int t,
-                                          const d4* __restrict__ bt, double* __restrict__ w, int stride) {
+__device__ __forceinline__ void ps_pull_end(const PSolveDev& ps, const PsPull& q, const d4* __restrict__ bt,
+                                            double* __restrict__ w, int stride) {
     double x = 0.0, y = 0.0, z = 0.0;
-    for (int e = pp[t]; e < pp[t + 1]; ++e) {
-        const d4 a = ld_cg(ps.acc + ps.pull_idx[e]);
-        x += a.x;
-        y += a.y;
-        z += a.z;
+    d4 b;
+    if (bt) b = ld(bt);
+    if (q.e0 < q.e1) {
+        const d4 a = ld_cg(ps.acc + q.i0);
+        const bool two = q.e0 + 1 < q.e1;
+        d4 c;
+        if (two) c = ld_cg(ps.acc + q.i1);
+        x += a.x; y += a.y; z += a.z;
+        if (two) { x += c.x; y += c.y; z += c.z; }
+        for (int e = q.e0 + 2; e < q.e1; ++e) {
+            const d4 d = ld_cg(ps.acc + ps.pull_idx[e]);
+            x += d.x; y += d.y; z += d.z;
+        }
     }
-    if (bt) {
-        const d4 a = ld(bt);
-        x += a.x;
-        y += a.y;
-        z += a.z;
-    }
+    if (bt) { x += b.x; y += b.y; z += b.z; }
     w[0] = x;
     w[stride] = y;
     w[2 * stride] = z;
 }
 
-// The static blocks a front's forward sweep reads, fetched into L2 ahead of use.
-__device__ __forceinline__ void ps_fwd_prefetch(const PSolveDev& ps, int s) {
-    const int ns = ps.p[s] / 3, fs = ps.f[s] / 3;
-    prefetch_l2(ps.xinv + ps.xoff[s], sizeof(double) * ns * ns);
-    prefetch_l2(ps.panel + ps.poff[s], sizeof(double) * fs * ns);
-}
-__device__ __forceinline__ void ps_bwd_prefetch(const PSolveDev& ps, int s) {
-    const int ns = ps.p[s] / 3, nu = ps.f[s] / 3 - ns;
-    prefetch_l2(ps.pant + ps.toff[s], sizeof(double) * ns * nu);
-    prefetch_l2(ps.xinvt + ps.xoff[s], sizeof(double) * ns * ns);
-}
-
-__device__ __forceinline__ void ps_fwd_cta(const PSolveDev& ps, int s, const d4* __restrict__ b,
-                                           d4* __restrict__ y, double* __restrict__ smd) {
-    const int tid = threadIdx.x, nt = blockDim.x;
-    const int begin = ps.begin[s], ns = ps.p[s] / 3, fs = ps.f[s] / 3, nu = fs - ns;
-    double* w = smd;                   // [3][fs]
-    double* yv = w + 3 * fs;           // [3][ns]
-    double* red = yv + 3 * ns;         // [3][GV_MAXG * GV_ROWS]
-    const int* pp = ps.pull_ptr + ps.pull_off[s];
-    for (int t = tid; t < fs; t += nt) ps_gather(ps, pp, t, t < ns ? b + begin + t : nullptr, w + t, fs);
+// Column-major product on one CTA with three right-hand sides: t_c,i = sum_k
+// A[k * lda + i] v[c * ldv + k] for rows r_lo <= i < r_hi and k < K (TRI 1: only
+// k <= i; TRI 2: only k >= i).  wait() blocks until the vectors are there and returns
+// false to give up; fill() then brings them to v.  Work items are (row, chunk) pairs,
+// the row fastest (coalesced loads), all three columns to a lane.  SPLIT: a lane for
+// each column too, for tasks too small to fill a CTA (a chunk is a serial chain of
+// FP64 FMAs, at least 64 cycles each, so a third of the chain per lane), and each
+// thread loads up to PS_CH entries of its first item before the wait.
+// fin(i, t0, t1, t2) stores.
+template <int TRI, bool SPLIT, class Wait, class Fill, class Fin>
+__device__ __forceinline__ bool ps_rows(const double* __restrict__ A, long lda, int r_lo, int r_hi, int K,
+                                        const double* __restrict__ v, int ldv, double* __restrict__ red, Wait wait,
+                                        Fill fill, Fin fin) {
+    const int nt = blockDim.x, tid = threadIdx.x;
+    const int G = gv_groups(K), C = (K + G - 1) / G;
+    constexpr int RS = GV_ROWS * GV_MAXG;      // stride between the three columns' partial sums
+    auto range = [&](int i, int g, int& k0, int& k1) {
+        k0 = g * C;
+        k1 = min(K, k0 + C);
+        if (TRI == 1) k1 = min(k1, i + 1);
+        if (TRI == 2) k0 = max(k0, i);
+    };
+    // item -> (column, chunk, row)
+    auto decode = [&](int item, int R, int& c, int& g, int& r) {
+        const int q = item / R;
+        r = item - q * R;
+        g = SPLIT ? q % G : q;
+        c = SPLIT ? q / G : 0;
+    };
+    double a[SPLIT ? PS_CH : 1];
+    if (SPLIT) {
+        const int R = min(GV_ROWS, r_hi - r_lo);
+        if (tid < 3 * R * G) {
+            int c, g, r, k0, k1;
+            decode(tid, R, c, g, r);
+            range(r_lo + r, g, k0, k1);
+            const double* col = A + (long)k0 * lda + r_lo + r;
+            const int n = k1 - k0;
+#pragma unroll
+            for (int q = 0; q < PS_CH; ++q) {
+                a[SPLIT ? q : 0] = q < n ? *col : 0.0;
+                col += lda;
+            }
+        }
+    }
+    if (!wait()) return false;
+    fill();
     __syncthreads();
-    const double* X = ps.xinv + ps.xoff[s];
-    const double* Pn = ps.panel + ps.poff[s];
-    cm_gemv3(X, ns, ns, ns, 1, w, fs, red, [&](int i, double t0, double t1, double t2) {
-        yv[i] = t0;
-        yv[ns + i] = t1;
-        yv[2 * ns + i] = t2;
-    });
-    d4* acc = ps.acc + ps.aoff[s];
-    cm_gemv3(Pn + ns, fs, nu, ns, 0, yv, ns, red, [&](int i, double t0, double t1, double t2) {
-        st(acc + i, w[ns + i] - t0, w[fs + ns + i] - t1, w[2 * fs + ns + i] - t2);
-    });
-    for (int t = tid; t < ns; t += nt) st(y + begin + t, yv[t], yv[ns + t], yv[2 * ns + t]);
+    for (int i0 = r_lo; i0 < r_hi; i0 += GV_ROWS) {
+        const int R = min(GV_ROWS, r_hi - i0);
+        for (int item = tid; item < (SPLIT ? 3 : 1) * R * G; item += nt) {
+            int c, g, r, k0, k1;
+            decode(item, R, c, g, r);
+            range(i0 + r, g, k0, k1);
+            const double* col = A + (long)k0 * lda + i0 + r;
+            if (SPLIT) {
+                const double* vc = v + c * ldv + k0;
+                const int n = k1 - k0;
+                double s = 0.0;
+                int q0 = 0;
+                if (i0 == r_lo && item == tid) {
+#pragma unroll
+                    for (int q = 0; q < PS_CH; ++q) {
+                        if (q >= n) break;
+                        s += a[SPLIT ? q : 0] * vc[q];
+                    }
+                    q0 = PS_CH;
+                    col += (long)PS_CH * lda;
+                }
+#pragma unroll 8
+                for (int q = q0; q < n; ++q) {
+                    s += *col * vc[q];
+                    col += lda;
+                }
+                red[c * RS + g * GV_ROWS + r] = s;
+            } else {
+                double a0 = 0.0, a1 = 0.0, a2 = 0.0;
+#pragma unroll 4
+                for (int k = k0; k < k1; ++k) {
+                    const double x = *col;
+                    col += lda;
+                    a0 += x * v[k];
+                    a1 += x * v[ldv + k];
+                    a2 += x * v[2 * ldv + k];
+                }
+                red[g * GV_ROWS + r] = a0;
+                red[RS + g * GV_ROWS + r] = a1;
+                red[2 * RS + g * GV_ROWS + r] = a2;
+            }
+        }
+        __syncthreads();
+        for (int e = tid; e < 3 * R; e += nt) {
+            const int c = e / R, r = e - c * R, i = i0 + r;
+            // the row's chunks with entries: [gl, gh)
+            const int gl = TRI == 2 ? i / C : 0, gh = TRI == 1 ? i / C + 1 : G;
+            double t = 0.0;
+            for (int g = gl; g < gh; ++g) t += red[c * RS + g * GV_ROWS + r];
+            red[c * RS + r] = t;
+        }
+        __syncthreads();
+        for (int r = tid; r < R; r += nt) fin(i0 + r, red[r], red[RS + r], red[2 * RS + r]);
+        __syncthreads();
+    }
+    return true;
 }
 
-// Warp path, forward: w is this warp's [3][PS_LD] gathered right-hand side, then
-// [3][PS_LD] of y_s.  Both products give one lane to each (row, column) pair, so
-// that a front of ns or nu rows keeps 3 ns or 3 nu lanes busy instead of ns or
-// nu (the fronts here have 4-24 pivot rows); a pair's sum runs over k in
-// ascending order, as with one lane per row.
-__device__ __forceinline__ void ps_fwd_warp(const PSolveDev& ps, int s, const d4* __restrict__ b,
-                                            d4* __restrict__ y, double* __restrict__ w) {
+// Half A forward, rows [r_lo, r_hi).  With PRE the lookups of up to PS_PULL positions a
+// thread come before the wait.
+constexpr int PS_PULL = 2;
+template <bool PRE, class Wait>
+__device__ __forceinline__ bool ps_fwd_a(const PSolveDev& ps, int s, int r_lo, int r_hi, const d4* __restrict__ b,
+                                         d4* __restrict__ y, double* __restrict__ smd, Wait wait) {
+    const int tid = threadIdx.x, nt = blockDim.x;
+    const int begin = ps.begin[s], ns = ps.p[s] / 3;
+    double* w = smd;                       // [3][ns], positions below r_hi
+    double* red = w + 3 * ns;              // [3][GV_MAXG * GV_ROWS]
+    const int* pp = ps.pull_ptr + ps.pull_off[s];
+    constexpr int NP = PRE ? PS_PULL : 0;
+    PsPull pull[PS_PULL];
+#pragma unroll
+    for (int q = 0; q < NP; ++q)
+        if (tid + q * nt < r_hi) pull[q] = ps_pull_begin(ps, pp, tid + q * nt);
+    return ps_rows<1, PRE>(
+        ps.xinv + ps.xoff[s], ns, r_lo, r_hi, ns, w, ns, red, wait,
+        [&]() {
+#pragma unroll
+            for (int q = 0; q < NP; ++q) {
+                const int t = tid + q * nt;
+                if (t < r_hi) ps_pull_end(ps, pull[q], b + begin + t, w + t, ns);
+            }
+            for (int t = tid + NP * nt; t < r_hi; t += nt)
+                ps_pull_end(ps, ps_pull_begin(ps, pp, t), b + begin + t, w + t, ns);
+        },
+        [&](int i, double t0, double t1, double t2) { st(y + begin + i, t0, t1, t2); });
+}
+
+// Half B forward, rows [r_lo, r_hi) of the update vector.  y_s is read through L2 (other
+// CTAs of the launch may have written it).
+template <bool PRE, class Wait>
+__device__ __forceinline__ bool ps_fwd_b(const PSolveDev& ps, int s, int r_lo, int r_hi, const d4* __restrict__ y,
+                                         double* __restrict__ smd, Wait wait) {
+    const int tid = threadIdx.x, nt = blockDim.x;
+    const int begin = ps.begin[s], ns = ps.p[s] / 3, fs = ps.f[s] / 3, nr = r_hi - r_lo;
+    double* yv = smd;                      // [3][ns]
+    double* w = yv + 3 * ns;               // [3][nr]
+    double* red = w + 3 * nr;              // [3][GV_MAXG * GV_ROWS]
+    const int* pp = ps.pull_ptr + ps.pull_off[s] + ns + r_lo;
+    constexpr int NP = PRE ? 1 : 0;
+    PsPull pull{0, 0, 0, 0};
+    if (NP && tid < nr) pull = ps_pull_begin(ps, pp, tid);
+    d4* acc = ps.acc + ps.aoff[s];
+    return ps_rows<0, PRE>(
+        ps.panel + ps.poff[s] + ns, fs, r_lo, r_hi, ns, yv, ns, red, wait,
+        [&]() {
+            for (int t = tid; t < ns; t += nt) {
+                const d4 a = ld_cg(y + begin + t);
+                yv[t] = a.x;
+                yv[ns + t] = a.y;
+                yv[2 * ns + t] = a.z;
+            }
+            if (NP && tid < nr) ps_pull_end(ps, pull, nullptr, w + tid, nr);
+            for (int t = tid + NP * nt; t < nr; t += nt) ps_pull_end(ps, ps_pull_begin(ps, pp, t), nullptr, w + t, nr);
+        },
+        [&](int i, double t0, double t1, double t2) {
+            const double* q = w + i - r_lo;
+            st(acc + i, q[0] - t0, q[nr] - t1, q[2 * nr] - t2);
+        });
+}
+
+// Half A backward, rows [r_lo, r_hi) into ps.wbuf.
+template <bool PRE, class Wait>
+__device__ __forceinline__ bool ps_bwd_a(const PSolveDev& ps, int s, int r_lo, int r_hi, const d4* __restrict__ y,
+                                         double* __restrict__ smd, Wait wait) {
+    const int tid = threadIdx.x, nt = blockDim.x;
+    const int begin = ps.begin[s], ns = ps.p[s] / 3, nu = ps.f[s] / 3 - ns, nr = r_hi - r_lo;
+    double* xu = smd;                      // [3][nu]
+    double* w = xu + 3 * nu;               // [3][nr]
+    double* red = w + 3 * nr;              // [3][GV_MAXG * GV_ROWS]
+    const int* un = ps.unode + ps.uptr[s];
+    constexpr int NP = PRE ? PS_PULL : 0;
+    int src[PS_PULL];
+#pragma unroll
+    for (int q = 0; q < NP; ++q) src[q] = tid + q * nt < nu ? un[tid + q * nt] : 0;
+    auto put = [&](int k, int node) {
+        const d4 a = ld_cg(ps.xint + node);
+        xu[k] = a.x;
+        xu[nu + k] = a.y;
+        xu[2 * nu + k] = a.z;
+    };
+    return ps_rows<0, PRE>(
+        ps.pant + ps.toff[s], ns, r_lo, r_hi, nu, xu, nu, red, wait,
+        [&]() {
+            for (int t = tid; t < nr; t += nt) {
+                const d4 a = ld_cg(y + begin + r_lo + t);
+                w[t] = a.x;
+                w[nr + t] = a.y;
+                w[2 * nr + t] = a.z;
+            }
+#pragma unroll
+            for (int q = 0; q < NP; ++q)
+                if (tid + q * nt < nu) put(tid + q * nt, src[q]);
+            for (int k = tid + NP * nt; k < nu; k += nt) put(k, un[k]);
+        },
+        [&](int i, double t0, double t1, double t2) {
+            const double* q = w + i - r_lo;
+            st(ps.wbuf + begin + i, q[0] - t0, q[nr] - t1, q[2 * nr] - t2);
+        });
+}
+
+// Half B backward, rows [r_lo, r_hi), and the per-node output.  wsrc: where w_s is
+// (ps.wbuf, or y at a root, which has no half A).
+template <bool PRE, class Wait>
+__device__ __forceinline__ bool ps_bwd_b(const PSolveDev& ps, const DevParams& P, int s, int r_lo, int r_hi,
+                                         const d4* __restrict__ wsrc, d4* __restrict__ out, int mode,
+                                         const int* __restrict__ contact, const d4* __restrict__ nb,
+                                         const double* __restrict__ cc, d4* __restrict__ f, int* __restrict__ case_,
+                                         double* __restrict__ c_out, double* __restrict__ smd, Wait wait) {
+    const int tid = threadIdx.x, nt = blockDim.x;
+    const int begin = ps.begin[s], ns = ps.p[s] / 3;
+    double* w = smd;                       // [3][ns], positions from r_lo
+    double* red = w + 3 * ns;              // [3][GV_MAXG * GV_ROWS]
+    return ps_rows<2, PRE>(
+        ps.xinvt + ps.xoff[s], ns, r_lo, r_hi, ns, w, ns, red, wait,
+        [&]() {
+            for (int t = r_lo + tid; t < ns; t += nt) {
+                const d4 a = ld_cg(wsrc + begin + t);
+                w[t] = a.x;
+                w[ns + t] = a.y;
+                w[2 * ns + t] = a.z;
+            }
+        },
+        [&](int i, double t0, double t1, double t2) {
+            const int row = begin + i;
+            st(ps.xint + row, t0, t1, t2);
+            finish_row(P, row, t0, t1, t2, out, mode, contact, nb, cc, f, case_, c_out);
+        });
+}
+
+// A task of a large front: rows of one half, or all of it (PS_AB).
+template <bool PRE, class Wait>
+__device__ __forceinline__ bool ps_fwd_cta(const PSolveDev& ps, int s, int phase, int r_lo, int r_hi,
+                                           const d4* __restrict__ b, d4* __restrict__ y, double* __restrict__ smd,
+                                           Wait wait) {
+    const int ns = ps.p[s] / 3, nu = ps.f[s] / 3 - ns;
+    const bool whole = phase == PS_AB;
+    if (phase != PS_B && !ps_fwd_a<PRE>(ps, s, whole ? 0 : r_lo, whole ? ns : r_hi, b, y, smd, wait)) return false;
+    if (phase == PS_A) return true;
+    return ps_fwd_b<PRE>(ps, s, whole ? 0 : r_lo, whole ? nu : r_hi, y, smd, [&]() { return whole || wait(); });
+}
+template <bool PRE, class Wait>
+__device__ __forceinline__ bool ps_bwd_cta(const PSolveDev& ps, const DevParams& P, int s, int phase, int r_lo,
+                                           int r_hi, const d4* __restrict__ y, d4* __restrict__ out, int mode,
+                                           const int* __restrict__ contact, const d4* __restrict__ nb,
+                                           const double* __restrict__ cc, d4* __restrict__ f, int* __restrict__ case_,
+                                           double* __restrict__ c_out, double* __restrict__ smd, Wait wait) {
+    const int ns = ps.p[s] / 3, nu = ps.f[s] / 3 - ns;
+    const bool whole = phase == PS_AB, a = phase == PS_A || (whole && nu > 0);
+    if (a && !ps_bwd_a<PRE>(ps, s, whole ? 0 : r_lo, whole ? ns : r_hi, y, smd, wait)) return false;
+    if (phase == PS_A) return true;
+    return ps_bwd_b<PRE>(ps, P, s, whole ? 0 : r_lo, whole ? ns : r_hi, nu > 0 ? ps.wbuf : y, out, mode, contact, nb,
+                         cc, f, case_, c_out, smd, [&]() { return a || wait(); });
+}
+
+// Small fronts, on the nt lanes of a warp or of a CTA (sync: their barrier): one lane
+// per (row, column) pair, so that a front of ns or nu rows keeps 3 ns or 3 nu lanes
+// busy; a pair's sum runs over k in ascending order.  w: [6][PS_LD].
+template <class Sync>
+__device__ __forceinline__ void ps_fwd_small(const PSolveDev& ps, int s, const d4* __restrict__ b,
+                                             d4* __restrict__ y, double* __restrict__ w, int lane, int nt, Sync sync) {
     constexpr int L = PS_LD;
-    const int lane = threadIdx.x & 31;
     const int begin = ps.begin[s], ns = ps.p[s] / 3, fs = ps.f[s] / 3, nu = fs - ns;
     double* yv = w + 3 * L;
     const int* pp = ps.pull_ptr + ps.pull_off[s];
-    for (int t = lane; t < fs; t += 32) ps_gather(ps, pp, t, t < ns ? b + begin + t : nullptr, w + t, L);
-    __syncwarp();
+    for (int t = lane; t < fs; t += nt)
+        ps_pull_end(ps, ps_pull_begin(ps, pp, t), t < ns ? b + begin + t : nullptr, w + t, L);
+    sync();
     // y_s = L_ss^-1 w_s (lower triangle)
     const double* X = ps.xinv + ps.xoff[s];
-    for (int q = lane; q < 3 * ns; q += 32) {
+    for (int q = lane; q < 3 * ns; q += nt) {
         const int i = q / 3, col = q - 3 * i;
         const double* wc = w + col * L;
         double a = 0.0;
@@ -550,11 +728,11 @@ __device__ __forceinline__ void ps_fwd_warp(const PSolveDev& ps, int s, const d4
         for (int k = 0; k <= i; ++k) a += X[(long)k * ns + i] * wc[k];
         yv[col * L + i] = a;
     }
-    __syncwarp();
+    sync();
     // update vector: w_U - L_Us y_s
     const double* Pn = ps.panel + ps.poff[s] + ns;
     double* acc = reinterpret_cast<double*>(ps.acc + ps.aoff[s]);
-    for (int q = lane; q < 3 * nu; q += 32) {
+    for (int q = lane; q < 3 * nu; q += nt) {
         const int i = q / 3, col = q - 3 * i;
         const double* yc = yv + col * L;
         double a = 0.0;
@@ -562,93 +740,30 @@ __device__ __forceinline__ void ps_fwd_warp(const PSolveDev& ps, int s, const d4
         for (int k = 0; k < ns; ++k) a += Pn[(long)k * fs + i] * yc[k];
         acc[4 * i + col] = w[col * L + ns + i] - a;
     }
-    for (int t = lane; t < ns; t += 32) st(y + begin + t, yv[t], yv[L + t], yv[2 * L + t]);
+    for (int t = lane; t < ns; t += nt) st(y + begin + t, yv[t], yv[L + t], yv[2 * L + t]);
 }
 
-// Level kernel of L y = b: CTAs [0, n_big) take one large front each, the others
-// PS_WARPS small fronts each (one per warp).
-__global__ void __launch_bounds__(256) k_ps_fwd(PSolveDev ps, const int* __restrict__ big, int n_big,
-                                                const int* __restrict__ small, int n_small,
-                                                const d4* __restrict__ b, d4* __restrict__ y) {
-    extern __shared__ double smd[];
-    if ((int)blockIdx.x < n_big) {
-        ps_fwd_prefetch(ps, big[blockIdx.x]);
-        ps_fwd_cta(ps, big[blockIdx.x], b, y, smd);
-        return;
-    }
-    const int warp = threadIdx.x >> 5;
-    const int q = ((int)blockIdx.x - n_big) * PS_WARPS + warp;
-    if (q < n_small) ps_fwd_warp(ps, small[q], b, y, smd + warp * 6 * PS_LD);
-}
-
-template <bool YL2 = false>
-__device__ __forceinline__ void ps_bwd_cta(const PSolveDev& ps, const DevParams& P, int s, const d4* __restrict__ y,
-                                           d4* __restrict__ out, int mode, const int* __restrict__ contact,
-                                           const d4* __restrict__ nb, const double* __restrict__ cc,
-                                           d4* __restrict__ f, int* __restrict__ case_, double* __restrict__ c_out,
-                                           double* __restrict__ smd) {
-    const int tid = threadIdx.x, nt = blockDim.x;
-    const int begin = ps.begin[s], ns = ps.p[s] / 3, fs = ps.f[s] / 3, nu = fs - ns;
-    double* w = smd;                   // [3][ns]
-    double* xu = w + 3 * ns;           // [3][nu]
-    double* red = xu + 3 * nu;         // [3][GV_MAXG * GV_ROWS]
-    const int* un = ps.unode + ps.uptr[s];
-    for (int t = tid; t < ns; t += nt) {
-        const d4 a = YL2 ? ld_cg(y + begin + t) : ld(y + begin + t);   // y written in the same launch: L2 only
-        w[t] = a.x;
-        w[ns + t] = a.y;
-        w[2 * ns + t] = a.z;
-    }
-    for (int k = tid; k < nu; k += nt) {
-        const d4 a = ld_cg(ps.xint + un[k]);
-        xu[k] = a.x;
-        xu[nu + k] = a.y;
-        xu[2 * nu + k] = a.z;
-    }
-    __syncthreads();
-    // w -= L_Us^T x_U (the transposed update block is ns x nu column-major)
-    cm_gemv3(ps.pant + ps.toff[s], ns, ns, nu, 0, xu, nu, red, [&](int i, double t0, double t1, double t2) {
-        w[i] -= t0;
-        w[ns + i] -= t1;
-        w[2 * ns + i] -= t2;
-    });
-    // x = L_ss^-T w, then the per-node output
-    cm_gemv3(ps.xinvt + ps.xoff[s], ns, ns, ns, 2, w, ns, red, [&](int i, double t0, double t1, double t2) {
-        const int row = begin + i;
-        st(ps.xint + row, t0, t1, t2);
-        finish_row(P, row, t0, t1, t2, out, mode, contact, nb, cc, f, case_, c_out);
-    });
-}
-
-// Warp path, backward: w is this warp's [3][PS_LD] right-hand side, then
-// [3][PS_LD] of x_U, later of x_s.  One lane per (row, column) pair, as forward.
-template <bool YL2 = false>
-__device__ __forceinline__ void ps_bwd_warp(const PSolveDev& ps, const DevParams& P, int s, const d4* __restrict__ y,
-                                            d4* __restrict__ out, int mode, const int* __restrict__ contact,
-                                            const d4* __restrict__ nb, const double* __restrict__ cc,
-                                            d4* __restrict__ f, int* __restrict__ case_,
-                                            double* __restrict__ c_out, double* __restrict__ w) {
+template <class Sync>
+__device__ __forceinline__ void ps_bwd_small(const PSolveDev& ps, const DevParams& P, int s, const d4* __restrict__ y,
+                                             d4* __restrict__ out, int mode, const int* __restrict__ contact,
+                                             const d4* __restrict__ nb, const double* __restrict__ cc,
+                                             d4* __restrict__ f, int* __restrict__ case_, double* __restrict__ c_out,
+                                             double* __restrict__ w, int lane, int nt, Sync sync) {
     constexpr int L = PS_LD;
-    const int lane = threadIdx.x & 31;
     const int begin = ps.begin[s], ns = ps.p[s] / 3, fs = ps.f[s] / 3, nu = fs - ns;
-    double* xu = w + 3 * L;
+    double* xu = w + 3 * L;                // x_U, later x_s
     const int* un = ps.unode + ps.uptr[s];
-    for (int t = lane; t < ns; t += 32) {
-        const d4 a = YL2 ? ld_cg(y + begin + t) : ld(y + begin + t);
-        w[t] = a.x;
-        w[L + t] = a.y;
-        w[2 * L + t] = a.z;
+    for (int t = lane; t < fs; t += nt) {
+        const d4 a = ld_cg(t < ns ? y + begin + t : ps.xint + un[t - ns]);
+        double* p = t < ns ? w + t : xu + t - ns;
+        p[0] = a.x;
+        p[L] = a.y;
+        p[2 * L] = a.z;
     }
-    for (int k = lane; k < nu; k += 32) {
-        const d4 a = ld_cg(ps.xint + un[k]);
-        xu[k] = a.x;
-        xu[L + k] = a.y;
-        xu[2 * L + k] = a.z;
-    }
-    __syncwarp();
+    sync();
     // w_s -= L_Us^T x_U (the transposed update block is ns x nu column-major)
     const double* T = ps.pant + ps.toff[s];
-    for (int q = lane; q < 3 * ns; q += 32) {
+    for (int q = lane; q < 3 * ns; q += nt) {
         const int i = q / 3, col = q - 3 * i;
         const double* xc = xu + col * L;
         double a = 0.0;
@@ -656,10 +771,10 @@ __device__ __forceinline__ void ps_bwd_warp(const PSolveDev& ps, const DevParams
         for (int k = 0; k < nu; ++k) a += T[(long)k * ns + i] * xc[k];
         w[col * L + i] -= a;
     }
-    __syncwarp();
+    sync();
     // x_s = L_ss^-T w_s (upper triangle of the transposed inverse), into xu
     const double* XT = ps.xinvt + ps.xoff[s];
-    for (int q = lane; q < 3 * ns; q += 32) {
+    for (int q = lane; q < 3 * ns; q += nt) {
         const int i = q / 3, col = q - 3 * i;
         const double* wc = w + col * L;
         double a = 0.0;
@@ -667,8 +782,8 @@ __device__ __forceinline__ void ps_bwd_warp(const PSolveDev& ps, const DevParams
         for (int k = i; k < ns; ++k) a += XT[(long)k * ns + i] * wc[k];
         xu[col * L + i] = a;
     }
-    __syncwarp();
-    for (int t = lane; t < ns; t += 32) {
+    sync();
+    for (int t = lane; t < ns; t += nt) {
         const double a0 = xu[t], a1 = xu[L + t], a2 = xu[2 * L + t];
         const int row = begin + t;
         st(ps.xint + row, a0, a1, a2);
@@ -676,8 +791,23 @@ __device__ __forceinline__ void ps_bwd_warp(const PSolveDev& ps, const DevParams
     }
 }
 
-// Level kernel of L^T x = y (and the per-node output): large fronts per CTA, small
-// fronts per warp, as for the forward sweep.
+// Level kernels: CTAs [0, n_big) take one large front each, the others PS_WARPS small
+// fronts each (one per warp).
+__global__ void __launch_bounds__(256) k_ps_fwd(PSolveDev ps, const int* __restrict__ big, int n_big,
+                                                const int* __restrict__ small, int n_small,
+                                                const d4* __restrict__ b, d4* __restrict__ y) {
+    extern __shared__ double smd[];
+    if ((int)blockIdx.x < n_big) {
+        const int s = big[blockIdx.x];
+        ps_fwd_cta<false>(ps, s, PS_AB, 0, 0, b, y, smd, []() { return true; });
+        return;
+    }
+    const int warp = threadIdx.x >> 5;
+    const int q = ((int)blockIdx.x - n_big) * PS_WARPS + warp;
+    if (q < n_small)
+        ps_fwd_small(ps, small[q], b, y, smd + warp * 6 * PS_LD, threadIdx.x & 31, 32, []() { __syncwarp(); });
+}
+
 __global__ void __launch_bounds__(256) k_ps_bwd(PSolveDev ps, DevParams P, const int* __restrict__ big, int n_big,
                                                 const int* __restrict__ small, int n_small, const d4* __restrict__ y,
                                                 d4* __restrict__ out, int mode, const int* __restrict__ contact,
@@ -686,204 +816,156 @@ __global__ void __launch_bounds__(256) k_ps_bwd(PSolveDev ps, DevParams P, const
                                                 double* __restrict__ c_out) {
     extern __shared__ double smd[];
     if ((int)blockIdx.x < n_big) {
-        ps_bwd_prefetch(ps, big[blockIdx.x]);
-        ps_bwd_cta(ps, P, big[blockIdx.x], y, out, mode, contact, nb, cc, f, case_, c_out, smd);
+        const int s = big[blockIdx.x];
+        ps_bwd_cta<false>(ps, P, s, PS_AB, 0, 0, y, out, mode, contact, nb, cc, f, case_, c_out, smd,
+                   []() { return true; });
         return;
     }
     const int warp = threadIdx.x >> 5;
     const int q = ((int)blockIdx.x - n_big) * PS_WARPS + warp;
     if (q < n_small)
-        ps_bwd_warp(ps, P, small[q], y, out, mode, contact, nb, cc, f, case_, c_out, smd + warp * 6 * PS_LD);
+        ps_bwd_small(ps, P, small[q], y, out, mode, contact, nb, cc, f, case_, c_out, smd + warp * 6 * PS_LD,
+                     threadIdx.x & 31, 32, []() { __syncwarp(); });
 }
 
-// ---- tree-scheduled sweeps: one launch per sweep instead of one per level.
-// CTAs take work items from a ticket counter in a topological order (children
-// before parents for L y = b, the reverse for L^T x = y) and, before an item,
-// wait for the done flags of the fronts it reads: its children's update vectors
-// (forward) or its parent's solution (backward; the parent's own wait covers the
-// ancestors above it).  An item only waits on items with smaller tickets, which
-// CTAs already running hold, and the smallest unfinished ticket never waits, so
-// the launch makes progress whatever the number of CTAs resident.  A front's
-// arithmetic is that of the level kernels, so the results are the same bits.
-// Every wait is bounded (dc_wait.cuh): one that gives up sets the sticky fault
-// word, and every CTA stops taking items once the word is set.
+// ---- tree-scheduled sweeps: one launch for both sweeps of a global step (or one
+// for each).  CTAs take tasks from a ticket counter in a topological order: a
+// group of small fronts (a warp each), one front as a whole, or some rows of one
+// half of a large front.  Before a task a CTA waits until what it reads is complete:
+//   forward, whole or half A   every child's forward tasks
+//   backward, whole or half A  the parent's backward tasks (the parent's own wait
+//                              covers the ancestors above it)
+//   half B                     the front's own half-A tasks
+//   backward at a root         its own forward tasks
+// Each front counts its finished tasks in four counters (forward, forward half A,
+// backward, backward half A) whose targets are ps.need.  A task waits only on tasks
+// with smaller tickets, which CTAs already running hold, and the smallest unfinished
+// ticket never waits, so a launch makes progress whatever the number of resident CTAs.
+// A row's arithmetic is that of the level kernels, so the results are the same bits.
+// Every wait is bounded (dc_wait.cuh): one that gives up sets the sticky fault word,
+// and every CTA stops taking tasks once the word is set.
+//
+// Why large fronts are split by rows: an SM does one FP64 warp instruction in 19
+// cycles (measured; 64 for a warp alone), so the top fronts of one large cloth (400
+// pivots, an 80,000-entry triangle at 200 x 200 nodes) kept one CTA busy for tens of
+// microseconds each while the rest of the chip waited for them.
 
-// One thread takes the next ticket for the CTA; n_items once the fault word is set.
-__device__ __forceinline__ int ps_take(const PSolveDev& ps, int* ticket, int* s_item) {
-    if (threadIdx.x == 0) *s_item = dc_fault_set(ps.fault) ? ps.n_items : atomicAdd(ticket, 1);
-    __syncthreads();
-    return *s_item;
-}
-
-__global__ void __launch_bounds__(256) k_ps_fwd_tree(PSolveDev ps, const d4* __restrict__ b, d4* __restrict__ y) {
-    extern __shared__ double smd[];
-    __shared__ int s_item, s_ok;
-    int* ticket = ps.sched;
-    int* done = ps.sched + 1;
-    for (;;) {
-        const int it = ps_take(ps, ticket, &s_item);
-        if (it >= ps.n_items) return;
-        const int q0 = ps.tq_ptr[it], nq = ps.tq_ptr[it + 1] - q0;
-        const int s0 = ps.tq_sn[q0];
-        if (ps.f[s0] / 3 > PS_SMALL) {
-            ps_fwd_prefetch(ps, s0);
-            if (threadIdx.x == 0) {
-                bool ok = true;
-                for (int q = ps.cptr[s0]; ok && q < ps.cptr[s0 + 1]; ++q) ok = dc_wait_flag(done + ps.child[q], ps.fault);
-                s_ok = ok;
-            }
-            __syncthreads();
-            if (!s_ok) return;
-            ps_fwd_cta(ps, s0, b, y, smd);
-            __threadfence();
-            __syncthreads();
-            if (threadIdx.x == 0) dc_st_release(done + s0, 1);
-        } else {
-            const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-            if (warp < nq) {
-                const int s = ps.tq_sn[q0 + warp];
-                int ok = 1;
-                if (lane == 0)
-                    for (int q = ps.cptr[s]; ok && q < ps.cptr[s + 1]; ++q) ok = dc_wait_flag(done + ps.child[q], ps.fault);
-                ok = __shfl_sync(0xffffffffu, ok, 0);
-                if (ok) {
-                    ps_fwd_warp(ps, s, b, y, smd + warp * 6 * PS_LD);
-                    __threadfence();
-                    __syncwarp();
-                    if (lane == 0) dc_st_release(done + s, 1);
-                }
-            }
-            __syncthreads();   // every warp has read s_item before it is rewritten
+// The task's dependencies (one thread); false when a wait gave up.
+__device__ __forceinline__ bool ps_wait(const PSolveDev& ps, bool fwd, bool fused, int s, int phase) {
+    int* f = ps.sched + 1;                         // forward, forward half A
+    int* b = ps.sched + 2 * ps.S + 2;              // backward, backward half A
+    if (fwd) {
+        if (phase == PS_B) return dc_wait_count(f + ps.S + s, ps.need[s].y, ps.fault);
+        bool ok = true;
+        for (int q = ps.cptr[s]; ok && q < ps.cptr[s + 1]; ++q) {
+            const int c = ps.child[q];
+            ok = dc_wait_count(f + c, ps.need[c].x, ps.fault);
         }
+        return ok;
     }
+    const int par = ps.parent[s];
+    if (par < 0) return !fused || dc_wait_count(f + s, ps.need[s].x, ps.fault);
+    if (phase == PS_B) return dc_wait_count(b + ps.S + s, ps.need[s].w, ps.fault);
+    return dc_wait_count(b + par, ps.need[par].z, ps.fault);
+}
+// The counter a finished task adds to.
+__device__ __forceinline__ int* ps_counter(const PSolveDev& ps, bool fwd, int s, int phase) {
+    int* base = fwd ? ps.sched + 1 : ps.sched + 2 * ps.S + 2;
+    const bool mid = phase == PS_A && ps.parent[s] >= 0;   // (a root's forward ends with half A)
+    return base + (mid ? ps.S : 0) + s;
 }
 
-__global__ void __launch_bounds__(256) k_ps_bwd_tree(PSolveDev ps, DevParams P, const d4* __restrict__ y,
-                                                     d4* __restrict__ out, int mode, const int* __restrict__ contact,
-                                                     const d4* __restrict__ nb, const double* __restrict__ cc,
-                                                     d4* __restrict__ f, int* __restrict__ case_,
-                                                     double* __restrict__ c_out) {
-    extern __shared__ double smd[];
+// FWD / BWD: which sweeps this launch runs (both: the backward tasks follow the
+// forward ones in ticket order).  ALONE: no groups of small fronts (ps.alone); such a
+// context has fewer tasks than the chip has room for, its time is the chain of waits,
+// and the kernel loads what it can before them.  The other kernel keeps four CTAs on
+// an SM instead, whose work hides one another's waits.
+template <bool FWD, bool BWD, bool ALONE>
+__device__ __forceinline__ void ps_run(const PSolveDev& ps, const DevParams& P, const d4* __restrict__ b,
+                                       d4* __restrict__ y, d4* __restrict__ out, int mode,
+                                       const int* __restrict__ contact, const d4* __restrict__ nb,
+                                       const double* __restrict__ cc, d4* __restrict__ f, int* __restrict__ case_,
+                                       double* __restrict__ c_out, double* __restrict__ smd) {
     __shared__ int s_item, s_ok;
-    int* ticket = ps.sched + ps.S + 1;
-    int* done = ps.sched + ps.S + 2;
+    int* ticket = FWD ? ps.sched : ps.sched + 2 * ps.S + 1;
+    const int nf = FWD ? ps.n_ftask : 0, n = nf + (BWD ? ps.n_btask : 0);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     for (;;) {
-        const int t = ps_take(ps, ticket, &s_item);
-        if (t >= ps.n_items) return;
-        const int it = ps.n_items - 1 - t;   // the forward order reversed: parents first
-        const int q0 = ps.tq_ptr[it], nq = ps.tq_ptr[it + 1] - q0;
-        const int s0 = ps.tq_sn[q0];
-        if (ps.f[s0] / 3 > PS_SMALL) {
-            ps_bwd_prefetch(ps, s0);
-            if (threadIdx.x == 0) {
-                const int par = ps.parent[s0];
-                s_ok = par < 0 || dc_wait_flag(done + par, ps.fault);
-            }
-            __syncthreads();
-            if (!s_ok) return;
-            ps_bwd_cta(ps, P, s0, y, out, mode, contact, nb, cc, f, case_, c_out, smd);
-            __threadfence();
-            __syncthreads();
-            if (threadIdx.x == 0) dc_st_release(done + s0, 1);
-        } else {
-            const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-            if (warp < nq) {
-                const int s = ps.tq_sn[q0 + warp];
-                int ok = 1;
-                if (lane == 0) {
-                    const int par = ps.parent[s];
-                    ok = par < 0 || dc_wait_flag(done + par, ps.fault);
-                }
-                ok = __shfl_sync(0xffffffffu, ok, 0);
-                if (ok) {
-                    ps_bwd_warp(ps, P, s, y, out, mode, contact, nb, cc, f, case_, c_out,
-                                smd + warp * 6 * PS_LD);
-                    __threadfence();
-                    __syncwarp();
-                    if (lane == 0) dc_st_release(done + s, 1);
-                }
-            }
-            __syncthreads();
-        }
-    }
-}
-
-// Both sweeps of one global step as one launch: tickets [0, n) are the forward
-// items, [n, 2n) the backward items (the forward order reversed).  A backward
-// item waits for its parent's backward flag, or, at a root, for the root's
-// forward flag; every wait is again on a smaller ticket, so the launch makes
-// progress whatever the number of resident CTAs.  The backward work of small
-// trees runs while the forward sweeps of large ones are still in their upper
-// levels.  Same arithmetic as the two launches, so the same bits.
-__global__ void __launch_bounds__(256) k_ps_sweeps_tree(PSolveDev ps, DevParams P, const d4* __restrict__ b,
-                                                        d4* __restrict__ y, d4* __restrict__ out, int mode,
-                                                        const int* __restrict__ contact,
-                                                        const d4* __restrict__ nb, const double* __restrict__ cc,
-                                                        d4* __restrict__ f, int* __restrict__ case_,
-                                                        double* __restrict__ c_out) {
-    extern __shared__ double smd[];
-    __shared__ int s_item, s_ok;
-    int* ticket = ps.sched;
-    int* done_f = ps.sched + 1;
-    int* done_b = ps.sched + ps.S + 2;
-    const int n = ps.n_items;
-    for (;;) {
-        if (threadIdx.x == 0) s_item = dc_fault_set(ps.fault) ? 2 * n : atomicAdd(ticket, 1);
+        if (tid == 0) s_item = dc_fault_set(ps.fault) ? n : atomicAdd(ticket, 1);
         __syncthreads();
         const int t = s_item;
-        if (t >= 2 * n) return;
-        const bool fwd = t < n;
-        const int it = fwd ? t : n - 1 - (t - n);
-        const int q0 = ps.tq_ptr[it], nq = ps.tq_ptr[it + 1] - q0;
-        const int s0 = ps.tq_sn[q0];
-        if (ps.f[s0] / 3 > PS_SMALL) {
-            if (fwd) ps_fwd_prefetch(ps, s0);
-            else ps_bwd_prefetch(ps, s0);
-            if (threadIdx.x == 0) {
-                bool ok = true;
-                if (fwd) {
-                    for (int q = ps.cptr[s0]; ok && q < ps.cptr[s0 + 1]; ++q)
-                        ok = dc_wait_flag(done_f + ps.child[q], ps.fault);
-                } else {
-                    const int par = ps.parent[s0];
-                    ok = par < 0 ? dc_wait_flag(done_f + s0, ps.fault) : dc_wait_flag(done_b + par, ps.fault);
-                }
-                s_ok = ok;
+        if (t >= n) return;
+        const bool fwd = FWD && (!BWD || t < nf);
+        const int4 task = fwd ? ps.ftask[t] : ps.btask[t - nf];
+        if (ALONE || task.y != PS_GROUP) {
+            const int s = task.x;
+            auto wait = [&]() {
+                if (tid == 0) s_ok = ps_wait(ps, fwd, FWD, s, task.y);
+                __syncthreads();
+                return s_ok != 0;
+            };
+            if (ALONE && task.y == PS_FRONT) {
+                if (!wait()) return;
+                auto sync = []() { __syncthreads(); };
+                if (fwd) ps_fwd_small(ps, s, b, y, smd, tid, blockDim.x, sync);
+                else ps_bwd_small(ps, P, s, y, out, mode, contact, nb, cc, f, case_, c_out, smd, tid, blockDim.x, sync);
+            } else if (fwd) {
+                if (!ps_fwd_cta<ALONE>(ps, s, task.y, task.z, task.w, b, y, smd, wait)) return;
+            } else {
+                if (!ps_bwd_cta<ALONE>(ps, P, s, task.y, task.z, task.w, y, out, mode, contact, nb, cc, f, case_, c_out,
+                                       smd, wait))
+                    return;
             }
             __syncthreads();
-            if (!s_ok) return;
-            if (fwd) ps_fwd_cta(ps, s0, b, y, smd);
-            else ps_bwd_cta<true>(ps, P, s0, y, out, mode, contact, nb, cc, f, case_, c_out, smd);
-            __threadfence();
-            __syncthreads();
-            if (threadIdx.x == 0) dc_st_release((fwd ? done_f : done_b) + s0, 1);
+            if (tid == 0) dc_add_release(ps_counter(ps, fwd, s, task.y), 1);
         } else {
-            const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-            if (warp < nq) {
-                const int s = ps.tq_sn[q0 + warp];
+            if (warp < task.z) {
+                const int s = ps.tq_sn[task.x + warp];
                 int ok = 1;
-                if (lane == 0) {
-                    if (fwd) {
-                        for (int q = ps.cptr[s]; ok && q < ps.cptr[s + 1]; ++q)
-                            ok = dc_wait_flag(done_f + ps.child[q], ps.fault);
-                    } else {
-                        const int par = ps.parent[s];
-                        ok = par < 0 ? dc_wait_flag(done_f + s, ps.fault) : dc_wait_flag(done_b + par, ps.fault);
-                    }
-                }
+                if (lane == 0) ok = ps_wait(ps, fwd, FWD, s, PS_AB);
                 ok = __shfl_sync(0xffffffffu, ok, 0);
+                __syncwarp();              // lane 0's acquire orders every lane's reads
                 if (ok) {
-                    if (fwd) ps_fwd_warp(ps, s, b, y, smd + warp * 6 * PS_LD);
-                    else ps_bwd_warp<true>(ps, P, s, y, out, mode, contact, nb, cc, f, case_, c_out,
-                                           smd + warp * 6 * PS_LD);
-                    __threadfence();
+                    auto sync = []() { __syncwarp(); };
+                    double* w = smd + warp * 6 * PS_LD;
+                    if (fwd) ps_fwd_small(ps, s, b, y, w, lane, 32, sync);
+                    else ps_bwd_small(ps, P, s, y, out, mode, contact, nb, cc, f, case_, c_out, w, lane, 32, sync);
                     __syncwarp();
-                    if (lane == 0) dc_st_release((fwd ? done_f : done_b) + s, 1);
+                    if (lane == 0) dc_add_release(ps_counter(ps, fwd, s, PS_AB), 1);
                 }
             }
             __syncthreads();   // every warp has read s_item before it is rewritten
         }
     }
+}
+
+template <bool ALONE>
+__global__ void __launch_bounds__(256, ALONE ? 1 : 4) k_ps_fwd_tree(PSolveDev ps, const d4* __restrict__ b,
+                                                                    d4* __restrict__ y) {
+    extern __shared__ double smd[];
+    const DevParams none{};
+    ps_run<true, false, ALONE>(ps, none, b, y, nullptr, 0, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, smd);
+}
+
+template <bool ALONE>
+__global__ void __launch_bounds__(256, ALONE ? 1 : 4)
+    k_ps_bwd_tree(PSolveDev ps, DevParams P, d4* __restrict__ y, d4* __restrict__ out, int mode,
+                  const int* __restrict__ contact, const d4* __restrict__ nb, const double* __restrict__ cc,
+                  d4* __restrict__ f, int* __restrict__ case_, double* __restrict__ c_out) {
+    extern __shared__ double smd[];
+    ps_run<false, true, ALONE>(ps, P, nullptr, y, out, mode, contact, nb, cc, f, case_, c_out, smd);
+}
+
+// Both sweeps of one global step as one launch: the backward work of small trees
+// runs while the forward sweeps of large ones are still in their upper levels.
+template <bool ALONE>
+__global__ void __launch_bounds__(256, ALONE ? 1 : 4)
+    k_ps_sweeps_tree(PSolveDev ps, DevParams P, const d4* __restrict__ b, d4* __restrict__ y, d4* __restrict__ out,
+                     int mode, const int* __restrict__ contact, const d4* __restrict__ nb,
+                     const double* __restrict__ cc, d4* __restrict__ f, int* __restrict__ case_,
+                     double* __restrict__ c_out) {
+    extern __shared__ double smd[];
+    ps_run<true, true, ALONE>(ps, P, b, y, out, mode, contact, nb, cc, f, case_, c_out, smd);
 }
 
 __global__ void k_finalize(int m, double h, const d4* __restrict__ x_n, const d4* __restrict__ v,
@@ -993,40 +1075,44 @@ cudaError_t psolve_configure(int max_fs) {
     std::lock_guard<std::mutex> lock(mu);
     const size_t need = ps_level_smem(max_fs, 1);
     if (need <= configured) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(k_ps_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_ps_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_ps_fwd_tree, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_ps_bwd_tree, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_ps_sweeps_tree, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
+    cudaError_t e = cudaSuccess;
+    for (const void* k : {(const void*)k_ps_fwd, (const void*)k_ps_bwd, (const void*)k_ps_fwd_tree<false>,
+                          (const void*)k_ps_fwd_tree<true>, (const void*)k_ps_bwd_tree<false>,
+                          (const void*)k_ps_bwd_tree<true>, (const void*)k_ps_sweeps_tree<false>,
+                          (const void*)k_ps_sweeps_tree<true>})
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
     if (e == cudaSuccess) configured = need;
     return e;
 }
 
-cudaError_t psolve_tree_grid(int max_fs, int* grid_f, int* grid_b, size_t* smem_out) {
+cudaError_t psolve_tree_grid(int max_fs, bool alone, int* grid, size_t* smem_out) {
     const size_t smem = ps_level_smem(max_fs, 1);
     *smem_out = smem;
-    int dev = 0, sms = 0, nf = 0, nb = 0;
+    int dev = 0, sms = 0, n = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nf, k_ps_fwd_tree, 256, smem);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_ps_bwd_tree, 256, smem);
+    if (e == cudaSuccess)
+        e = alone ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_ps_sweeps_tree<true>, 256, smem)
+                  : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_ps_sweeps_tree<false>, 256, smem);
     if (e != cudaSuccess) return e;
-    *grid_f = sms * std::max(1, nf);
-    *grid_b = sms * std::max(1, nb);
+    *grid = sms * std::max(1, n);
     return cudaSuccess;
+}
+
+static void run_fwd_tree(const PSolveDev& ps, const d4* b, d4* y, cudaStream_t s) {
+    const int grid = std::min(ps.tree_grid, ps.n_ftask);
+    auto k = ps.alone ? k_ps_fwd_tree<true> : k_ps_fwd_tree<false>;
+    k<<<grid, 256, ps.tree_smem, s>>>(ps, b, y);
 }
 
 void launch_solve_fwd(const DevMesh& dm, const d4* b, d4* y, cudaStream_t s) {
     if (dm.solver == 1) {
         const PSolveDev& ps = dm.ps;
         if (ps.tree) {
-            if (ps.n_items == 0) return;
-            cudaMemsetAsync(ps.sched, 0, sizeof(int) * (ps.S + 1), s);
+            if (ps.n_ftask == 0) return;
+            cudaMemsetAsync(ps.sched, 0, sizeof(int) * (2 * (size_t)ps.S + 1), s);
             dc_note_launch();
-            k_ps_fwd_tree<<<std::min(ps.tree_grid_f, ps.n_items), 256, ps.tree_smem, s>>>(ps, b, y);
+            run_fwd_tree(ps, b, y, s);
             return;
         }
         for (int l = 0; l < ps.nlev; ++l) {
@@ -1045,22 +1131,23 @@ void launch_solve_fwd(const DevMesh& dm, const d4* b, d4* y, cudaStream_t s) {
 }
 void launch_solve_fwd_skip(const DevMesh& dm, const d4* b, d4* y, int skip, cudaStream_t s) {
     const PSolveDev& ps = dm.ps;
-    cudaMemsetAsync(ps.sched, 0, sizeof(int) * (ps.S + 1), s);
+    cudaMemsetAsync(ps.sched, 0, sizeof(int) * (2 * (size_t)ps.S + 1), s);
     const int ticket = skip;   // pageable source: copied before the call returns
     cudaMemcpyAsync(ps.sched, &ticket, sizeof(int), cudaMemcpyHostToDevice, s);
     dc_note_launch();
-    k_ps_fwd_tree<<<std::min(ps.tree_grid_f, ps.n_items), 256, ps.tree_smem, s>>>(ps, b, y);
+    run_fwd_tree(ps, b, y, s);
 }
 void launch_solve_bwd(const DevMesh& dm, const DevParams& P, const d4* y, d4* out, int mode, const int* contact,
                       const d4* nb, const double* c, d4* f, int* case_, double* c_out, cudaStream_t s) {
     if (dm.solver == 1) {
         const PSolveDev& ps = dm.ps;
         if (ps.tree) {
-            if (ps.n_items == 0) return;
-            cudaMemsetAsync(ps.sched + ps.S + 1, 0, sizeof(int) * (ps.S + 1), s);
+            if (ps.n_btask == 0) return;
+            cudaMemsetAsync(ps.sched + 2 * (size_t)ps.S + 1, 0, sizeof(int) * (2 * (size_t)ps.S + 1), s);
             dc_note_launch();
-            k_ps_bwd_tree<<<std::min(ps.tree_grid_b, ps.n_items), 256, ps.tree_smem, s>>>(
-                ps, P, y, out, mode, contact, nb, c, f, case_, c_out);
+            const int grid = std::min(ps.tree_grid, ps.n_btask);
+            auto k = ps.alone ? k_ps_bwd_tree<true> : k_ps_bwd_tree<false>;
+            k<<<grid, 256, ps.tree_smem, s>>>(ps, P, const_cast<d4*>(y), out, mode, contact, nb, c, f, case_, c_out);
             return;
         }
         for (int l = ps.nlev - 1; l >= 0; --l) {
@@ -1083,11 +1170,12 @@ bool launch_solve_sweeps(const DevMesh& dm, const DevParams& P, const d4* b, d4*
                          cudaStream_t s) {
     const PSolveDev& ps = dm.ps;
     if (dm.solver != 1 || !ps.tree || !ps.fused) return false;
-    if (ps.n_items == 0) return true;
-    cudaMemsetAsync(ps.sched, 0, sizeof(int) * 2 * (ps.S + 1), s);
+    if (ps.n_ftask == 0) return true;
+    cudaMemsetAsync(ps.sched, 0, sizeof(int) * 2 * (2 * (size_t)ps.S + 1), s);
     dc_note_launch();
-    k_ps_sweeps_tree<<<std::min(std::max(ps.tree_grid_f, ps.tree_grid_b), 2 * ps.n_items), 256, ps.tree_smem, s>>>(
-        ps, P, b, y, out, mode, contact, nb, c, f, case_, c_out);
+    const int grid = std::min(ps.tree_grid, ps.n_ftask + ps.n_btask);
+    auto k = ps.alone ? k_ps_sweeps_tree<true> : k_ps_sweeps_tree<false>;
+    k<<<grid, 256, ps.tree_smem, s>>>(ps, P, b, y, out, mode, contact, nb, c, f, case_, c_out);
     return true;
 }
 void launch_finalize(const DevMesh& dm, const DevParams& P, const d4* x_n, const d4* v, d4* x_np1,

@@ -577,16 +577,28 @@ dc_status upload_params(dc_ctx* c, ParamPrep& pp) {
         dc_build_tree_items(frm, tq_ptr, tq_sn);
         std::vector<int> pull_off, pull_ptr, pull_idx;
         dc_build_pull_lists(frm, pp.ps.aoff, 1, pull_off, pull_ptr, pull_idx);
-        int *d_tq_ptr, *d_tq_sn, *d_sched, *d_pull_off, *d_pull_ptr, *d_pull_idx;
-        if ((s = upload(c, F, &d_tq_ptr, tq_ptr)) || (s = upload(c, F, &d_tq_sn, tq_sn)) ||
-            (s = dalloc(c, F, &d_sched, 2 * ((size_t)frm.S + 1))) || (s = upload(c, F, &d_pull_off, pull_off)) ||
+        std::vector<int4> ftask, btask, need;
+        bool alone = false;
+        dc_build_ps_tasks(frm, tq_ptr, tq_sn, ftask, btask, need, alone);
+        int *d_tq_sn, *d_sched, *d_pull_off, *d_pull_ptr, *d_pull_idx;
+        int4 *d_ftask, *d_btask, *d_need;
+        d4* d_wbuf;
+        if ((s = upload(c, F, &d_ftask, ftask)) || (s = upload(c, F, &d_btask, btask)) ||
+            (s = upload(c, F, &d_need, need)) || (s = upload(c, F, &d_tq_sn, tq_sn)) ||
+            (s = dalloc(c, F, &d_wbuf, (size_t)std::max(MF, 1))) ||
+            (s = dalloc(c, F, &d_sched, 2 * (2 * (size_t)frm.S + 1))) || (s = upload(c, F, &d_pull_off, pull_off)) ||
             (s = upload(c, F, &d_pull_ptr, pull_ptr)) || (s = upload(c, F, &d_pull_idx, pull_idx)))
             return s;
         PSolveDev& ps = dm.ps;
         ps.S = frm.S;
-        ps.n_items = (int)tq_ptr.size() - 1;
+        ps.n_ftask = (int)ftask.size();
+        ps.n_btask = (int)btask.size();
+        ps.ftask = d_ftask;
+        ps.btask = d_btask;
+        ps.need = d_need;
+        ps.wbuf = d_wbuf;
+        ps.alone = alone ? 1 : 0;
         ps.parent = fd.parent;
-        ps.tq_ptr = d_tq_ptr;
         ps.tq_sn = d_tq_sn;
         ps.sched = d_sched;
         ps.pull_off = d_pull_off;
@@ -646,7 +658,7 @@ dc_status upload_params(dc_ctx* c, ParamPrep& pp) {
         int mx = 0;
         for (int v : c->ps_maxbig) mx = std::max(mx, v);
         CK(psolve_configure(mx));
-        CK(psolve_tree_grid(mx, &dm.ps.tree_grid_f, &dm.ps.tree_grid_b, &dm.ps.tree_smem));
+        CK(psolve_tree_grid(mx, dm.ps.alone != 0, &dm.ps.tree_grid, &dm.ps.tree_smem));
     }
     {
         // per level, where each instance's fronts start in lvl_sn (an instance's
@@ -737,8 +749,16 @@ size_t estimate_device_bytes(const dc_ctx* c, const MeshPrep& mp, const ParamPre
             add(8 * ff); add(8 * ((size_t)r.S + 1)); add(8 * r.pr_i.size());
         }
         add((size_t)pp.ps.acc_nodes * d4b); add(MF * d4b);
-        // tree schedule: items (at most one per front), two ticket/flag arrays
-        add(4 * ((size_t)r.S + 1)); add(4 * (size_t)r.S); add(8 * ((size_t)r.S + 1));
+        // tree schedule: tasks, targets, two ticket/counter arrays, the backward's w
+        {
+            std::vector<int> tq_ptr, tq_sn;
+            std::vector<int4> ftask, btask, need;
+            bool alone = false;
+            dc_build_tree_items(r, tq_ptr, tq_sn);
+            dc_build_ps_tasks(r, tq_ptr, tq_sn, ftask, btask, need, alone);
+            add(vbytes(ftask)); add(vbytes(btask)); add(vbytes(need));
+        }
+        add(4 * (size_t)r.S); add(8 * (2 * (size_t)r.S + 1)); add(MF * d4b);
         // pull lists of the child gather
         size_t nodes = 0;
         for (int q = 0; q < r.S; ++q) nodes += r.f[q] / 3 + 1;

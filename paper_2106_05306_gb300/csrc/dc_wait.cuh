@@ -17,16 +17,22 @@ static __device__ __forceinline__ void dc_st_release(int* p, int v) {
 static __device__ __forceinline__ bool dc_fault_set(const unsigned long long* fault) {
     return *reinterpret_cast<const volatile unsigned long long*>(fault) != 0ull;
 }
-// Waits until *flag is nonzero; false when the fault word is (or gets) set.
-static __device__ bool dc_wait_flag(const int* flag, unsigned long long* fault) {
+// Adds to a counter of finished tasks after the caller's writes and, behind a
+// barrier, its CTA's or warp's (release: cumulative over what the barrier ordered).
+static __device__ __forceinline__ void dc_add_release(int* p, int v) {
+    asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+// Waits until *count reaches target; false when the fault word is (or gets) set.
+static __device__ bool dc_wait_count(const int* count, int target, unsigned long long* fault) {
     for (int i = 0; i < DC_SPIN_LIMIT; ++i) {
-        if (dc_ld_acquire(flag)) {
-            __threadfence();
-            return true;
-        }
+        if (dc_ld_acquire(count) >= target) return true;
         if ((i & 31) == 31 && dc_fault_set(fault)) return false;
         __nanosleep(i < 64 ? 32 : 256);
     }
     atomicExch(fault, 1ull);
     return false;
+}
+// Waits until *flag is nonzero.
+static __device__ __forceinline__ bool dc_wait_flag(const int* flag, unsigned long long* fault) {
+    return dc_wait_count(flag, 1, fault);
 }
