@@ -462,7 +462,7 @@ def fma_peak(precision=64, n_iter=None):
 
 def front_factor(A, p, threads=512, use_tc=True, use_gscr=False):
     """One dense front through the adjoint preconditioner's factorisation (a test
-    hook; threads, use_tc and use_gscr are checked and change nothing): A is a symmetric (n, n) array, p the pivot count.  Returns (F, Linv):
+    hook; threads and use_gscr are checked and change nothing): A is a symmetric (n, n) array, p the pivot count.  Returns (F, Linv):
     F holds D and the unit-lower L in its first p columns and the Schur complement
     in its trailing lower triangle (float32, (n, n)); Linv is the inverse of L's
     pivot block ((p, p))."""

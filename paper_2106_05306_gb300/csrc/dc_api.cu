@@ -596,7 +596,7 @@ dc_status dc_debug_front_factor(int32_t n, int32_t p, const float* A, float* out
     else if (!use_gscr && one_cta_front_bytes(n, p, use_tc != 0) > 227 * 1024)
         err = "dc_debug_front_factor: front too large for shared memory; set use_gscr";
     else
-        st = ff_debug_factor(n, p, A, out, linv_out, &err);
+        st = ff_debug_factor(n, p, A, out, linv_out, use_tc, &err);
     if (st != DC_OK) g_create_err = err;
     return st;
 }

@@ -333,9 +333,10 @@ void launch_count_cases(const int* contact, const int* case_, int m_free,
 
 // Launches of one numeric factorisation of the fronts, in order (dc_front_factor.cu):
 // launch q works on the tiles FrontDev::tasks[begin .. begin + count).
-enum { FF_EXTEND = 0, FF_PANEL = 1, FF_UPDATE = 2, FF_FINISH = 3 };
+enum { FF_EXTEND = 0, FF_PANEL = 1, FF_UPDATE = 2, FF_UPDATE_TC = 3, FF_INVERSE = 4 };
 struct FrontLaunch {
-    int kind, k, level, begin, count;  // k: panel (FF_PANEL, FF_UPDATE)
+    int kind, k, level, begin, count;  // k: panel, or columns per task (FF_INVERSE)
+    int smem = 0;                      // dynamic shared memory (FF_INVERSE)
 };
 struct FrontPlan {
     std::vector<FrontLaunch> launches;
@@ -352,7 +353,7 @@ struct FrontDev {
     const int* p;
     const long long* off;
     const long long* acc_off;
-    const long long* binv_off;         // per front: offset of its factorised diagonal blocks
+    const long long* binv_off;         // per front: offset of its diagonal-block inverses
     const long long* linv_off;         // per front: offset of the inverse of its pivot block
     const int* uptr;
     const int* unode;
@@ -369,7 +370,7 @@ struct FrontDev {
     const double* pr_coef;
     float* pool;                       // fronts (lower triangles used)
     float* acc;                        // per-front update vectors of the forward solve
-    float* binv;                       // factorised 32x32 diagonal blocks (L below, D on the diagonal)
+    float* binv;                       // inverses of the 32x32 unit-lower diagonal blocks
     float* linv;                       // inverses of the unit-lower pivot blocks (p x p, column-major)
     float* rvec;                       // [3 m_free] right-hand side
     float* zvec;                       // [3 m_free] D^-1 L^-1 r

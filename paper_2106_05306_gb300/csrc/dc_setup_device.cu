@@ -429,6 +429,7 @@ dc_status upload_params(dc_ctx* c, ParamPrep& pp) {
         return DC_ERR_INVALID;
     }
     CK(frontal_configure(frm.max_f));
+    CK(ff_configure());
     free_pool(c, c->front_allocs);
     auto& F = c->front_allocs;
     FrontDev fd{};
