@@ -72,10 +72,12 @@ dc_status ff_debug_factor(int n, int p, const float* A, float* out, float* linv_
 size_t frontal_solve_smem(int max_f);
 // Raises the shared-memory limits of the solve kernels (fronts of up to max_f unknowns).
 cudaError_t frontal_configure(int max_f);
-// Launch shape of the tree-scheduled solves for fronts of at most max_f
-// unknowns: the CTAs of each kernel that fit on the device at once, and the
-// dynamic shared memory.
-cudaError_t frontal_tree_grid(int max_f, int* grid_f, int* grid_b, size_t* smem);
+// Launch shape of the tree-scheduled solve for fronts of at most max_f unknowns: the
+// CTAs that fit on the device at once, and the dynamic shared memory.
+cudaError_t frontal_tree_grid(int max_f, int* grid, size_t* smem);
+// Its tasks; order: the fronts in topological order, farthest from their root first.
+void ms_plan(const HostFronts& fr, const std::vector<int>& order, std::vector<int4>& ftask, std::vector<int4>& btask,
+             std::vector<int4>& need);
 // Assembles the constrained matrix into the fronts and factorises them.
 void frontal_factorize(const DevMesh& dm, const AdjDev& ad, const FrontDev& fd, const FrontPlan& plan, cudaStream_t s,
                        KTimer* kt = nullptr);
@@ -83,10 +85,11 @@ void frontal_factorize(const DevMesh& dm, const AdjDev& ad, const FrontDev& fd, 
 // lvl_sn[lvl_ptr[l] .. lvl_ptr[l+1]), the largest has lvl_maxf[l] unknowns.
 // act_sn / act_ptr (optional): device list of the fronts to solve, level l at
 // act_sn[act_ptr[l] .. act_ptr[l+1]) (act_ptr on the host); fronts of masked
-// instances may be listed (they exit at once), active ones must be.  With
-// fd.tree the two solves are one launch each over act_tq[0 .. n_act_tq) (the
-// same fronts in fd.tq's order), or over fd.tq when act_tq is null.
+// instances may be listed (they exit at once), active ones must be.  With fd.tree both
+// solves are one launch over the tasks fd.ftask[act_f[0 .. n_act_f)], then
+// fd.btask[act_b[0 .. n_act_b)] (the same fronts, in order), or over all tasks when
+// act_f is null.
 void frontal_precond(const AdjDev& ad, const FrontDev& fd, const int* lvl_ptr, int nlev, const int* lvl_maxf,
                      int n_free, const d4* w, d4* out, cudaStream_t s, KTimer* kt = nullptr,
-                     const int* act_sn = nullptr, const int* act_ptr = nullptr, const int* act_tq = nullptr,
-                     int n_act_tq = 0);
+                     const int* act_sn = nullptr, const int* act_ptr = nullptr, const int* act_f = nullptr,
+                     int n_act_f = 0, const int* act_b = nullptr, int n_act_b = 0);

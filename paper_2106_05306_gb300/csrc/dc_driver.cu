@@ -315,12 +315,13 @@ dc_status ensure_adjoint(dc_ctx* c) {
     RET(dalloc(c, P, &c->dparam_acc, 4 * (size_t)B));
     RET(dalloc(c, P, &c->dparam_part, (size_t)c->sg.npchunk));
     if (B > 1 && c->prm.adj_precond == 0) {
-        RET(dalloc(c, P, &c->d_act_sn, (size_t)std::max(c->fr.S, 1)));
+        const size_t n_act = std::max<size_t>(c->ms_finst_h.size() + c->ms_binst_h.size(), 1);   // (at least one per front)
+        RET(dalloc(c, P, &c->d_act_sn, n_act));
         RET(dalloc(c, P, &c->d_act_ch, (size_t)std::max(c->sg.nchunk, 1)));
         if (c->h_act_sn) cudaFreeHost(c->h_act_sn);
         if (c->h_act_ch) cudaFreeHost(c->h_act_ch);
         c->h_act_sn = c->h_act_ch = nullptr;
-        CK(cudaMallocHost(&c->h_act_sn, sizeof(int) * (size_t)std::max(c->fr.S, 1)));
+        CK(cudaMallocHost(&c->h_act_sn, sizeof(int) * n_act));
         CK(cudaMallocHost(&c->h_act_ch, sizeof(int) * (size_t)std::max(c->sg.nchunk, 1)));
     }
     const size_t need = 3 * (size_t)(mr + 1) * B + 4 * (size_t)B + 64;
@@ -347,7 +348,8 @@ void precond(dc_ctx* c, const AdjDev& ad, const d4* w, d4* out) {
     if (c->prm.adj_precond == 0) {
         frontal_precond(ad, c->fdv, c->fr.lvl_ptr.data(), c->nlev, c->lvl_maxf.data(), dm.m_free, w, out, s,
                         &c->kt, c->act_on ? c->d_act_sn : nullptr, c->act_ptr.data(),
-                        c->act_on ? c->d_act_sn : nullptr, c->n_act_tq);
+                        c->act_on ? c->d_act_sn : nullptr, c->n_act_f, c->act_on ? c->d_act_sn + c->n_act_f : nullptr,
+                        c->n_act_b);
         return;
     }
     // node-block inverse, projected P^-1, node-block inverse
@@ -373,9 +375,12 @@ dc_status build_active_lists(dc_ctx* c) {
     int pos = 0, cnt = 0;
     for (int i = 0; i < B; ++i) cnt += c->gs[i].act;
     if (c->fdv.tree) {
-        for (int s : c->tq_h)
-            if (c->gs[c->sn_inst_h[s]].act) c->h_act_sn[pos++] = s;
-        c->n_act_tq = pos;
+        for (size_t q = 0; q < c->ms_finst_h.size(); ++q)
+            if (c->gs[c->ms_finst_h[q]].act) c->h_act_sn[pos++] = (int)q;
+        c->n_act_f = pos;
+        for (size_t q = 0; q < c->ms_binst_h.size(); ++q)
+            if (c->gs[c->ms_binst_h[q]].act) c->h_act_sn[pos++] = (int)q;
+        c->n_act_b = pos - c->n_act_f;
     } else {
         for (int l = 0; l < nl; ++l) {
             c->act_ptr[l] = pos;

@@ -12,7 +12,10 @@
 // Fronts are dense column-major f x f blocks (DOF granularity, 3 per node) in
 // one pool; only their lower triangles are used.  Their numeric factorisation is
 // in dc_front_factor.cu; this file has the assembly and the solves.
+#include <algorithm>
 #include <mutex>
+#include <utility>
+#include <vector>
 
 #include "dc_adjoint.h"
 #include "dc_internal.h"
@@ -142,31 +145,32 @@ __device__ __forceinline__ void prefetch_l2(const void* p, size_t bytes) {
         asm volatile("prefetch.global.L2 [%0];" ::"l"(c + o));
 }
 
-// Column-major matrix-vector product on one CTA: t_i = sum_k A[k * lda + i] v_k for
-// rows i < nrows and k < K (k <= i when tri).  Rows go in passes of GV_ROWS; the
-// k range is cut into G contiguous chunks with G a function of K alone, every
-// (row, chunk) partial sum is one work item (consecutive items take consecutive
-// rows: coalesced), and a row's partial sums are added in chunk order.  The
-// arithmetic thus depends only on (nrows, K), never on the CTA size, so a front
-// gives the same bits whatever else shares its level.  fin(i, t_i) stores.
+// Column-major matrix-vector product on one CTA: t_i = sum_k A[k * lda + i] v_k for rows
+// r_lo <= i < r_hi and k < K (k <= i when TRI).  Rows go in passes of GV_ROWS; the k range
+// is cut into at most GV_MAXG contiguous chunks, their number a function of K alone, every
+// (row, chunk) partial sum is one work item (consecutive items take consecutive rows:
+// coalesced), and a row's partial sums are added in chunk order.  A row's arithmetic
+// thus depends only on (i, K), never on the CTA size or on the rows that share its CTA.
+// PAD: items of a pass are numbered for GV_ROWS rows (whole fronts), else for the rows
+// there are (short row blocks).  fin(i, t_i) stores.
 constexpr int GV_ROWS = 128;
 constexpr int GV_MAXG = 8;
 __host__ __device__ constexpr int gv_groups(int K) { return K <= 8 ? 1 : (K + 7) / 8 < GV_MAXG ? (K + 7) / 8 : GV_MAXG; }
 
-template <class Fin>
-__device__ __forceinline__ void cm_gemv(const float* __restrict__ A, long lda, int nrows, int K, bool tri,
+template <bool TRI, bool PAD, class Fin>
+__device__ __forceinline__ void cm_gemv(const float* __restrict__ A, long lda, int r_lo, int r_hi, int K,
                                         const float* __restrict__ v, float* __restrict__ red, Fin fin) {
     const int nt = blockDim.x, tid = threadIdx.x;
-    const int G = gv_groups(K);
-    const int C = (K + G - 1) / G;
-    for (int i0 = 0; i0 < nrows; i0 += GV_ROWS) {
-        for (int item = tid; item < GV_ROWS * G; item += nt) {
-            const int r = item % GV_ROWS, g = item / GV_ROWS, i = i0 + r;
+    const int G = gv_groups(K), C = (K + G - 1) / G;
+    for (int i0 = r_lo; i0 < r_hi; i0 += GV_ROWS) {
+        const int R = min(GV_ROWS, r_hi - i0), Rp = PAD ? GV_ROWS : R;
+        for (int item = tid; item < Rp * G; item += nt) {
+            const int g = item / Rp, r = item - g * Rp, i = i0 + r;
             float acc = 0.0f;
-            if (i < nrows) {
+            if (r < R) {
                 const int k0 = g * C;
                 int k1 = min(K, k0 + C);
-                if (tri) k1 = min(k1, i + 1);
+                if (TRI) k1 = min(k1, i + 1);
                 const float* a = A + i;
 #pragma unroll 4
                 for (int k = k0; k < k1; ++k) acc += a[(long)k * lda] * v[k];
@@ -174,7 +178,7 @@ __device__ __forceinline__ void cm_gemv(const float* __restrict__ A, long lda, i
             red[g * GV_ROWS + r] = acc;
         }
         __syncthreads();
-        if (tid < GV_ROWS && i0 + tid < nrows) {
+        if (tid < R) {
             float t = 0.0f;
             for (int q = 0; q < G; ++q) t += red[q * GV_ROWS + tid];
             fin(i0 + tid, t);
@@ -183,190 +187,261 @@ __device__ __forceinline__ void cm_gemv(const float* __restrict__ A, long lda, i
     }
 }
 
-// The blocks a front's solves read, fetched into L2 ahead of use.
-__device__ __forceinline__ void msolve_prefetch(const FrontDev& fd, int s) {
-    const int f = fd.f[s], p = fd.p[s];
-    prefetch_l2(fd.linv + fd.linv_off[s], sizeof(float) * p * p);
-    prefetch_l2(fd.pool + fd.off[s], sizeof(float) * (size_t)p * f);
+// Forward substitution L y = r for front s, then z = D^-1 y, in two halves: half A is
+// y_s = L_ss^-1 w_s with the stored explicit inverse (and z_s), half B the update vector
+// w_U - L_Us y_s that the parent adds in, each over rows [r_lo, r_hi).  w is the children's
+// update entries (pull lists: children in order), then r on the pivots -- the sums of a
+// child-by-child scatter into zeroed storage.  Vectors that other CTAs of a launch write
+// are read through L2.
+__device__ __forceinline__ float ms_pull(const FrontDev& fd, const int* __restrict__ pp, int t) {
+    const int node = t / 3, comp = t - 3 * node;
+    float a = 0.0f;
+    for (int e = pp[node]; e < pp[node + 1]; ++e) a += __ldcg(fd.acc + fd.pull_idx[e] + comp);
+    return a;
 }
-
-// Forward substitution L y = r for front s (one CTA), then z = D^-1 y.  y_s =
-// L_ss^-1 w_s with the stored explicit inverse; the rows below accumulate
-// -L_Us y_s into the front's update vector, which the parent adds in.  The
-// children's update vectors are read through L2 (other CTAs of a tree-scheduled
-// launch write them).
-__device__ __forceinline__ void msolve_fwd_front(const FrontDev& fd, int s, float* __restrict__ w) {
+template <class Wait>
+__device__ __forceinline__ bool ms_fwd_a(const FrontDev& fd, int s, int r_lo, int r_hi, float* __restrict__ w,
+                                         Wait wait) {
     const int tid = threadIdx.x, nt = blockDim.x;
+    const int f = fd.f[s], p = fd.p[s], base = 3 * fd.begin[s];
     const float* F = fd.pool + fd.off[s];
-    const float* X = fd.linv + fd.linv_off[s];
-    const int f = fd.f[s], p = fd.p[s];
-    const int base = 3 * fd.begin[s];
-    float* y = w + f;
-    float* red = y + f;                // [GV_MAXG][GV_ROWS] partial sums
-    // w = the children's update entries (pull lists: children in order), then r
-    // on the pivots -- the sums of a child-by-child scatter into zeroed storage
+    float* red = w + p;                // [GV_MAXG][GV_ROWS] partial sums
     const int* pp = fd.pull_ptr + fd.pull_off[s];
-    for (int t = tid; t < f; t += nt) {
-        const int node = t / 3, comp = t - 3 * node;
-        float a = 0.0f;
-        for (int e = pp[node]; e < pp[node + 1]; ++e) a += __ldcg(fd.acc + fd.pull_idx[e] + comp);
-        if (t < p) a += fd.rvec[base + t];
-        w[t] = a;
-    }
+    // the pivot of this thread's row of the first pass, ahead of the wait
+    const float d0 = r_lo + tid < r_hi ? F[(long)(r_lo + tid) * f + r_lo + tid] : 1.0f;
+    if (!wait()) return false;
+    for (int t = tid; t < r_hi; t += nt) w[t] = ms_pull(fd, pp, t) + fd.rvec[base + t];
     __syncthreads();
-    cm_gemv(X, p, p, p, true, w, red, [&](int i, float t) { y[i] = t; });
-    float* acc = fd.acc + fd.acc_off[s];
-    cm_gemv(F + p, f, f - p, p, false, y, red, [&](int i, float t) { acc[i] = w[p + i] - t; });
-    for (int t = tid; t < p; t += nt) fd.zvec[base + t] = y[t] / F[(long)t * f + t];
+    cm_gemv<true, false>(fd.linv + fd.linv_off[s], p, r_lo, r_hi, p, w, red, [&](int i, float t) {
+        fd.yvec[base + i] = t;
+        fd.zvec[base + i] = t / (i == r_lo + tid ? d0 : F[(long)i * f + i]);
+    });
+    return true;
 }
-
-// Forward substitution over one level (CTA per front of sn_list).
-__global__ void __launch_bounds__(FT) k_msolve_fwd(FrontDev fd, const int* __restrict__ sn_list,
-                                                    const double* __restrict__ mask) {
-    extern __shared__ float w[];
-    const int s = sn_list[blockIdx.x];
-    if (mask && mask[fd.sn_inst[s]] == 0.0) return;
-    msolve_prefetch(fd, s);
-    msolve_fwd_front(fd, s, w);
-}
-
-// Backward substitution L^T x = z for front s (one CTA), top-down: x_s =
-// L_ss^-T (z_s - L_Us^T x_U).  One warp per row (lanes along the row), two rows
-// per warp at a time; a row's sum does not depend on the CTA size.  x_U is read
-// through L2 (the ancestors' CTAs of a tree-scheduled launch write it).
-__device__ __forceinline__ void msolve_bwd_front(const FrontDev& fd, int s, float* __restrict__ sm) {
+template <class Wait>
+__device__ __forceinline__ bool ms_fwd_b(const FrontDev& fd, int s, int r_lo, int r_hi, float* __restrict__ y,
+                                         Wait wait) {
     const int tid = threadIdx.x, nt = blockDim.x;
-    const float* F = fd.pool + fd.off[s];
-    const float* X = fd.linv + fd.linv_off[s];
-    const int f = fd.f[s], p = fd.p[s], nu = f - p;
-    const int base = 3 * fd.begin[s];
-    float* w = sm;
-    float* xu = sm + p;
+    const int f = fd.f[s], p = fd.p[s], base = 3 * fd.begin[s], nr = r_hi - r_lo;
+    float* w = y + p;                  // [nr]
+    float* red = w + nr;               // [GV_MAXG][GV_ROWS]
+    const int* pp = fd.pull_ptr + fd.pull_off[s];
+    float* acc = fd.acc + fd.acc_off[s];
+    if (!wait()) return false;
+    for (int t = tid; t < p; t += nt) y[t] = __ldcg(fd.yvec + base + t);
+    for (int t = tid; t < nr; t += nt) w[t] = ms_pull(fd, pp, p + r_lo + t);
+    __syncthreads();
+    cm_gemv<false, false>(fd.pool + fd.off[s] + p, f, r_lo, r_hi, p, y, red,
+                          [&](int i, float t) { acc[i] = w[i - r_lo] - t; });
+    return true;
+}
+
+// Rows [r_lo, r_hi) of a row-major product, one warp per row (lanes along the row), two
+// rows per warp at a time: t_i = sum_{k_lo(i) <= k < K} A[i * lda + k] v_k.  A row's sum does
+// not depend on the CTA size.
+template <bool UPPER, class Fin>
+__device__ __forceinline__ void rm_gemv(const float* __restrict__ A, long lda, int r_lo, int r_hi, int K,
+                                        const float* __restrict__ v, Fin fin) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int i = r_lo + warp; i < r_hi; i += 2 * nw) {
+        const int i2 = i + nw;
+        const bool two = i2 < r_hi;
+        const float* r1 = A + (long)i * lda;
+        const float* r2 = A + (long)(two ? i2 : i) * lda;
+        float s1 = 0.0f, s2 = 0.0f;
+        if (UPPER) {
+#pragma unroll 4
+            for (int k = i + lane; k < K; k += 32) s1 += r1[k] * v[k];
+            if (two)
+#pragma unroll 4
+                for (int k = i2 + lane; k < K; k += 32) s2 += r2[k] * v[k];
+        } else if (two) {
+#pragma unroll 4
+            for (int k = lane; k < K; k += 32) {
+                const float x = v[k];
+                s1 += r1[k] * x;
+                s2 += r2[k] * x;
+            }
+        } else {
+#pragma unroll 4
+            for (int k = lane; k < K; k += 32) s1 += r1[k] * v[k];
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+            s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+        }
+        if (lane == 0) {
+            fin(i, s1);
+            if (two) fin(i2, s2);
+        }
+    }
+}
+
+// Backward substitution L^T x = z for front s: half A is w_s = z_s - L_Us^T x_U (kept in
+// yvec, which the forward sweep is done with), half B x_s = L_ss^-T w_s.
+template <class Wait>
+__device__ __forceinline__ bool ms_bwd_a(const FrontDev& fd, int s, int r_lo, int r_hi, float* __restrict__ xu,
+                                         Wait wait) {
+    const int tid = threadIdx.x, nt = blockDim.x;
+    const int f = fd.f[s], p = fd.p[s], nu = f - p, base = 3 * fd.begin[s];
+    const float* A = fd.pool + fd.off[s] + p;
     const int* un = fd.unode + fd.uptr[s];
-    for (int t = tid; t < p; t += nt) w[t] = fd.zvec[base + t];
+    for (int i = r_lo + (tid >> 5); i < r_hi; i += nt >> 5)
+        for (int k = 32 * (tid & 31); k < nu; k += 1024)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(A + (long)i * f + k));
+    if (!wait()) return false;
     for (int k = tid; k < nu; k += nt) xu[k] = __ldcg(fd.xvec + 3 * un[k / 3] + k % 3);
     __syncthreads();
-    const int lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
-    for (int t = warp; t < p; t += 2 * nw) {
-        const int t2 = t + nw;
-        const bool two = t2 < p;
-        const float* r1 = F + (long)t * f + p;
-        const float* r2 = F + (long)(two ? t2 : t) * f + p;
-        float s1 = 0.0f, s2 = 0.0f;
-        for (int k = lane; k < nu; k += 32) {
-            const float x = xu[k];
-            s1 += r1[k] * x;
-            s2 += r2[k] * x;
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-            s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-        }
-        if (lane == 0) {
-            w[t] -= s1;
-            if (two) w[t2] -= s2;
-        }
-    }
+    rm_gemv<false>(A, f, r_lo, r_hi, nu, xu,
+                   [&](int i, float t) { fd.yvec[base + i] = __ldcg(fd.zvec + base + i) - t; });
     __syncthreads();
-    for (int i = warp; i < p; i += 2 * nw) {
-        const int i2 = i + nw;
-        const bool two = i2 < p;
-        const float* c1 = X + (long)i * p;   // column i of L_ss^-1 = row i of L_ss^-T
-        const float* c2 = X + (long)(two ? i2 : i) * p;
-        float s1 = 0.0f, s2 = 0.0f;
-        for (int k = i + lane; k < p; k += 32) s1 += c1[k] * w[k];
-        if (two)
-            for (int k = i2 + lane; k < p; k += 32) s2 += c2[k] * w[k];
-        for (int o = 16; o > 0; o >>= 1) {
-            s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-            s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-        }
-        if (lane == 0) {
-            fd.xvec[base + i] = s1;
-            if (two) fd.xvec[base + i2] = s2;
-        }
-    }
+    return true;
+}
+template <class Wait>
+__device__ __forceinline__ bool ms_bwd_b(const FrontDev& fd, int s, int r_lo, int r_hi, float* __restrict__ w,
+                                         Wait wait) {
+    const int tid = threadIdx.x, nt = blockDim.x;
+    const int p = fd.p[s], base = 3 * fd.begin[s];
+    const float* X = fd.linv + fd.linv_off[s];   // column i of L_ss^-1 = row i of L_ss^-T
+    for (int i = r_lo + (tid >> 5); i < r_hi; i += nt >> 5)
+        for (int k = i + 32 * (tid & 31); k < p; k += 1024)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(X + (long)i * p + k));
+    if (!wait()) return false;
+    const float* src = fd.f[s] > p ? fd.yvec : fd.zvec;   // (a root has no half A)
+    for (int t = r_lo + tid; t < p; t += nt) w[t] = __ldcg(src + base + t);
+    __syncthreads();
+    rm_gemv<true>(X, p, r_lo, r_hi, p, w, [&](int i, float t) { fd.xvec[base + i] = t; });
+    __syncthreads();
+    return true;
 }
 
-// Backward substitution over one level (CTA per front of sn_list).
+// The whole of front s on one CTA: both halves with the vectors kept in shared memory (the
+// same sums in the same order).
+template <class Wait>
+__device__ __forceinline__ bool ms_fwd_whole(const FrontDev& fd, int s, float* __restrict__ w, Wait wait) {
+    const int tid = threadIdx.x, nt = blockDim.x;
+    const int f = fd.f[s], p = fd.p[s], base = 3 * fd.begin[s];
+    const float* F = fd.pool + fd.off[s];
+    float* y = w + f;
+    float* red = y + p;                // [GV_MAXG][GV_ROWS]
+    const int* pp = fd.pull_ptr + fd.pull_off[s];
+    if (!wait()) return false;
+    for (int t = tid; t < f; t += nt) w[t] = ms_pull(fd, pp, t) + (t < p ? fd.rvec[base + t] : 0.0f);
+    __syncthreads();
+    cm_gemv<true, true>(fd.linv + fd.linv_off[s], p, 0, p, p, w, red, [&](int i, float t) { y[i] = t; });
+    float* acc = fd.acc + fd.acc_off[s];
+    cm_gemv<false, true>(F + p, f, 0, f - p, p, y, red, [&](int i, float t) { acc[i] = w[p + i] - t; });
+    for (int t = tid; t < p; t += nt) fd.zvec[base + t] = y[t] / F[(long)t * f + t];
+    return true;
+}
+template <class Wait>
+__device__ __forceinline__ bool ms_bwd_whole(const FrontDev& fd, int s, float* __restrict__ w, Wait wait) {
+    const int tid = threadIdx.x, nt = blockDim.x;
+    const int f = fd.f[s], p = fd.p[s], nu = f - p, base = 3 * fd.begin[s];
+    const float* F = fd.pool + fd.off[s];
+    float* xu = w + p;
+    const int* un = fd.unode + fd.uptr[s];
+    if (!wait()) return false;
+    for (int t = tid; t < p; t += nt) w[t] = __ldcg(fd.zvec + base + t);
+    for (int k = tid; k < nu; k += nt) xu[k] = __ldcg(fd.xvec + 3 * un[k / 3] + k % 3);
+    __syncthreads();
+    if (nu > 0) {
+        rm_gemv<false>(F + p, f, 0, p, nu, xu, [&](int i, float t) { w[i] -= t; });
+        __syncthreads();
+    }
+    rm_gemv<true>(fd.linv + fd.linv_off[s], p, 0, p, p, w, [&](int i, float t) { fd.xvec[base + i] = t; });
+    __syncthreads();
+    return true;
+}
+
+// A task of front s: rows of one half, or all of it (MS_AB).
+template <bool fwd, class Wait>
+__device__ __forceinline__ bool ms_front(const FrontDev& fd, int s, int phase, int r_lo, int r_hi,
+                                         float* __restrict__ sm, Wait wait) {
+    if (phase == MS_AB) return fwd ? ms_fwd_whole(fd, s, sm, wait) : ms_bwd_whole(fd, s, sm, wait);
+    if (fwd)
+        return phase == MS_A ? ms_fwd_a(fd, s, r_lo, r_hi, sm, wait) : ms_fwd_b(fd, s, r_lo, r_hi, sm, wait);
+    return phase == MS_A ? ms_bwd_a(fd, s, r_lo, r_hi, sm, wait) : ms_bwd_b(fd, s, r_lo, r_hi, sm, wait);
+}
+
+// Substitution over one level (CTA per front of sn_list).
+__global__ void __launch_bounds__(FT) k_msolve_fwd(FrontDev fd, const int* __restrict__ sn_list,
+                                                    const double* __restrict__ mask) {
+    extern __shared__ float sm[];
+    const int s = sn_list[blockIdx.x];
+    if (mask && mask[fd.sn_inst[s]] == 0.0) return;
+    ms_front<true>(fd, s, MS_AB, 0, 0, sm, []() { return true; });
+}
 __global__ void __launch_bounds__(FT) k_msolve_bwd(FrontDev fd, const int* __restrict__ sn_list,
                                                     const double* __restrict__ mask) {
     extern __shared__ float sm[];
     const int s = sn_list[blockIdx.x];
     if (mask && mask[fd.sn_inst[s]] == 0.0) return;
-    msolve_prefetch(fd, s);
-    msolve_bwd_front(fd, s, sm);
+    ms_front<false>(fd, s, MS_AB, 0, 0, sm, []() { return true; });
 }
 
-// Tree-scheduled solves: one launch per sweep.  Persistent CTAs take the fronts
-// of items[0 .. n_items) (a topological order, children first) from a ticket
-// counter; the backward sweep takes them in reverse.  Before a front a CTA waits
-// (bounded, dc_wait.cuh) for its children's done flags (forward) or its
-// parent's (backward).  A front is only ever waited on by fronts of its own
-// instance, and an instance is masked whole, so a masked front is skipped
-// without a flag.  An item waits only on items with smaller tickets, held by
-// CTAs already running, so the launch completes whatever the number resident.
-// Threads per CTA of a tree-scheduled solve: the fronts on the dependency chain
-// are the large ones, so wide CTAs pay (measured on the 256-cloth batch: 128
-// threads 1.50 s, 256 threads 1.09 s, 512 threads 1.02 s of solves per bench step).
+// Tree-scheduled solves, one launch per sweep.  Persistent CTAs take tasks -- a front, or
+// some rows of one half of a large one -- from a ticket counter in a topological order
+// (forward: children first; backward: parents first), and before a task wait (bounded,
+// dc_wait.cuh) for what it reads: its front's children (forward), its parent (backward),
+// or its own half A (half B).  A front is only ever waited on by fronts of its own
+// instance, and an instance is masked whole, so a masked front is skipped without
+// counting.  A task waits only on tasks with smaller tickets, held by CTAs already
+// running, so a launch completes whatever the number resident.
+// Why large fronts are split: one CTA reads the factor at about 0.1 TB/s, so the chain of
+// the top fronts set the time while the chip waited (one 200 x 200 cloth: 2.35 ms for the
+// two sweeps over a 0.5 GB factor).
+// Threads per CTA and CTAs per SM: a front is a chain of latencies, so many CTAs share an SM
+// where there are many fronts (96 cloths, the gradient call: forward at 3 CTAs 53.3 ms,
+// at 4 51.2), and the fronts on the dependency chain are the large ones, so wide CTAs pay.
 constexpr int MT = 512;
 
-__device__ __forceinline__ int ms_take(const FrontDev& fd, int* ticket, int n_items, int* s_item) {
-    if (threadIdx.x == 0) *s_item = dc_fault_set(fd.fault) ? n_items : atomicAdd(ticket, 1);
-    __syncthreads();
-    const int t = *s_item;
-    __syncthreads();   // every thread has read the ticket before it is rewritten
-    return t;
-}
-
-__global__ void __launch_bounds__(MT) k_msolve_fwd_tree(FrontDev fd, const int* __restrict__ items, int n_items,
-                                                        const double* __restrict__ mask) {
-    extern __shared__ float w[];
-    __shared__ int s_item, s_ok;
-    int* ticket = fd.sched;
-    int* done = fd.sched + 1;
-    for (;;) {
-        const int t = ms_take(fd, ticket, n_items, &s_item);
-        if (t >= n_items) return;
-        const int s = items[t];
-        if (mask && mask[fd.sn_inst[s]] == 0.0) continue;
-        msolve_prefetch(fd, s);
-        if (threadIdx.x == 0) {
-            bool ok = true;
-            for (int q = fd.cptr[s]; ok && q < fd.cptr[s + 1]; ++q) ok = dc_wait_flag(done + fd.child[q], fd.fault);
-            s_ok = ok;
-        }
-        __syncthreads();
-        if (!s_ok) return;
-        msolve_fwd_front(fd, s, w);
-        __threadfence();
-        __syncthreads();
-        if (threadIdx.x == 0) dc_st_release(done + s, 1);
-    }
-}
-
-__global__ void __launch_bounds__(MT) k_msolve_bwd_tree(FrontDev fd, const int* __restrict__ items, int n_items,
-                                                        const double* __restrict__ mask) {
+template <bool FWD>
+__global__ void __launch_bounds__(MT, FWD ? 4 : 3) k_msolve_tree(FrontDev fd, const int* __restrict__ list, int n,
+                                                       const double* __restrict__ mask) {
     extern __shared__ float sm[];
     __shared__ int s_item, s_ok;
-    int* ticket = fd.sched + fd.S + 1;
-    int* done = fd.sched + fd.S + 2;
+    int* ticket = fd.sched + (FWD ? 0 : 2 * fd.S + 1);
+    int* done = ticket + 1;                        // ends, then half-A ends
     for (;;) {
-        const int t = ms_take(fd, ticket, n_items, &s_item);
-        if (t >= n_items) return;
-        const int s = items[n_items - 1 - t];
-        if (mask && mask[fd.sn_inst[s]] == 0.0) continue;
-        msolve_prefetch(fd, s);
-        if (threadIdx.x == 0) {
-            const int par = fd.parent[s];
-            s_ok = par < 0 || dc_wait_flag(done + par, fd.fault);
+        if (threadIdx.x == 0) s_item = dc_fault_set(fd.fault) ? n : atomicAdd(ticket, 1);
+        __syncthreads();
+        const int t = s_item;
+        if (t >= n) return;
+        const int4 task = (FWD ? fd.ftask : fd.btask)[list ? list[t] : t];
+        const int s = task.x, phase = task.y;
+        if (mask && mask[fd.sn_inst[s]] == 0.0) {
+            __syncthreads();                       // every thread has read the ticket
+            continue;
         }
+        if (phase == MS_AB) {
+            const int f = fd.f[s], p = fd.p[s];
+            prefetch_l2(fd.linv + fd.linv_off[s], sizeof(float) * p * p);
+            prefetch_l2(fd.pool + fd.off[s], sizeof(float) * (size_t)p * f);
+        }
+        auto wait = [&]() {
+            if (threadIdx.x == 0) {
+                bool ok = true;
+                if (phase == MS_B && fd.parent[s] >= 0) {
+                    ok = dc_wait_count(done + fd.S + s, FWD ? fd.need[s].y : fd.need[s].w, fd.fault);
+                } else if (FWD) {
+                    for (int q = fd.cptr[s]; ok && q < fd.cptr[s + 1]; ++q)
+                        ok = dc_wait_count(done + fd.child[q], fd.cneed[q], fd.fault);
+                } else {
+                    const int par = fd.parent[s];
+                    ok = par < 0 || dc_wait_count(done + par, fd.need[par].z, fd.fault);
+                }
+                s_ok = ok;
+            }
+            __syncthreads();
+            return s_ok != 0;
+        };
+        if (!ms_front<FWD>(fd, s, phase, task.z, task.w, sm, wait)) return;
         __syncthreads();
-        if (!s_ok) return;
-        msolve_bwd_front(fd, s, sm);
-        __threadfence();
-        __syncthreads();
-        if (threadIdx.x == 0) dc_st_release(done + s, 1);
+        if (threadIdx.x == 0) {
+            const bool mid = phase == MS_A && fd.parent[s] >= 0;   // (a root's forward ends with half A)
+            dc_add_release(done + (mid ? fd.S : 0) + s, 1);
+        }
     }
 }
 
@@ -423,8 +498,8 @@ cudaError_t frontal_configure(int max_f) {
     std::lock_guard<std::mutex> lock(mu);
     const size_t sb = frontal_solve_smem(max_f);
     if (sb > solve_bytes) {
-        for (const void* k : {(const void*)k_msolve_fwd, (const void*)k_msolve_bwd, (const void*)k_msolve_fwd_tree,
-                              (const void*)k_msolve_bwd_tree}) {
+        for (const void* k : {(const void*)k_msolve_fwd, (const void*)k_msolve_bwd, (const void*)k_msolve_tree<true>,
+                              (const void*)k_msolve_tree<false>}) {
             cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sb);
             if (e != cudaSuccess) return e;
         }
@@ -433,18 +508,74 @@ cudaError_t frontal_configure(int max_f) {
     return cudaSuccess;
 }
 
-cudaError_t frontal_tree_grid(int max_f, int* grid_f, int* grid_b, size_t* smem_out) {
+cudaError_t frontal_tree_grid(int max_f, int* grid, size_t* smem_out) {
     const size_t smem = frontal_solve_smem(max_f);
     *smem_out = smem;
-    int dev = 0, sms = 0, nf = 0, nb = 0;
+    int dev = 0, sms = 0, n = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nf, k_msolve_fwd_tree, MT, smem);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_msolve_bwd_tree, MT, smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_msolve_tree<true>, MT, smem);
     if (e != cudaSuccess) return e;
-    *grid_f = sms * (nf > 0 ? nf : 1);
-    *grid_b = sms * (nb > 0 ? nb : 1);
+    *grid = sms * (n > 0 ? n : 1);
     return cudaSuccess;
+}
+
+// Tasks of the tree-scheduled solve (FrontDev::ftask, btask, need): fronts farthest from
+// their root first (backward: nearest first), those of one depth together: half A and
+// whole fronts, then half B, so that a CTA waiting for a half A seldom holds up a task
+// that is ready.  A front whose two products have at most `target` entries is one task;
+// else each half is cut into row blocks of about that many, in multiples of eight rows (a
+// 32-byte sector of every column): 16 tasks per SM and sweep, within [4096, 65536]
+// entries (8192 entries, 32 KB, take an SM about 0.3 us, well below the cost of starting
+// a task).  No split changes a bit of the result.
+void ms_plan(const HostFronts& fr, const std::vector<int>& order, std::vector<int4>& ftask, std::vector<int4>& btask,
+             std::vector<int4>& need) {
+    long long total = 0;
+    for (int s = 0; s < fr.S; ++s) total += (long long)fr.p[s] * (fr.p[s] + 1) / 2 + (long long)fr.p[s] * (fr.f[s] - fr.p[s]);
+    const long long target = std::min<long long>(65536, std::max<long long>(4096, total / (152 * 16)));
+    need.assign(fr.S, make_int4(1, 0, 1, 0));
+    ftask.clear();
+    btask.clear();
+    auto blocks = [&](std::vector<int4>& out, int s, int phase, int rows, auto work) {
+        int n = 0;
+        for (int r = 0; r < rows; ++n) {
+            long long w = 0;
+            int e = r;
+            while (e < rows && (w < target || e % 8)) w += work(e++);
+            out.push_back(make_int4(s, phase, r, e));
+            r = e;
+        }
+        return n;
+    };
+    std::vector<int> depth(fr.S, 0);
+    for (int s = fr.S - 1; s >= 0; --s) depth[s] = fr.parent[s] >= 0 ? depth[fr.parent[s]] + 1 : 0;
+    std::vector<std::pair<int, int>> span;   // fronts of one depth
+    for (int q = 0; q < fr.S;) {
+        int e = q;
+        while (e < fr.S && depth[order[e]] == depth[order[q]]) ++e;
+        span.push_back({q, e});
+        q = e;
+    }
+    auto emit = [&](std::vector<int4>& out, const std::pair<int, int>& sp, bool fwd) {
+        for (int second = 0; second < 2; ++second)
+            for (int q = sp.first; q < sp.second; ++q) {
+                const int s = order[q];
+                const long long p = fr.p[s], nu = fr.f[s] - p;
+                if (p * (p + 1) / 2 + p * nu <= target) {
+                    if (!second) out.push_back(make_int4(s, MS_AB, 0, 0));
+                } else if (fwd && !second) {
+                    (nu > 0 ? need[s].y : need[s].x) = blocks(out, s, MS_A, (int)p, [&](int i) { return (long long)i + 1; });
+                } else if (fwd && nu > 0) {
+                    need[s].x = blocks(out, s, MS_B, (int)nu, [&](int) { return p; });
+                } else if (!fwd && !second && nu > 0) {
+                    need[s].w = blocks(out, s, MS_A, (int)p, [&](int) { return nu; });
+                } else if (!fwd && second) {
+                    need[s].z = blocks(out, s, MS_B, (int)p, [&](int i) { return p - i; });
+                }
+            }
+    };
+    for (const auto& sp : span) emit(ftask, sp, true);
+    for (size_t k = span.size(); k-- > 0;) emit(btask, span[k], false);
 }
 
 static int solve_threads(int mf) { return mf <= 64 ? 128 : (mf <= 128 ? 256 : (mf <= 256 ? 512 : FT)); }
@@ -461,19 +592,18 @@ void frontal_factorize(const DevMesh& dm, const AdjDev& ad, const FrontDev& fd, 
 
 void frontal_precond(const AdjDev& ad, const FrontDev& fd, const int* lvl_ptr, int nlev, const int* lvl_maxf,
                      int n_free, const d4* w, d4* out, cudaStream_t s, KTimer* kt, const int* act_sn,
-                     const int* act_ptr, const int* act_tq, int n_act_tq) {
+                     const int* act_ptr, const int* act_f, int n_act_f, const int* act_b, int n_act_b) {
     dc_note_launch();
     k_pre_in<<<nblk(n_free, 128), 128, 0, s>>>(n_free, ad.type, ad.nb, w, fd.rvec, ad.node_inst, ad.mask);
     if (fd.tree) {
-        const int* items = act_tq ? act_tq : fd.tq;
-        const int n = act_tq ? n_act_tq : fd.S;
-        if (n > 0) {
-            cudaMemsetAsync(fd.sched, 0, sizeof(int) * 2 * ((size_t)fd.S + 1), s);
+        const int nf = act_f ? n_act_f : fd.n_ftask, nb = act_f ? n_act_b : fd.n_btask;
+        if (nf > 0) {
+            cudaMemsetAsync(fd.sched, 0, sizeof(int) * (4 * (size_t)fd.S + 2), s);
             if (kt) kt->begin(DC_KT_MSOLVE);
             dc_note_launch();
-            k_msolve_fwd_tree<<<n < fd.tree_grid_f ? n : fd.tree_grid_f, MT, fd.tree_smem, s>>>(fd, items, n, ad.mask);
+            k_msolve_tree<true><<<std::min(nf, fd.tree_grid), MT, fd.tree_smem, s>>>(fd, act_f, nf, ad.mask);
             dc_note_launch();
-            k_msolve_bwd_tree<<<n < fd.tree_grid_b ? n : fd.tree_grid_b, MT, fd.tree_smem, s>>>(fd, items, n, ad.mask);
+            k_msolve_tree<false><<<std::min(nb, fd.tree_grid), MT, fd.tree_smem, s>>>(fd, act_b, nb, ad.mask);
             if (kt) kt->end(DC_KT_MSOLVE);
         }
         dc_note_launch();

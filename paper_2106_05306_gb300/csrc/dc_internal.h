@@ -342,6 +342,8 @@ struct FrontPlan {
     std::vector<FrontLaunch> launches;
 };
 
+enum { MS_A = 0, MS_B = 1, MS_AB = 2 };
+
 // Device view of the multifrontal structure and its per-step numeric storage.
 struct FrontDev {
     int S, NP, max_f;
@@ -375,9 +377,10 @@ struct FrontDev {
     float* rvec;                       // [3 m_free] right-hand side
     float* zvec;                       // [3 m_free] D^-1 L^-1 r
     float* xvec;                       // [3 m_free] solution
-    // tree-scheduled solves (one launch per sweep): the fronts in a topological
-    // order (children first), their parents, and the launches' ticket counters
-    // and done flags
+    float* yvec;                       // [3 m_free] L^-1 r, then the backward sweep's w
+    // tree-scheduled solves (one launch per sweep): tasks (x, y, z, w) in a
+    // topological order, front x as a whole (y = MS_AB) or rows [z, w) of its half A / B,
+    // and per front how many tasks end each phase (forward, its half A, backward, its half A)
     int tree;                          // 1: tree-scheduled solves, 0: one launch per level
     // gather of the children's update vectors into front s: node t < f/3 sums the
     // 3-float entries acc[pull_idx[e] ..] for e in [pull_ptr[pull_off[s] + t],
@@ -385,11 +388,15 @@ struct FrontDev {
     const int* pull_off;               // [S]
     const int* pull_ptr;
     const int* pull_idx;
-    const int* tq;                     // [S]
+    int n_ftask, n_btask;
+    const int4* ftask;
+    const int4* btask;
+    const int4* need;                  // [S]
+    const int* cneed;                  // the forward target of each entry of child
     const int* parent;                 // [S] -1 at a root
-    int* sched;                        // [2][S + 1]: ticket, then per-front done flags (fwd; bwd)
+    int* sched;                        // [2][2 S + 1]: ticket, tasks done per front, half-A tasks done (fwd; bwd)
     unsigned long long* fault;         // sticky: set when a dependency wait gave up
-    int tree_grid_f, tree_grid_b;      // host: CTAs of a tree-scheduled launch
+    int tree_grid;                     // host: CTAs of a tree-scheduled launch
     size_t tree_smem;                  // host: its dynamic shared memory
     const int2* tasks;                 // tile lists of the factorisation (FrontPlan)
 };

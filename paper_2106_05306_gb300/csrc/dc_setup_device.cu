@@ -503,22 +503,38 @@ dc_status upload_params(dc_ctx* c, ParamPrep& pp) {
         std::vector<int> acc_base(frm.S), pull_off, pull_ptr, pull_idx;
         for (int q = 0; q < frm.S; ++q) acc_base[q] = (int)frm.acc_off[q];
         dc_build_pull_lists(frm, acc_base, 3, pull_off, pull_ptr, pull_idx);
-        int *d_tq, *d_parent, *d_sched, *d_pull_off, *d_pull_ptr, *d_pull_idx;
-        if ((s = upload(c, F, &d_tq, tq_sn)) || (s = upload(c, F, &d_parent, frm.parent)) ||
-            (s = dalloc(c, F, &d_sched, 2 * ((size_t)frm.S + 1))) || (s = upload(c, F, &d_pull_off, pull_off)) ||
+        std::vector<int4> ftask, btask, need;
+        ms_plan(frm, tq_sn, ftask, btask, need);
+        std::vector<int> cneed;
+        for (int ch : frm.child) cneed.push_back(need[ch].x);
+        int *d_parent, *d_sched, *d_pull_off, *d_pull_ptr, *d_pull_idx, *d_cneed;
+        int4 *d_ftask, *d_btask, *d_need;
+        if ((s = upload(c, F, &d_cneed, cneed))) return s;
+        if ((s = upload(c, F, &d_ftask, ftask)) || (s = upload(c, F, &d_btask, btask)) ||
+            (s = upload(c, F, &d_need, need)) || (s = upload(c, F, &d_parent, frm.parent)) ||
+            (s = dalloc(c, F, &d_sched, 4 * (size_t)frm.S + 2)) || (s = dalloc(c, F, &fd.yvec, n3)) ||
+            (s = upload(c, F, &d_pull_off, pull_off)) ||
             (s = upload(c, F, &d_pull_ptr, pull_ptr)) || (s = upload(c, F, &d_pull_idx, pull_idx)))
             return s;
         fd.pull_off = d_pull_off;
         fd.pull_ptr = d_pull_ptr;
         fd.pull_idx = d_pull_idx;
-        fd.tq = d_tq;
+        fd.n_ftask = (int)ftask.size();
+        fd.n_btask = (int)btask.size();
+        fd.ftask = d_ftask;
+        fd.btask = d_btask;
+        fd.need = d_need;
+        fd.cneed = d_cneed;
         fd.parent = d_parent;
         fd.sched = d_sched;
         fd.fault = c->counters + 3;
         fd.tree = std::getenv("DC_LEVEL_SOLVES") ? 0 : 1;
-        CK(frontal_tree_grid(frm.max_f, &fd.tree_grid_f, &fd.tree_grid_b, &fd.tree_smem));
-        c->tq_h = std::move(tq_sn);
-        c->sn_inst_h = sn_inst;
+        CK(frontal_tree_grid(frm.max_f, &fd.tree_grid, &fd.tree_smem));
+        // instance of every task, for the lists of the instances still iterating
+        c->ms_finst_h.clear();
+        c->ms_binst_h.clear();
+        for (const int4& t : ftask) c->ms_finst_h.push_back(sn_inst[t.x]);
+        for (const int4& t : btask) c->ms_binst_h.push_back(sn_inst[t.x]);
     }
     c->fdv = fd;
     c->fds[0] = fd;
@@ -733,7 +749,18 @@ size_t estimate_device_bytes(const dc_ctx* c, const MeshPrep& mp, const ParamPre
         add(4 * (size_t)r.linv_size);
     }
     add(4 * (size_t)r.acc_size); add(12 * MF); add(12 * MF); add(12 * MF);
-    add(4 * (size_t)r.S); add(4 * (size_t)r.S); add(8 * ((size_t)r.S + 1));   // tree order, parents, tickets/flags
+    add(4 * (size_t)r.S); add(16 * (size_t)r.S + 8); add(12 * MF);   // parents, ticket/counters, y
+    {
+        std::vector<int> tq_ptr, tq_sn;
+        std::vector<int4> ftask, btask, need;
+        dc_build_tree_items(r, tq_ptr, tq_sn);
+        ms_plan(r, tq_sn, ftask, btask, need);
+        add(vbytes(ftask)); add(vbytes(btask)); add(vbytes(need)); add(vbytes(r.child));
+        if (B > 1) {   // task and chunk lists of the instances still iterating
+            add(4 * (ftask.size() + btask.size()));
+            add(4 * mp.chunks.size());
+        }
+    }
     {
         size_t nodes = 0;   // pull lists of the children's update vectors
         for (int q = 0; q < r.S; ++q) nodes += r.f[q] / 3 + 1;
