@@ -17,6 +17,7 @@
 // for bending) and a fixed-order per-node gather.
 #include "dc_internal.h"
 #include "dc_adjoint.h"
+#include "dc_gather.cuh"
 #include "dc_obstacle.cuh"
 #include "dc_polar.cuh"
 
@@ -212,95 +213,168 @@ __global__ void k_adj_setup_node(DevMesh dm, AdjDev ad, const d4* __restrict__ v
 // ----------------------------------------------------------------- H application
 
 // Element pass: per triangle E = h^2 w (dF - Dp[dF]) with dF = A_t z, stored as the
-// vertex-1 and vertex-2 columns E g_a^T; per vertex u = h^2 w_b (dq - Dp_b[dq]).
+// vertex-1 and vertex-2 columns E g_a^T; per vertex u = h^2 w_b (dq - Dp_b[dq]).  ST: a
+// triangle on three lanes, SN: a vertex, as in the forward local step.
+template <bool ST, bool SN>
 __global__ void k_adj_elem(DevMesh dm, AdjDev ad, const d4* __restrict__ z, d4* __restrict__ c1,
-                           d4* __restrict__ c2, d4* __restrict__ bu) {
-    int id = blockIdx.x * blockDim.x + threadIdx.x;
+                           d4* __restrict__ c2, d4* __restrict__ bu, int n_tri_threads) {
+    const int tid = blockIdx.x * blockDim.x + threadIdx.x;
     const double h2 = ad.h * ad.h;
-    if (id < dm.T) {
+    if (tid < n_tri_threads) {
+        const Lane3 L;
+        const int item = ST ? (tid >> 5) * 10 + L.group : tid;
+        const int id = min(item, dm.T - 1);
+        if (!ST && item >= dm.T) return;
         int4 tr = dm.tri[id];
-        if (ad.mask && ad.mask[ad.node_inst[tr.x]] == 0.0) return;
+        const bool off = ad.mask && ad.mask[ad.node_inst[tr.x]] == 0.0;
+        if (ST ? __all_sync(0xffffffffu, off) : off) return;
         d4 g = ld(dm.G + id);
-        d4 z0 = ld(z + tr.x), z1 = ld(z + tr.y), z2 = ld(z + tr.z);
-        double e1[3] = {z1.x - z0.x, z1.y - z0.y, z1.z - z0.z};
-        double e2[3] = {z2.x - z0.x, z2.y - z0.y, z2.z - z0.z};
-        double dF0[3], dF1[3];
-        for (int k = 0; k < 3; ++k) {
-            dF0[k] = e1[k] * g.x + e2[k] * g.z;
-            dF1[k] = e1[k] * g.y + e2[k] * g.w;
-        }
         d4 A0 = ld(ad.tr0 + id), A1 = ld(ad.tr1 + id), A2 = ld(ad.tr2 + id);
         double R0[3] = {A0.x, A0.y, A0.z}, R1[3] = {A1.x, A1.y, A1.z};
         double s00 = A0.w, s01 = A1.w, s11 = A2.x, itr = A2.y;
-        double r00 = R0[0] * dF0[0] + R0[1] * dF0[1] + R0[2] * dF0[2];
-        double r01 = R0[0] * dF1[0] + R0[1] * dF1[1] + R0[2] * dF1[2];
-        double r10 = R1[0] * dF0[0] + R1[1] * dF0[1] + R1[2] * dF0[2];
-        double r11 = R1[0] * dF1[0] + R1[1] * dF1[1] + R1[2] * dF1[2];
-        double om = (r10 - r01) * itr;
-        double w = h2 * dm.wt[id];
-        double E0[3], E1[3];
-        for (int k = 0; k < 3; ++k) {
-            double p0 = dF0[k] - R0[k] * r00 - R1[k] * r10;   // (I - R R^T) dF, column 0
-            double p1 = dF1[k] - R0[k] * r01 - R1[k] * r11;   // column 1
-            double dR0 = om * R1[k] + p0 * s00 + p1 * s01;    // R Om + (..) S^-1, column 0
-            double dR1 = -om * R0[k] + p0 * s01 + p1 * s11;   // column 1
-            E0[k] = w * (dF0[k] - dR0);
-            E1[k] = w * (dF1[k] - dR1);
+        double dF0[3], dF1[3];
+        if (ST) {
+            const double z0 = comp(z, tr.x, L.c), z1 = comp(z, tr.y, L.c), z2 = comp(z, tr.z, L.c);
+            const double e1 = z1 - z0, e2 = z2 - z0;
+            L.all(fma(e1, g.x, e2 * g.z), dF0);
+            L.all(fma(e1, g.y, e2 * g.w), dF1);
+        } else {
+            d4 z0 = ld(z + tr.x), z1 = ld(z + tr.y), z2 = ld(z + tr.z);
+            double e1[3] = {z1.x - z0.x, z1.y - z0.y, z1.z - z0.z};
+            double e2[3] = {z2.x - z0.x, z2.y - z0.y, z2.z - z0.z};
+            for (int k = 0; k < 3; ++k) {
+                dF0[k] = fma(e1[k], g.x, e2[k] * g.z);
+                dF1[k] = fma(e1[k], g.y, e2[k] * g.w);
+            }
         }
-        st(c1 + id, E0[0] * g.x + E1[0] * g.y, E0[1] * g.x + E1[1] * g.y, E0[2] * g.x + E1[2] * g.y);
-        st(c2 + id, E0[0] * g.z + E1[0] * g.w, E0[1] * g.z + E1[1] * g.w, E0[2] * g.z + E1[2] * g.w);
+        // (fused multiply-adds spelled out: both variants, and any later one, round alike)
+        auto dot = [](const double a[3], const double b[3]) {
+            return fma(a[2], b[2], fma(a[0], b[0], a[1] * b[1]));
+        };
+        const double r00 = dot(R0, dF0), r01 = dot(R0, dF1), r10 = dot(R1, dF0), r11 = dot(R1, dF1);
+        const double om = (r10 - r01) * itr;
+        const double w = h2 * dm.wt[id];
+        auto column = [&](double R0k, double R1k, double dF0k, double dF1k, double& E0, double& E1) {
+            const double p0 = fma(-R1k, r10, fma(-R0k, r00, dF0k));   // (I - R R^T) dF, column 0
+            const double p1 = fma(-R1k, r11, fma(-R0k, r01, dF1k));   // column 1
+            const double dR0 = fma(p1, s01, fma(p0, s00, om * R1k));  // R Om + (..) S^-1, column 0
+            const double dR1 = fma(p1, s11, fma(p0, s01, -om * R0k)); // column 1
+            E0 = w * (dF0k - dR0);
+            E1 = w * (dF1k - dR1);
+        };
+        if (ST) {
+            const int c = L.c;
+            auto mine = [&](const double v[3]) { return c == 0 ? v[0] : c == 1 ? v[1] : v[2]; };
+            double E0, E1;
+            column(mine(R0), mine(R1), mine(dF0), mine(dF1), E0, E1);
+            if (L.on && item < dm.T && !off) {
+                comp(c1, id, c) = fma(E0, g.x, E1 * g.y);
+                comp(c2, id, c) = fma(E0, g.z, E1 * g.w);
+            }
+            return;
+        }
+        double E0[3], E1[3];
+        for (int k = 0; k < 3; ++k) column(R0[k], R1[k], dF0[k], dF1[k], E0[k], E1[k]);
+        st(c1 + id, fma(E0[0], g.x, E1[0] * g.y), fma(E0[1], g.x, E1[1] * g.y), fma(E0[2], g.x, E1[2] * g.y));
+        st(c2 + id, fma(E0[0], g.z, E1[0] * g.w), fma(E0[1], g.z, E1[1] * g.w), fma(E0[2], g.z, E1[2] * g.w));
         return;
     }
-    int b = id - dm.T;
-    if (b >= dm.m) return;
-    if (ad.mask && ad.mask[ad.node_inst[b]] == 0.0) return;
-    double dq[3] = {0, 0, 0};
-    for (int k = dm.bptr[b]; k < dm.bptr[b + 1]; ++k) {
-        d4 zz = ld(z + dm.bidx[k]);
-        double l = dm.bval[k];
-        dq[0] += l * zz.x; dq[1] += l * zz.y; dq[2] += l * zz.z;
+    if (!SN) {
+        const int b = tid - n_tri_threads;
+        if (b >= dm.m) return;
+        if (ad.mask && ad.mask[ad.node_inst[b]] == 0.0) return;
+        double dq[3] = {0, 0, 0};
+        for (int k = dm.bptr[b]; k < dm.bptr[b + 1]; ++k) {
+            d4 zz = ld(z + dm.bidx[k]);
+            double l = dm.bval[k];
+            dq[0] += l * zz.x; dq[1] += l * zz.y; dq[2] += l * zz.z;
+        }
+        d4 q = ld(ad.bq + b);
+        const double qd = fma(q.z, dq[2], fma(q.x, dq[0], q.y * dq[1]));
+        const double w = h2 * dm.wb[b];
+        const double k1 = 1.0 - q.w;
+        st(bu + b, w * fma(k1, dq[0], q.w * qd * q.x), w * fma(k1, dq[1], q.w * qd * q.y),
+           w * fma(k1, dq[2], q.w * qd * q.z));
+        return;
     }
+    const Lane3 L;
+    const int first = ((tid - n_tri_threads) >> 5) * 10, item = first + L.group;
+    if (first >= dm.m) return;             // (whole warps)
+    const int b = min(item, dm.m - 1), c = L.c;
+    const bool off = ad.mask && ad.mask[ad.node_inst[b]] == 0.0;
+    if (__all_sync(0xffffffffu, off)) return;
+    const int lo = dm.bptr[b], hi = dm.bptr[b + 1];
+    double dq = 0.0;
+    list4(lo, hi, dm.bidx, dm.bval, [&](int k, const int j[4], const double l[4]) {
+        double u[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) u[q] = comp(z, j[q], c);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (k + q < hi) dq += l[q] * u[q];
+    });
+    double d[3];
+    L.all(dq, d);
     d4 q = ld(ad.bq + b);
-    double qd = q.x * dq[0] + q.y * dq[1] + q.z * dq[2];
-    double w = h2 * dm.wb[b];
-    double k1 = 1.0 - q.w;
-    st(bu + b, w * (k1 * dq[0] + q.w * qd * q.x), w * (k1 * dq[1] + q.w * qd * q.y),
-       w * (k1 * dq[2] + q.w * qd * q.z));
+    const double qd = fma(q.z, d[2], fma(q.x, d[0], q.y * d[1]));
+    const double w = h2 * dm.wb[b];
+    const double k1 = 1.0 - q.w;
+    if (L.on && item < dm.m && !off)
+        comp(bu, b, c) = w * fma(k1, dq, q.w * qd * (c == 0 ? q.x : c == 1 ? q.y : q.z));
 }
 
 // Gather of the element pass.  mode 0: out = Pi_B (H z)  (free nodes)
 //                               mode 1: out = w - Pi_B (H z)
 //                               mode 2: out = w - H z (no projection; free nodes)
 //                               mode 3: out = element part only (all m nodes)
+template <bool SN>
 __global__ void k_adj_gather(DevMesh dm, AdjDev ad, int mode, const d4* __restrict__ z,
                              const d4* __restrict__ c1, const d4* __restrict__ c2,
                              const d4* __restrict__ bu, const d4* __restrict__ w, d4* __restrict__ out) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    int n = (mode == 3) ? dm.m : dm.m_free;
-    if (i >= n) return;
-    if (ad.mask && ad.mask[ad.node_inst[i]] == 0.0) return;
-    double r0 = 0, r1 = 0, r2 = 0;
-    for (int k = dm.iptr[i]; k < dm.iptr[i + 1]; ++k) {
-        int e = dm.iidx[k];
-        int t = e / 3, a = e - 3 * t;
-        if (a == 1) {
-            d4 c = ld(c1 + t);
-            r0 += c.x; r1 += c.y; r2 += c.z;
-        } else if (a == 2) {
-            d4 c = ld(c2 + t);
-            r0 += c.x; r1 += c.y; r2 += c.z;
-        } else {
-            d4 ca = ld(c1 + t), cb = ld(c2 + t);
-            r0 -= ca.x + cb.x; r1 -= ca.y + cb.y; r2 -= ca.z + cb.z;
+    // SN: a node on three lanes; each finishes the node's value and stores its component
+    const Lane3 L;
+    const int n = (mode == 3) ? dm.m : dm.m_free, tid = blockIdx.x * blockDim.x + threadIdx.x;
+    const int first = SN ? (tid >> 5) * 10 : tid, item = first + (SN ? L.group : 0);
+    if (first >= n) return;                // (SN: whole warps)
+    const int i = min(item, n - 1);
+    const bool off = ad.mask && ad.mask[ad.node_inst[i]] == 0.0;
+    if (SN ? __all_sync(0xffffffffu, off) : off) return;
+    double r[3] = {0, 0, 0};
+    if (SN) {
+        L.all(dc_gather_elements(dm, i, L.c, 0.0, c1, c2, bu), r);
+        if (!L.on || item >= n || off) return;
+    } else {
+        for (int k = dm.iptr[i]; k < dm.iptr[i + 1]; ++k) {
+            int e = dm.iidx[k];
+            int t = e / 3, a = e - 3 * t;
+            if (a == 1) {
+                d4 c = ld(c1 + t);
+                r[0] += c.x; r[1] += c.y; r[2] += c.z;
+            } else if (a == 2) {
+                d4 c = ld(c2 + t);
+                r[0] += c.x; r[1] += c.y; r[2] += c.z;
+            } else {
+                d4 ca = ld(c1 + t), cb = ld(c2 + t);
+                r[0] -= ca.x + cb.x; r[1] -= ca.y + cb.y; r[2] -= ca.z + cb.z;
+            }
+        }
+        for (int k = dm.tbptr[i]; k < dm.tbptr[i + 1]; ++k) {
+            double l = dm.tbval[k];
+            d4 u = ld(bu + dm.tbidx[k]);
+            r[0] += l * u.x; r[1] += l * u.y; r[2] += l * u.z;
         }
     }
-    for (int k = dm.tbptr[i]; k < dm.tbptr[i + 1]; ++k) {
-        double l = dm.tbval[k];
-        d4 u = ld(bu + dm.tbidx[k]);
-        r0 += l * u.x; r1 += l * u.y; r2 += l * u.z;
-    }
+    double r0 = r[0], r1 = r[1], r2 = r[2];
+    auto store = [&](double a, double b, double c) {
+        if (!SN) {
+            st(out + i, a, b, c);
+            return;
+        }
+        comp(out, i, L.c) = L.c == 0 ? a : L.c == 1 ? b : c;
+        if (L.c == 2) comp(out, i, 3) = 0.0;   // (the Krylov reductions run over the padding)
+    };
     if (mode == 3) {
-        st(out + i, r0, r1, r2);
+        store(r0, r1, r2);
         return;
     }
     d4 zi = ld(z + i);
@@ -327,7 +401,7 @@ __global__ void k_adj_gather(DevMesh dm, AdjDev ad, int mode, const d4* __restri
         r0 = wi.x - r0; r1 = wi.y - r1; r2 = wi.z - r2;
         if (type == 1 && mode == 1) r0 = r1 = r2 = 0.0;
     }
-    st(out + i, r0, r1, r2);
+    store(r0, r1, r2);
 }
 
 // out = base + D+ w  (base may be null)
@@ -692,10 +766,15 @@ void adj_rhs(const DevMesh& dm, const AdjDev& ad, const d4* gx, const d4* gv, d4
 }
 void adj_apply_H(const DevMesh& dm, const AdjDev& ad, int mode, const d4* z, const d4* w, d4* out, cudaStream_t s) {
     dc_note_launch();
-    k_adj_elem<<<nblk((long)dm.T + dm.m, dm.bs_elem), dm.bs_elem, 0, s>>>(dm, ad, z, ad.c1, ad.c2, ad.bu);
+    const bool st = dm.T <= DC_SPLIT_TRIS, sn = dm.m <= DC_SPLIT_NODES;
+    const int nt = dc_group_threads(dm.T, st);
+    auto ke = st ? (sn ? k_adj_elem<true, true> : k_adj_elem<true, false>)
+                 : (sn ? k_adj_elem<false, true> : k_adj_elem<false, false>);
+    ke<<<nblk((long)nt + dc_group_threads(dm.m, sn), dm.bs_elem), dm.bs_elem, 0, s>>>(dm, ad, z, ad.c1, ad.c2, ad.bu, nt);
     int n = (mode == 3) ? dm.m : dm.m_free;
     dc_note_launch();
-    k_adj_gather<<<nblk(n, dm.bs_gather), dm.bs_gather, 0, s>>>(dm, ad, mode, z, ad.c1, ad.c2, ad.bu, w, out);
+    auto kg = sn ? k_adj_gather<true> : k_adj_gather<false>;
+    kg<<<nblk(dc_group_threads(n, sn), dm.bs_gather), dm.bs_gather, 0, s>>>(dm, ad, mode, z, ad.c1, ad.c2, ad.bu, w, out);
 }
 void adj_dplus(const DevMesh& dm, const AdjDev& ad, const d4* base, const d4* w, d4* out, cudaStream_t s) {
     dc_note_launch();

@@ -526,7 +526,7 @@ cudaError_t frontal_tree_grid(int max_f, int* grid, size_t* smem_out) {
 // that is ready.  A front whose two products have at most `target` entries is one task;
 // else each half is cut into row blocks of about that many, in multiples of eight rows (a
 // 32-byte sector of every column): 16 tasks per SM and sweep, within [4096, 65536]
-// entries (8192 entries, 32 KB, take an SM about 0.3 us, well below the cost of starting
+// entries (4096 entries, 16 KB, take an SM about 0.2 us, well below the cost of starting
 // a task).  No split changes a bit of the result.
 void ms_plan(const HostFronts& fr, const std::vector<int>& order, std::vector<int4>& ftask, std::vector<int4>& btask,
              std::vector<int4>& need) {

@@ -221,6 +221,7 @@ struct DevMesh {
     const int* fptr;                   // L^-1 rows (CSR), rows 0..m_free-1
     const int* fidx;
     const double* fval;
+    int fwd_contig;                    // 1: the columns of every L^-1 row are consecutive and end at the row
     int n_long, n_short;               // L^-1 rows split by length (CTA / warp per row)
     const int* long_rows;
     const int* short_rows;

@@ -17,6 +17,7 @@
 
 #include "dc_internal.h"
 #include "dc_obstacle.cuh"
+#include "dc_gather.cuh"
 #include "dc_polar.cuh"
 #include "dc_wait.cuh"
 
@@ -138,12 +139,49 @@ __device__ __forceinline__ void polar3x2(const double F[6], double R[6]) {
     dc_polar3x2(F, R, sinv, &itr);
 }
 
-// Local step.  Threads [0, T): triangles; [T, T + m): bending vertices.
+// Local step, triangles then bending vertices.  ST: a triangle on three lanes (150 FP64
+// instructions become 80 a lane), SN: a vertex on three lanes; else one thread each.
+// Where a vertex's rest shape is flat (s_b = 0) its projection is 0 and the velocity part
+// of A_b x is not needed (but by the mass splitting).
+template <bool ST, bool SN>
 __global__ void k_local(DevMesh dm, DevParams P, const d4* __restrict__ x_n, const d4* __restrict__ v,
-                        d4* __restrict__ c1, d4* __restrict__ c2, d4* __restrict__ bu) {
-    int id = blockIdx.x * blockDim.x + threadIdx.x;
+                        d4* __restrict__ c1, d4* __restrict__ c2, d4* __restrict__ bu, int n_tri_threads) {
+    const int tid = blockIdx.x * blockDim.x + threadIdx.x;
     const double h = P.h;
-    if (id < dm.T) {
+    if (tid < n_tri_threads) {
+        if (ST) {
+            const Lane3 L;
+            const int id = min((tid >> 5) * 10 + L.group, dm.T - 1);
+            const bool on = L.on && (tid >> 5) * 10 + L.group < dm.T;
+            const int c = L.c;
+            const int4 tr = dm.tri[id];
+            const d4 g = ld(dm.G + id);
+            const double w = dm.wt[id] * h;
+            const double x0 = comp(x_n, tr.x, c), x1 = comp(x_n, tr.y, c), x2 = comp(x_n, tr.z, c);
+            const double v0 = comp(v, tr.x, c), v1 = comp(v, tr.y, c), v2 = comp(v, tr.z, c);
+            const double e1 = x1 - x0, e2 = x2 - x0, f1 = v1 - v0, f2 = v2 - v0;
+            const double Fn0 = e1 * g.x + e2 * g.z, Fn1 = e1 * g.y + e2 * g.w;
+            const double F0 = Fn0 + h * (f1 * g.x + f2 * g.z), F1 = Fn1 + h * (f1 * g.y + f2 * g.w);
+            double F[6], R[6], sinv[3], itr;
+            L.all(F0, F);
+            L.all(F1, F + 3);
+            double R0, R1;
+            if (dc_polar3x2(F, R, sinv, &itr)) {
+                R0 = c == 0 ? R[0] : c == 1 ? R[1] : R[2];
+                R1 = c == 0 ? R[3] : c == 1 ? R[4] : R[5];
+            } else {
+                R0 = sinv[0] * F0 + sinv[1] * F1;
+                R1 = sinv[1] * F0 + sinv[2] * F1;
+            }
+            const double D0 = w * (R0 - (P.mass_split ? F0 : Fn0)), D1 = w * (R1 - (P.mass_split ? F1 : Fn1));
+            if (on) {
+                comp(c1, id, c) = D0 * g.x + D1 * g.y;
+                comp(c2, id, c) = D0 * g.z + D1 * g.w;
+            }
+            return;
+        }
+        const int id = tid;
+        if (id >= dm.T) return;
         int4 tr = dm.tri[id];
         d4 g = ld(dm.G + id);
         double w = dm.wt[id] * h;
@@ -171,146 +209,182 @@ __global__ void k_local(DevMesh dm, DevParams P, const d4* __restrict__ x_n, con
         st(c2 + id, D[0] * g.z + D[3] * g.w, D[1] * g.z + D[4] * g.w, D[2] * g.z + D[5] * g.w);
         return;
     }
-    int b = id - dm.T;
-    if (b >= dm.m) return;
-    double qn[3] = {0, 0, 0}, qv[3] = {0, 0, 0};
-    for (int k = dm.bptr[b]; k < dm.bptr[b + 1]; ++k) {
-        int j = dm.bidx[k];
-        double l = dm.bval[k];
-        d4 xj = ld(x_n + j), vj = ld(v + j);
-        qn[0] += l * xj.x; qn[1] += l * xj.y; qn[2] += l * xj.z;
-        qv[0] += l * vj.x; qv[1] += l * vj.y; qv[2] += l * vj.z;
+    if (!SN) {
+        const int b = tid - n_tri_threads;
+        if (b >= dm.m) return;
+        const double s = dm.sb[b];
+        const bool moving = s > 0.0 || P.mass_split;
+        double qn[3] = {0, 0, 0}, qv[3] = {0, 0, 0};
+        for (int k = dm.bptr[b]; k < dm.bptr[b + 1]; ++k) {
+            int j = dm.bidx[k];
+            double l = dm.bval[k];
+            d4 xj = ld(x_n + j);
+            qn[0] += l * xj.x; qn[1] += l * xj.y; qn[2] += l * xj.z;
+            if (moving) {
+                d4 vj = ld(v + j);
+                qv[0] += l * vj.x; qv[1] += l * vj.y; qv[2] += l * vj.z;
+            }
+        }
+        double q[3] = {qn[0] + h * qv[0], qn[1] + h * qv[1], qn[2] + h * qv[2]};
+        double p[3] = {0, 0, 0};
+        if (s > 0.0) {
+            double nq = sqrt(q[0] * q[0] + q[1] * q[1] + q[2] * q[2]);
+            if (nq > 1e-14 * s) {
+                double k = s / nq;
+                p[0] = k * q[0]; p[1] = k * q[1]; p[2] = k * q[2];
+            } else {
+                d4 qr = ld(dm.qrest + b);
+                p[0] = qr.x; p[1] = qr.y; p[2] = qr.z;
+            }
+        }
+        double w = dm.wb[b] * h;
+        const double* qr = P.mass_split ? q : qn;
+        st(bu + b, w * (p[0] - qr[0]), w * (p[1] - qr[1]), w * (p[2] - qr[2]));
+        return;
     }
-    double q[3] = {qn[0] + h * qv[0], qn[1] + h * qv[1], qn[2] + h * qv[2]};
-    double s = dm.sb[b];
-    double p[3] = {0, 0, 0};
+    const Lane3 L;
+    const int item = ((tid - n_tri_threads) >> 5) * 10 + L.group;
+    if (((tid - n_tri_threads) >> 5) * 10 >= dm.m) return;   // (whole warps)
+    const int b = min(item, dm.m - 1), c = L.c;
+    const double s = dm.sb[b];
+    const bool moving = s > 0.0 || P.mass_split;
+    double qn = 0.0, qv = 0.0;
+    list4(dm.bptr[b], dm.bptr[b + 1], dm.bidx, dm.bval, [&](int k, const int j[4], const double l[4]) {
+        const int n = dm.bptr[b + 1] - k;
+        double x[4], u[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            x[q] = comp(x_n, j[q], c);
+            u[q] = moving ? comp(v, j[q], c) : 0.0;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (q < n) {
+                qn += l[q] * x[q];
+                if (moving) qv += l[q] * u[q];
+            }
+    });
+    const double q = qn + h * qv;
+    double qa[3];
+    L.all(q, qa);
+    double p = 0.0;
     if (s > 0.0) {
-        double nq = sqrt(q[0] * q[0] + q[1] * q[1] + q[2] * q[2]);
+        double nq = sqrt(qa[0] * qa[0] + qa[1] * qa[1] + qa[2] * qa[2]);
         if (nq > 1e-14 * s) {
             double k = s / nq;
-            p[0] = k * q[0]; p[1] = k * q[1]; p[2] = k * q[2];
+            p = k * q;
         } else {
-            d4 qr = ld(dm.qrest + b);
-            p[0] = qr.x; p[1] = qr.y; p[2] = qr.z;
+            p = comp(dm.qrest, b, c);
         }
     }
-    double w = dm.wb[b] * h;
-    const double* qr = P.mass_split ? q : qn;
-    st(bu + b, w * (p[0] - qr[0]), w * (p[1] - qr[1]), w * (p[2] - qr[2]));
+    const double w = dm.wb[b] * h;
+    if (L.on && item < dm.m) comp(bu, b, c) = w * (p - (P.mass_split ? q : qn));
 }
 
+// Right-hand side.  SN: a free node on three lanes, else one thread.
+template <bool SN>
 __global__ void k_gather_rhs(DevMesh dm, DevParams P, const d4* __restrict__ v_n, const d4* __restrict__ c1,
                              const d4* __restrict__ c2, const d4* __restrict__ bu, const d4* __restrict__ f,
                              d4* __restrict__ b) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= dm.m_free) return;
-    d4 vn = ld(v_n + i);
-    double mi = dm.mass[i];
-    double r0 = mi * (vn.x + P.h * P.g[0]);
-    double r1 = mi * (vn.y + P.h * P.g[1]);
-    double r2 = mi * (vn.z + P.h * P.g[2]);
-    for (int k = dm.iptr[i]; k < dm.iptr[i + 1]; ++k) {
-        int e = dm.iidx[k];
-        int t = e / 3, a = e - 3 * t;
-        if (a == 1) {
-            d4 c = ld(c1 + t);
-            r0 += c.x; r1 += c.y; r2 += c.z;
-        } else if (a == 2) {
-            d4 c = ld(c2 + t);
-            r0 += c.x; r1 += c.y; r2 += c.z;
-        } else {
-            d4 ca = ld(c1 + t), cb = ld(c2 + t);
-            r0 -= ca.x + cb.x; r1 -= ca.y + cb.y; r2 -= ca.z + cb.z;
+    if (!SN) {
+        int i = blockIdx.x * blockDim.x + threadIdx.x;
+        if (i >= dm.m_free) return;
+        d4 vn = ld(v_n + i);
+        double mi = dm.mass[i];
+        double r0 = mi * (vn.x + P.h * P.g[0]);
+        double r1 = mi * (vn.y + P.h * P.g[1]);
+        double r2 = mi * (vn.z + P.h * P.g[2]);
+        for (int k = dm.iptr[i]; k < dm.iptr[i + 1]; ++k) {
+            int e = dm.iidx[k];
+            int t = e / 3, a = e - 3 * t;
+            if (a == 1) {
+                d4 c = ld(c1 + t);
+                r0 += c.x; r1 += c.y; r2 += c.z;
+            } else if (a == 2) {
+                d4 c = ld(c2 + t);
+                r0 += c.x; r1 += c.y; r2 += c.z;
+            } else {
+                d4 ca = ld(c1 + t), cb = ld(c2 + t);
+                r0 -= ca.x + cb.x; r1 -= ca.y + cb.y; r2 -= ca.z + cb.z;
+            }
         }
+        for (int k = dm.tbptr[i]; k < dm.tbptr[i + 1]; ++k) {
+            double l = dm.tbval[k];
+            d4 u = ld(bu + dm.tbidx[k]);
+            r0 += l * u.x; r1 += l * u.y; r2 += l * u.z;
+        }
+        d4 fi = ld(f + i);
+        st(b + i, r0 + P.h * fi.x, r1 + P.h * fi.y, r2 + P.h * fi.z);
+        return;
     }
-    for (int k = dm.tbptr[i]; k < dm.tbptr[i + 1]; ++k) {
-        double l = dm.tbval[k];
-        d4 u = ld(bu + dm.tbidx[k]);
-        r0 += l * u.x; r1 += l * u.y; r2 += l * u.z;
-    }
-    d4 fi = ld(f + i);
-    st(b + i, r0 + P.h * fi.x, r1 + P.h * fi.y, r2 + P.h * fi.z);
+    const int id = blockIdx.x * blockDim.x + threadIdx.x, i = id / 3, c = id - 3 * i;
+    if (i >= dm.m_free) return;
+    const double mi = dm.mass[i];
+    double r = mi * (comp(v_n, i, c) + P.h * (c == 0 ? P.g[0] : c == 1 ? P.g[1] : P.g[2]));
+    r = dc_gather_elements(dm, i, c, r, c1, c2, bu);
+    comp(b, i, c) = r + P.h * comp(f, i, c);
 }
 
-// y_i = sum_k Linv(i,k) b_k, one warp per row, fixed lane order.
-__device__ __forceinline__ void warp_row(const int* __restrict__ ptr, const int* __restrict__ idx,
-                                         const double* __restrict__ val, const d4* __restrict__ in, int row,
-                                         double& s0, double& s1, double& s2) {
-    int lane = threadIdx.x & 31;
-    s0 = s1 = s2 = 0.0;
-    for (int k = ptr[row] + lane; k < ptr[row + 1]; k += 32) {
-        double a = val[k];
-        d4 u = ld(in + idx[k]);
-        s0 += a * u.x; s1 += a * u.y; s2 += a * u.z;
-    }
+// Butterfly sums of three values over a warp (the sums of three separate butterflies):
+// once half of the lanes hold copies they take another value's adds, 8 FP64 instructions
+// instead of 15.  Lane 0 returns the three sums.
+__device__ __forceinline__ void warp_sum3(double& s0, double& s1, double& s2) {
+    const int lane = threadIdx.x & 31;
+    s0 += __shfl_xor_sync(0xffffffffu, s0, 16);
+    s1 += __shfl_xor_sync(0xffffffffu, s1, 16);
+    s2 += __shfl_xor_sync(0xffffffffu, s2, 16);
+    double a = lane & 16 ? s1 : s0;
+    a += __shfl_xor_sync(0xffffffffu, a, 8);
+    s2 += __shfl_xor_sync(0xffffffffu, s2, 8);
+    a = lane & 8 ? s2 : a;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-    }
+    for (int o = 4; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    s0 = a;
+    s1 = __shfl_sync(0xffffffffu, a, 16);
+    s2 = __shfl_sync(0xffffffffu, a, 8);
 }
 
 // Forward substitution with the explicit inverse factor, y = L^-1 b.  Rows with
 // more than LONG_ROW nonzeros (separator rows near the top of the elimination
 // tree) get a whole CTA each; the other rows one warp each.  Both reductions
-// run in a fixed order, so the result is bitwise repeatable.
+// run in a fixed order, so the result is bitwise repeatable.  CONTIG: every row's
+// columns are consecutive and end at the row itself (in a postordered elimination tree a
+// row of L^-1 is its node's subtree), so no index is read.
+template <bool CONTIG>
 __global__ void __launch_bounds__(256) k_solve_fwd(DevMesh dm, const d4* __restrict__ b, d4* __restrict__ y) {
     __shared__ double red[3][8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if ((int)blockIdx.x < dm.n_long) {
-        const int row = dm.long_rows[blockIdx.x];
-        double s0 = 0, s1 = 0, s2 = 0;
-        const int lo = dm.fptr[row], hi = dm.fptr[row + 1];
-        int k = lo + threadIdx.x;
-        for (; k + 256 < hi; k += 512) {
-            const double a0 = dm.fval[k], a1 = dm.fval[k + 256];
-            const d4 u0 = ld(b + dm.fidx[k]), u1 = ld(b + dm.fidx[k + 256]);
-            s0 += a0 * u0.x + a1 * u1.x; s1 += a0 * u0.y + a1 * u1.y; s2 += a0 * u0.z + a1 * u1.z;
-        }
-        if (k < hi) {
-            const double a = dm.fval[k];
-            const d4 u = ld(b + dm.fidx[k]);
-            s0 += a * u.x; s1 += a * u.y; s2 += a * u.z;
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-            s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-            s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-        }
-        if (lane == 0) { red[0][warp] = s0; red[1][warp] = s1; red[2][warp] = s2; }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            double t0 = 0, t1 = 0, t2 = 0;
-            for (int w = 0; w < 8; ++w) { t0 += red[0][w]; t1 += red[1][w]; t2 += red[2][w]; }
-            st(y + row, t0, t1, t2);
-        }
-        return;
-    }
+    const bool wide = (int)blockIdx.x < dm.n_long;
     const int q = ((int)blockIdx.x - dm.n_long) * 8 + warp;
-    if (q >= dm.n_short) return;
-    const int row = dm.short_rows[q];
-    double s0 = 0, s1 = 0, s2 = 0;
+    if (!wide && q >= dm.n_short) return;
+    const int row = wide ? dm.long_rows[blockIdx.x] : dm.short_rows[q];
     const int lo = dm.fptr[row], hi = dm.fptr[row + 1];
-    int k = lo + lane;
-    for (; k + 32 < hi; k += 64) {
-        const double a0 = dm.fval[k], a1 = dm.fval[k + 32];
-        const d4 u0 = ld(b + dm.fidx[k]), u1 = ld(b + dm.fidx[k + 32]);
+    const int stride = wide ? 256 : 32;
+    double s0 = 0, s1 = 0, s2 = 0;
+    auto at = [&](int k) { return ld(b + (CONTIG ? row - (hi - 1 - k) : dm.fidx[k])); };
+    int k = lo + (wide ? threadIdx.x : lane);
+    for (; k + stride < hi; k += 2 * stride) {
+        const double a0 = dm.fval[k], a1 = dm.fval[k + stride];
+        const d4 u0 = at(k), u1 = at(k + stride);
         s0 += a0 * u0.x + a1 * u1.x; s1 += a0 * u0.y + a1 * u1.y; s2 += a0 * u0.z + a1 * u1.z;
     }
     if (k < hi) {
         const double a = dm.fval[k];
-        const d4 u = ld(b + dm.fidx[k]);
+        const d4 u = at(k);
         s0 += a * u.x; s1 += a * u.y; s2 += a * u.z;
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+    warp_sum3(s0, s1, s2);
+    if (!wide) {
+        if (lane == 0) st(y + row, s0, s1, s2);
+        return;
     }
-    if (lane == 0) st(y + row, s0, s1, s2);
+    if (lane == 0) { red[0][warp] = s0; red[1][warp] = s1; red[2][warp] = s2; }
+    __syncthreads();
+    if (threadIdx.x < 3) {
+        double t = 0;
+        for (int w = 0; w < 8; ++w) t += red[threadIdx.x][w];
+        comp(y, row, threadIdx.x) = t;
+    }
 }
 
 // Per-node Signorini-Coulomb solve (Eq. contact_1-3, reading R5) in world
@@ -379,8 +453,15 @@ __global__ void k_solve_bwd(DevMesh dm, DevParams P, const d4* __restrict__ y, d
                             double* __restrict__ c_out) {
     int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (row >= dm.m_free) return;
-    double s0, s1, s2;
-    warp_row(dm.kptr, dm.kidx, dm.kval, y, row, s0, s1, s2);
+    double s0 = 0, s1 = 0, s2 = 0;
+    const int hi = dm.kptr[row + 1];
+#pragma unroll 4
+    for (int k = dm.kptr[row] + (threadIdx.x & 31); k < hi; k += 32) {
+        const double a = dm.kval[k];
+        const d4 u = ld(y + dm.kidx[k]);
+        s0 += a * u.x; s1 += a * u.y; s2 += a * u.z;
+    }
+    warp_sum3(s0, s1, s2);
     if ((threadIdx.x & 31) != 0) return;
     finish_row(P, row, s0, s1, s2, out, mode, contact, nb, cc, f, case_, c_out);
 }
@@ -1049,12 +1130,18 @@ void launch_detect(const DevMesh& dm, const DevParams& P, const d4* x_n, const d
 void launch_local(const DevMesh& dm, const DevParams& P, const d4* x_n, const d4* v, d4* c1, d4* c2,
                   d4* bu, cudaStream_t s) {
     dc_note_launch();
-    k_local<<<nblk((long)dm.T + dm.m, dm.bs_local), dm.bs_local, 0, s>>>(dm, P, x_n, v, c1, c2, bu);
+    const bool st = dm.T <= DC_SPLIT_TRIS, sn = dm.m <= DC_SPLIT_NODES;
+    const int nt = dc_group_threads(dm.T, st);
+    auto k = st ? (sn ? k_local<true, true> : k_local<true, false>) : (sn ? k_local<false, true> : k_local<false, false>);
+    k<<<nblk((long)nt + dc_group_threads(dm.m, sn), dm.bs_local), dm.bs_local, 0, s>>>(dm, P, x_n, v, c1, c2, bu, nt);
 }
 void launch_gather_rhs(const DevMesh& dm, const DevParams& P, const d4* v_n, const d4* c1, const d4* c2,
                        const d4* bu, const d4* f, d4* b, cudaStream_t s) {
     dc_note_launch();
-    k_gather_rhs<<<nblk(dm.m_free, dm.bs_gather), dm.bs_gather, 0, s>>>(dm, P, v_n, c1, c2, bu, f, b);
+    if (dm.m <= DC_SPLIT_NODES)
+        k_gather_rhs<true><<<nblk(3L * dm.m_free, dm.bs_gather), dm.bs_gather, 0, s>>>(dm, P, v_n, c1, c2, bu, f, b);
+    else
+        k_gather_rhs<false><<<nblk(dm.m_free, dm.bs_gather), dm.bs_gather, 0, s>>>(dm, P, v_n, c1, c2, bu, f, b);
 }
 namespace {
 size_t ps_smem(int fs) { return (6 * (size_t)fs + 3 * (size_t)GV_ROWS * GV_MAXG) * sizeof(double); }
@@ -1127,7 +1214,11 @@ void launch_solve_fwd(const DevMesh& dm, const d4* b, d4* y, cudaStream_t s) {
         return;
     }
     dc_note_launch();
-    k_solve_fwd<<<dm.n_long + nblk(dm.n_short, 8), 256, 0, s>>>(dm, b, y);
+    const int grid = dm.n_long + nblk(dm.n_short, 8);
+    if (dm.fwd_contig)
+        k_solve_fwd<true><<<grid, 256, 0, s>>>(dm, b, y);
+    else
+        k_solve_fwd<false><<<grid, 256, 0, s>>>(dm, b, y);
 }
 void launch_solve_fwd_skip(const DevMesh& dm, const d4* b, d4* y, int skip, cudaStream_t s) {
     const PSolveDev& ps = dm.ps;

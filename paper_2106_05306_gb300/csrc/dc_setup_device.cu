@@ -394,6 +394,13 @@ dc_status upload_params(dc_ctx* c, ParamPrep& pp) {
         (!c->mesh_rec.empty() && (s = upload(c, P, &d_mesh, c->mesh_rec))))
         return s;
     DevMesh& dm = c->dm;
+    dm.fwd_contig = 1;
+    for (int r = 0; r < MF && dm.fwd_contig; ++r)
+        for (int q = hfm.fptr[r]; q < hfm.fptr[r + 1]; ++q)
+            if (hfm.fidx[q] != r - (hfm.fptr[r + 1] - 1 - q)) {
+                dm.fwd_contig = 0;
+                break;
+            }
     dm.n_long = (int)pp.long_rows.size();
     dm.n_short = (int)pp.short_rows.size();
     dm.long_rows = d_long;
