@@ -61,14 +61,16 @@ __global__ void k_adj_setup_tri(DevMesh dm, const d4* __restrict__ x1, d4* __res
     const double s00 = sinv[0], s01 = sinv[1], s11 = sinv[2];
     // per vertex v of the triangle: a_v = (g_v0 R1 - g_v1 R0) / tr S, and the
     // projector P = I - R0 R0^T - R1 R1^T (the front assembly reads them for
-    // every pair of the triangle's vertices instead of forming them again)
+    // every pair of the triangle's vertices instead of forming them again), with tr S
+    // (0 for a collapsed triangle: a_v = 0)
+    const double trS = it > 0.0 ? 1.0 / it : 0.0;
     for (int v = 0; v < 3; ++v) {
         double gv0, gv1;
         if (v == 1) { gv0 = g.x; gv1 = g.y; }
         else if (v == 2) { gv0 = g.z; gv1 = g.w; }
         else { gv0 = -(g.x + g.z); gv1 = -(g.y + g.w); }
         st(tav + 4 * (long)t + v, (gv0 * R[3] - gv1 * R[0]) * it, (gv0 * R[4] - gv1 * R[1]) * it,
-           (gv0 * R[5] - gv1 * R[2]) * it);
+           (gv0 * R[5] - gv1 * R[2]) * it, trS);
     }
     double P[9];
     for (int r = 0; r < 3; ++r)

@@ -134,6 +134,7 @@ std::string dc_build_fronts(const HostMesh& hm, const HostFactor& hf, HostFronts
         colstart[j + 1] = colstart[j] + (int)rows[j].size();
     }
     const int NP = colstart[n];
+    constexpr int PR_WINDOW = 2048;
     fr.pr_i.resize(NP);
     fr.pr_j.resize(NP);
     fr.pr_dst.resize(NP);
@@ -180,9 +181,32 @@ std::string dc_build_fronts(const HostMesh& hm, const HostFactor& hf, HostFronts
                 if (i < j || i >= n || j >= n) continue;
                 contrib[pair_id(i, j)].push_back({-(b + 1), hm.bval[u] * hm.bval[v]});
             }
+    // Within windows of PR_WINDOW pairs the longest sums come first, so that a warp of the
+    // assembly holds pairs of one kind (diagonal, edge, bending only); a window stays within
+    // a few columns of the fronts.  A pair's sum keeps its own order.
+    std::vector<int> order(NP);
+    for (int id = 0; id < NP; ++id) order[id] = id;
+    auto work = [&](int id) {               // a triangle's term costs several bending terms
+        long w = 0;
+        for (const auto& e : contrib[id]) w += e.first >= 0 ? 64 : 1;
+        return w;
+    };
+    std::vector<long> cost(NP);
+    for (int id = 0; id < NP; ++id) cost[id] = work(id);
+    for (int w = 0; w < NP; w += PR_WINDOW)
+        std::stable_sort(order.begin() + w, order.begin() + std::min(NP, w + PR_WINDOW),
+                         [&](int a, int b) { return cost[a] > cost[b]; });
+    auto permute = [&](auto& v) {
+        auto u = v;
+        for (int id = 0; id < NP; ++id) v[id] = u[order[id]];
+    };
+    permute(fr.pr_i);
+    permute(fr.pr_j);
+    permute(fr.pr_dst);
+    permute(fr.pr_ld);
     fr.pr_cptr.assign(1, 0);
     for (int id = 0; id < NP; ++id) {
-        for (auto& e : contrib[id]) {
+        for (auto& e : contrib[order[id]]) {
             fr.pr_code.push_back(e.first);
             fr.pr_coef.push_back(e.second);
         }
