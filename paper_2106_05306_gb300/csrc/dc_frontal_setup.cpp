@@ -304,11 +304,25 @@ void dc_merge_psolve(const std::vector<HostPSolve>& P, HostPSolve& out) {
     out.n_pant = to;
 }
 
+constexpr int SMS = 152;
+
+// From 32 small fronts per SM on, groups of four on eight 128-thread CTAs an SM: with
+// groups of eight 60% of the warps stood at their CTA's barriers (an item's warps wait for
+// its slowest, a large front's phases do not fill 256 threads).  One solve of 16, 32, 64, 96,
+// 160 cloths (23000 to 267000 nodes), groups of eight -> four: 238 -> 238, 295 -> 333, 451
+// -> 449, 526 -> 500, 676 -> 595 us; one 200 x 200 cloth, bound by its top fronts, 36.8 -> 40.1
+// ms a rollout.
+int ps_kind(int n_small) {
+    return n_small <= 8 * SMS ? PS_KIND_ALONE : n_small <= 32 * SMS ? PS_KIND_GROUPS : PS_KIND_MANY;
+}
+
 // Work items of the tree-scheduled sweeps, in a topological order (every front
 // after its children): fronts farther from their root come first, so the longest
 // remaining chains start earliest.  A front of more than DC_PS_SMALL nodes is an
-// item alone (one CTA); smaller fronts of equal depth go up to DC_PS_WARPS to an
-// item (one warp each).  Item q is tq_sn[tq_ptr[q] .. tq_ptr[q + 1]).
+// item alone (one CTA); smaller fronts of equal depth go up to DC_PS_WARPS (half
+// of that in PS_KIND_MANY) to an item, one warp each, the larger ones first, since
+// an item's warps wait for its slowest (96 cloths: a rollout 63.6 -> 62.8 ms).  Item q is
+// tq_sn[tq_ptr[q] .. tq_ptr[q + 1]).
 void dc_build_tree_items(const HostFronts& fr, std::vector<int>& tq_ptr, std::vector<int>& tq_sn) {
     std::vector<int> depth(fr.S, 0), order(fr.S);
     for (int s = 0; s < fr.S; ++s) {
@@ -318,8 +332,12 @@ void dc_build_tree_items(const HostFronts& fr, std::vector<int>& tq_ptr, std::ve
     auto large = [&](int s) { return fr.f[s] / 3 > DC_PS_SMALL; };
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
         if (depth[a] != depth[b]) return depth[a] > depth[b];
-        return large(a) && !large(b);
+        if (large(a) != large(b)) return large(a);
+        return !large(a) && (long)fr.f[a] * fr.p[a] > (long)fr.f[b] * fr.p[b];
     });
+    int n_small = 0;
+    for (int s = 0; s < fr.S; ++s) n_small += !large(s);
+    const int group = ps_kind(n_small) == PS_KIND_MANY ? DC_PS_WARPS / 2 : DC_PS_WARPS;
     tq_ptr.assign(1, 0);
     tq_sn.clear();
     for (size_t k = 0; k < order.size();) {
@@ -328,7 +346,7 @@ void dc_build_tree_items(const HostFronts& fr, std::vector<int>& tq_ptr, std::ve
             tq_sn.push_back(s);
             ++k;
         } else {
-            for (int n = 0; k < order.size() && n < DC_PS_WARPS && !large(order[k]) && depth[order[k]] == depth[s]; ++n)
+            for (int n = 0; k < order.size() && n < group && !large(order[k]) && depth[order[k]] == depth[s]; ++n)
                 tq_sn.push_back(order[k++]);
         }
         tq_ptr.push_back((int)tq_sn.size());
@@ -349,8 +367,7 @@ void dc_build_tree_items(const HostFronts& fr, std::vector<int>& tq_ptr, std::ve
 // every SM has other work (200 x 200 nodes, 12 per SM: 24.0 ms in groups, 30.5 alone).
 // No choice here changes a bit of the result.
 void dc_build_ps_tasks(const HostFronts& fr, const std::vector<int>& tq_ptr, const std::vector<int>& tq_sn,
-                       std::vector<int4>& ftask, std::vector<int4>& btask, std::vector<int4>& need, bool& alone) {
-    constexpr int SMS = 152;
+                       std::vector<int4>& ftask, std::vector<int4>& btask, std::vector<int4>& need, int& kind) {
     auto large = [&](int s) { return fr.f[s] / 3 > DC_PS_SMALL; };
     long long total = 0;
     int n_small = 0;
@@ -360,7 +377,7 @@ void dc_build_ps_tasks(const HostFronts& fr, const std::vector<int>& tq_ptr, con
         n_small += !large(s);
     }
     const long long target = std::min<long long>(8192, std::max<long long>(1600, total / (SMS * 32)));
-    alone = n_small <= 8 * SMS;
+    kind = ps_kind(n_small);
     need.assign(fr.S, make_int4(1, 0, 1, 0));
     ftask.clear();
     btask.clear();
@@ -394,7 +411,7 @@ void dc_build_ps_tasks(const HostFronts& fr, const std::vector<int>& tq_ptr, con
                 const long long ns = fr.p[s] / 3, nu = fr.f[s] / 3 - ns;
                 if (!large(s)) {
                     if (second) continue;
-                    if (alone)
+                    if (kind == PS_KIND_ALONE)
                         for (int e = tq_ptr[q]; e < tq_ptr[q + 1]; ++e) out.push_back(make_int4(tq_sn[e], PS_FRONT, 0, 0));
                     else
                         out.push_back(make_int4(tq_ptr[q], PS_GROUP, tq_ptr[q + 1] - tq_ptr[q], 0));

@@ -523,6 +523,9 @@ __device__ __forceinline__ void ps_pull_end(const PSolveDev& ps, const PsPull& q
     w[2 * stride] = z;
 }
 
+// Rows of one pass of a CTA (its partial sums' shared memory; no bit depends on it).
+__host__ __device__ constexpr int ps_pass_rows(int threads) { return threads > 128 ? GV_ROWS : GV_ROWS / 2; }
+
 // Column-major product on one CTA with three right-hand sides: t_c,i = sum_k
 // A[k * lda + i] v[c * ldv + k] for rows r_lo <= i < r_hi and k < K (TRI 1: only
 // k <= i; TRI 2: only k >= i).  wait() blocks until the vectors are there and returns
@@ -538,7 +541,8 @@ __device__ __forceinline__ bool ps_rows(const double* __restrict__ A, long lda, 
                                         Fill fill, Fin fin) {
     const int nt = blockDim.x, tid = threadIdx.x;
     const int G = gv_groups(K), C = (K + G - 1) / G;
-    constexpr int RS = GV_ROWS * GV_MAXG;      // stride between the three columns' partial sums
+    const int ROWS = ps_pass_rows(nt);         // rows of a pass
+    const int RS = ROWS * GV_MAXG;             // stride between the three columns' partial sums
     auto range = [&](int i, int g, int& k0, int& k1) {
         k0 = g * C;
         k1 = min(K, k0 + C);
@@ -554,7 +558,7 @@ __device__ __forceinline__ bool ps_rows(const double* __restrict__ A, long lda, 
     };
     double a[SPLIT ? PS_CH : 1];
     if (SPLIT) {
-        const int R = min(GV_ROWS, r_hi - r_lo);
+        const int R = min(ROWS, r_hi - r_lo);
         if (tid < 3 * R * G) {
             int c, g, r, k0, k1;
             decode(tid, R, c, g, r);
@@ -571,8 +575,8 @@ __device__ __forceinline__ bool ps_rows(const double* __restrict__ A, long lda, 
     if (!wait()) return false;
     fill();
     __syncthreads();
-    for (int i0 = r_lo; i0 < r_hi; i0 += GV_ROWS) {
-        const int R = min(GV_ROWS, r_hi - i0);
+    for (int i0 = r_lo; i0 < r_hi; i0 += ROWS) {
+        const int R = min(ROWS, r_hi - i0);
         for (int item = tid; item < (SPLIT ? 3 : 1) * R * G; item += nt) {
             int c, g, r, k0, k1;
             decode(item, R, c, g, r);
@@ -597,7 +601,7 @@ __device__ __forceinline__ bool ps_rows(const double* __restrict__ A, long lda, 
                     s += *col * vc[q];
                     col += lda;
                 }
-                red[c * RS + g * GV_ROWS + r] = s;
+                red[c * RS + g * ROWS + r] = s;
             } else {
                 double a0 = 0.0, a1 = 0.0, a2 = 0.0;
 #pragma unroll 4
@@ -608,9 +612,9 @@ __device__ __forceinline__ bool ps_rows(const double* __restrict__ A, long lda, 
                     a1 += x * v[ldv + k];
                     a2 += x * v[2 * ldv + k];
                 }
-                red[g * GV_ROWS + r] = a0;
-                red[RS + g * GV_ROWS + r] = a1;
-                red[2 * RS + g * GV_ROWS + r] = a2;
+                red[g * ROWS + r] = a0;
+                red[RS + g * ROWS + r] = a1;
+                red[2 * RS + g * ROWS + r] = a2;
             }
         }
         __syncthreads();
@@ -619,7 +623,7 @@ __device__ __forceinline__ bool ps_rows(const double* __restrict__ A, long lda, 
             // the row's chunks with entries: [gl, gh)
             const int gl = TRI == 2 ? i / C : 0, gh = TRI == 1 ? i / C + 1 : G;
             double t = 0.0;
-            for (int g = gl; g < gh; ++g) t += red[c * RS + g * GV_ROWS + r];
+            for (int g = gl; g < gh; ++g) t += red[c * RS + g * ROWS + r];
             red[c * RS + r] = t;
         }
         __syncthreads();
@@ -956,17 +960,23 @@ __device__ __forceinline__ int* ps_counter(const PSolveDev& ps, bool fwd, int s,
     return base + (mid ? ps.S : 0) + s;
 }
 
+constexpr int ps_tree_threads(int kind) { return kind == PS_KIND_MANY ? 128 : 256; }
+constexpr int ps_tree_ctas(int kind) { return kind == PS_KIND_ALONE ? 1 : kind == PS_KIND_GROUPS ? 4 : 8; }
+// kernel instance of a kind
+#define PS_PICK(k, kind) ((kind) == PS_KIND_ALONE ? k<PS_KIND_ALONE> : (kind) == PS_KIND_GROUPS ? k<PS_KIND_GROUPS> : k<PS_KIND_MANY>)
+
 // FWD / BWD: which sweeps this launch runs (both: the backward tasks follow the
-// forward ones in ticket order).  ALONE: no groups of small fronts (ps.alone); such a
-// context has fewer tasks than the chip has room for, its time is the chain of waits,
-// and the kernel loads what it can before them.  The other kernel keeps four CTAs on
-// an SM instead, whose work hides one another's waits.
-template <bool FWD, bool BWD, bool ALONE>
+// forward ones in ticket order).  KIND (ps_kind): a context without groups of small fronts
+// has fewer tasks than the chip has room for, its time is the chain of waits, and the
+// kernel loads what it can before them.  The other kernels keep four CTAs of 256 or eight
+// of 128 threads on an SM instead, whose work hides one another's waits.
+template <bool FWD, bool BWD, int KIND>
 __device__ __forceinline__ void ps_run(const PSolveDev& ps, const DevParams& P, const d4* __restrict__ b,
                                        d4* __restrict__ y, d4* __restrict__ out, int mode,
                                        const int* __restrict__ contact, const d4* __restrict__ nb,
                                        const double* __restrict__ cc, d4* __restrict__ f, int* __restrict__ case_,
                                        double* __restrict__ c_out, double* __restrict__ smd) {
+    constexpr bool ALONE = KIND == PS_KIND_ALONE;
     __shared__ int s_item, s_ok;
     int* ticket = FWD ? ps.sched : ps.sched + 2 * ps.S + 1;
     const int nf = FWD ? ps.n_ftask : 0, n = nf + (BWD ? ps.n_btask : 0);
@@ -1020,33 +1030,33 @@ __device__ __forceinline__ void ps_run(const PSolveDev& ps, const DevParams& P, 
     }
 }
 
-template <bool ALONE>
-__global__ void __launch_bounds__(256, ALONE ? 1 : 4) k_ps_fwd_tree(PSolveDev ps, const d4* __restrict__ b,
+template <int KIND>
+__global__ void __launch_bounds__(ps_tree_threads(KIND), ps_tree_ctas(KIND)) k_ps_fwd_tree(PSolveDev ps, const d4* __restrict__ b,
                                                                     d4* __restrict__ y) {
     extern __shared__ double smd[];
     const DevParams none{};
-    ps_run<true, false, ALONE>(ps, none, b, y, nullptr, 0, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, smd);
+    ps_run<true, false, KIND>(ps, none, b, y, nullptr, 0, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, smd);
 }
 
-template <bool ALONE>
-__global__ void __launch_bounds__(256, ALONE ? 1 : 4)
+template <int KIND>
+__global__ void __launch_bounds__(ps_tree_threads(KIND), ps_tree_ctas(KIND))
     k_ps_bwd_tree(PSolveDev ps, DevParams P, d4* __restrict__ y, d4* __restrict__ out, int mode,
                   const int* __restrict__ contact, const d4* __restrict__ nb, const double* __restrict__ cc,
                   d4* __restrict__ f, int* __restrict__ case_, double* __restrict__ c_out) {
     extern __shared__ double smd[];
-    ps_run<false, true, ALONE>(ps, P, nullptr, y, out, mode, contact, nb, cc, f, case_, c_out, smd);
+    ps_run<false, true, KIND>(ps, P, nullptr, y, out, mode, contact, nb, cc, f, case_, c_out, smd);
 }
 
 // Both sweeps of one global step as one launch: the backward work of small trees
 // runs while the forward sweeps of large ones are still in their upper levels.
-template <bool ALONE>
-__global__ void __launch_bounds__(256, ALONE ? 1 : 4)
+template <int KIND>
+__global__ void __launch_bounds__(ps_tree_threads(KIND), ps_tree_ctas(KIND))
     k_ps_sweeps_tree(PSolveDev ps, DevParams P, const d4* __restrict__ b, d4* __restrict__ y, d4* __restrict__ out,
                      int mode, const int* __restrict__ contact, const d4* __restrict__ nb,
                      const double* __restrict__ cc, d4* __restrict__ f, int* __restrict__ case_,
                      double* __restrict__ c_out) {
     extern __shared__ double smd[];
-    ps_run<true, true, ALONE>(ps, P, b, y, out, mode, contact, nb, cc, f, case_, c_out, smd);
+    ps_run<true, true, KIND>(ps, P, b, y, out, mode, contact, nb, cc, f, case_, c_out, smd);
 }
 
 __global__ void k_finalize(int m, double h, const d4* __restrict__ x_n, const d4* __restrict__ v,
@@ -1163,24 +1173,27 @@ cudaError_t psolve_configure(int max_fs) {
     const size_t need = ps_level_smem(max_fs, 1);
     if (need <= configured) return cudaSuccess;
     cudaError_t e = cudaSuccess;
-    for (const void* k : {(const void*)k_ps_fwd, (const void*)k_ps_bwd, (const void*)k_ps_fwd_tree<false>,
-                          (const void*)k_ps_fwd_tree<true>, (const void*)k_ps_bwd_tree<false>,
-                          (const void*)k_ps_bwd_tree<true>, (const void*)k_ps_sweeps_tree<false>,
-                          (const void*)k_ps_sweeps_tree<true>})
+    for (const void* k :
+         {(const void*)k_ps_fwd, (const void*)k_ps_bwd, (const void*)k_ps_fwd_tree<PS_KIND_ALONE>,
+          (const void*)k_ps_fwd_tree<PS_KIND_GROUPS>, (const void*)k_ps_fwd_tree<PS_KIND_MANY>,
+          (const void*)k_ps_bwd_tree<PS_KIND_ALONE>, (const void*)k_ps_bwd_tree<PS_KIND_GROUPS>,
+          (const void*)k_ps_bwd_tree<PS_KIND_MANY>, (const void*)k_ps_sweeps_tree<PS_KIND_ALONE>,
+          (const void*)k_ps_sweeps_tree<PS_KIND_GROUPS>, (const void*)k_ps_sweeps_tree<PS_KIND_MANY>})
         if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
     if (e == cudaSuccess) configured = need;
     return e;
 }
 
-cudaError_t psolve_tree_grid(int max_fs, bool alone, int* grid, size_t* smem_out) {
-    const size_t smem = ps_level_smem(max_fs, 1);
+cudaError_t psolve_tree_grid(int max_fs, int kind, int* grid, size_t* smem_out) {
+    const int nt = ps_tree_threads(kind);
+    const size_t smem = std::max((6 * (size_t)max_fs + 3 * (size_t)ps_pass_rows(nt) * GV_MAXG) * sizeof(double),
+                                 (size_t)(nt / 32) * 6 * PS_LD * sizeof(double));
     *smem_out = smem;
     int dev = 0, sms = 0, n = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess)
-        e = alone ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_ps_sweeps_tree<true>, 256, smem)
-                  : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_ps_sweeps_tree<false>, 256, smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, PS_PICK(k_ps_sweeps_tree, kind), nt, smem);
     if (e != cudaSuccess) return e;
     *grid = sms * std::max(1, n);
     return cudaSuccess;
@@ -1188,8 +1201,8 @@ cudaError_t psolve_tree_grid(int max_fs, bool alone, int* grid, size_t* smem_out
 
 static void run_fwd_tree(const PSolveDev& ps, const d4* b, d4* y, cudaStream_t s) {
     const int grid = std::min(ps.tree_grid, ps.n_ftask);
-    auto k = ps.alone ? k_ps_fwd_tree<true> : k_ps_fwd_tree<false>;
-    k<<<grid, 256, ps.tree_smem, s>>>(ps, b, y);
+    auto k = PS_PICK(k_ps_fwd_tree, ps.kind);
+    k<<<grid, ps_tree_threads(ps.kind), ps.tree_smem, s>>>(ps, b, y);
 }
 
 void launch_solve_fwd(const DevMesh& dm, const d4* b, d4* y, cudaStream_t s) {
@@ -1237,8 +1250,8 @@ void launch_solve_bwd(const DevMesh& dm, const DevParams& P, const d4* y, d4* ou
             cudaMemsetAsync(ps.sched + 2 * (size_t)ps.S + 1, 0, sizeof(int) * (2 * (size_t)ps.S + 1), s);
             dc_note_launch();
             const int grid = std::min(ps.tree_grid, ps.n_btask);
-            auto k = ps.alone ? k_ps_bwd_tree<true> : k_ps_bwd_tree<false>;
-            k<<<grid, 256, ps.tree_smem, s>>>(ps, P, const_cast<d4*>(y), out, mode, contact, nb, c, f, case_, c_out);
+            auto k = PS_PICK(k_ps_bwd_tree, ps.kind);
+            k<<<grid, ps_tree_threads(ps.kind), ps.tree_smem, s>>>(ps, P, const_cast<d4*>(y), out, mode, contact, nb, c, f, case_, c_out);
             return;
         }
         for (int l = ps.nlev - 1; l >= 0; --l) {
@@ -1265,8 +1278,8 @@ bool launch_solve_sweeps(const DevMesh& dm, const DevParams& P, const d4* b, d4*
     cudaMemsetAsync(ps.sched, 0, sizeof(int) * 2 * (2 * (size_t)ps.S + 1), s);
     dc_note_launch();
     const int grid = std::min(ps.tree_grid, ps.n_ftask + ps.n_btask);
-    auto k = ps.alone ? k_ps_sweeps_tree<true> : k_ps_sweeps_tree<false>;
-    k<<<grid, 256, ps.tree_smem, s>>>(ps, P, b, y, out, mode, contact, nb, c, f, case_, c_out);
+    auto k = PS_PICK(k_ps_sweeps_tree, ps.kind);
+    k<<<grid, ps_tree_threads(ps.kind), ps.tree_smem, s>>>(ps, P, b, y, out, mode, contact, nb, c, f, case_, c_out);
     return true;
 }
 void launch_finalize(const DevMesh& dm, const DevParams& P, const d4* x_n, const d4* v, d4* x_np1,

@@ -50,3 +50,24 @@ def test_grouped_batch_is_bitwise_the_cloths_alone():
         cl.close()
     b.close()
     assert rel_inf(got[0].cpu().numpy(), _want(scs[0], rhs[0])) < 2e-11
+
+
+def test_many_small_fronts_are_bitwise_the_cloths_alone():
+    """Above 32 small fronts per SM: groups of four on CTAs of 128 threads."""
+    import torch
+    base = [scenes.batch_instance(s, n_steps=1) for s in range(12)]
+    scs = base * 12
+    rhs = [np.random.default_rng(s).standard_normal((sc.m, 3)) for s, sc in enumerate(base)]
+    b = make_batch(scs, global_solver=1)
+    got = b.split(b.global_solve(cuda(np.concatenate(rhs * 12))))
+    x = b.rollout(cuda(np.concatenate([sc.x0 for sc in scs])), cuda(np.concatenate([sc.v0 for sc in scs])), 1)[0]
+    x = b.split(x)
+    b.stats()
+    for i, sc in enumerate(base):
+        cl = make_cloth(sc, global_solver=1)
+        want = cl.global_solve(cuda(rhs[i]))
+        wx = cl.rollout(cuda(sc.x0), cuda(sc.v0), 1)[0]
+        cl.close()
+        for k in (0, 5, 11):
+            assert torch.equal(got[12 * k + i], want) and torch.equal(x[12 * k + i], wx)
+    b.close()
