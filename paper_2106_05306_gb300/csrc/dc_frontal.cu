@@ -164,14 +164,67 @@ constexpr int GV_ROWS = 128;
 constexpr int GV_MAXG = 8;
 __host__ __device__ constexpr int gv_groups(int K) { return K <= 8 ? 1 : (K + 7) / 8 < GV_MAXG ? (K + 7) / 8 : GV_MAXG; }
 
-template <bool TRI, bool PAD, class Fin>
+// PRE: the first GV_PRE entries of a thread's first two items come from its registers
+// (GemvPre, loaded before the vector was there); after() runs once the products of the first
+// pass are formed.
+constexpr int GV_PRE = 10;
+struct GemvPre {
+    float a[2][GV_PRE];
+    template <bool TRI, bool PAD>
+    __device__ __forceinline__ void load(const float* __restrict__ A, long lda, int r_lo, int r_hi, int K) {
+        const int G = gv_groups(K), C = (K + G - 1) / G;
+        const int R = min(GV_ROWS, r_hi - r_lo), Rp = PAD ? GV_ROWS : R;
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int item = threadIdx.x + j * blockDim.x, g = item / Rp, r = item - g * Rp, i = r_lo + r;
+            const int k0 = g * C;
+            int k1 = item < Rp * G && r < R ? min(K, k0 + C) : 0;
+            if (TRI) k1 = min(k1, i + 1);
+            const float* p = A + i + (long)k0 * lda;
+#pragma unroll
+            for (int q = 0; q < GV_PRE; ++q) {
+                a[j][q] = k0 + q < k1 ? *p : 0.0f;
+                p += lda;
+            }
+        }
+    }
+};
+struct GvNone {
+    __device__ __forceinline__ void operator()() const {}
+};
+
+template <bool TRI, bool PAD, bool PRE = false, class Fin, class After = GvNone>
 __device__ __forceinline__ void cm_gemv(const float* __restrict__ A, long lda, int r_lo, int r_hi, int K,
-                                        const float* __restrict__ v, float* __restrict__ red, Fin fin) {
+                                        const float* __restrict__ v, float* __restrict__ red, Fin fin,
+                                        const GemvPre* pre = nullptr, After after = After()) {
     const int nt = blockDim.x, tid = threadIdx.x;
     const int G = gv_groups(K), C = (K + G - 1) / G;
     for (int i0 = r_lo; i0 < r_hi; i0 += GV_ROWS) {
         const int R = min(GV_ROWS, r_hi - i0), Rp = PAD ? GV_ROWS : R;
-        for (int item = tid; item < Rp * G; item += nt) {
+        int first = tid;
+        if (PRE && i0 == r_lo) {
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int item = tid + j * nt, g = item / Rp, r = item - g * Rp, i = i0 + r;
+                if (item >= Rp * G) break;
+                float acc = 0.0f;
+                if (r < R) {
+                    const int k0 = g * C;
+                    int k1 = min(K, k0 + C);
+                    if (TRI) k1 = min(k1, i + 1);
+#pragma unroll
+                    for (int q = 0; q < GV_PRE; ++q)
+                        if (k0 + q < k1) acc += pre->a[j][q] * v[k0 + q];
+                    const float* a = A + i;
+#pragma unroll 8
+                    for (int k = k0 + GV_PRE; k < k1; ++k) acc += a[(long)k * lda] * v[k];
+                }
+                red[g * GV_ROWS + r] = acc;
+            }
+            after();
+            first = tid + 2 * nt;
+        }
+        for (int item = first; item < Rp * G; item += nt) {
             const int g = item / Rp, r = item - g * Rp, i = i0 + r;
             float acc = 0.0f;
             if (r < R) {
@@ -206,7 +259,28 @@ __device__ __forceinline__ float ms_pull(const FrontDev& fd, const int* __restri
     for (int e = pp[node]; e < pp[node + 1]; ++e) a += __ldcg(fd.acc + fd.pull_idx[e] + comp);
     return a;
 }
-template <class Wait>
+// The lookups of a position's pull list, and its value from them.
+struct MsPull {
+    int e0, e1, i0, i1;
+};
+__device__ __forceinline__ MsPull ms_pull_begin(const FrontDev& fd, const int* __restrict__ pp, int t) {
+    const int node = t / 3;
+    MsPull q{pp[node], pp[node + 1], 0, 0};
+    if (q.e0 < q.e1) q.i0 = fd.pull_idx[q.e0];
+    if (q.e0 + 1 < q.e1) q.i1 = fd.pull_idx[q.e0 + 1];
+    return q;
+}
+__device__ __forceinline__ float ms_pull_end(const FrontDev& fd, const MsPull& q, int t) {
+    const int comp = t % 3;
+    const float x = q.e0 < q.e1 ? __ldcg(fd.acc + q.i0 + comp) : 0.0f;
+    const float y = q.e0 + 1 < q.e1 ? __ldcg(fd.acc + q.i1 + comp) : 0.0f;
+    float a = 0.0f;
+    if (q.e0 < q.e1) a += x;
+    if (q.e0 + 1 < q.e1) a += y;
+    for (int e = q.e0 + 2; e < q.e1; ++e) a += __ldcg(fd.acc + fd.pull_idx[e] + comp);
+    return a;
+}
+template <bool FEW, class Wait>
 __device__ __forceinline__ bool ms_fwd_a(const FrontDev& fd, int s, int r_lo, int r_hi, float* __restrict__ w,
                                          Wait wait) {
     const int tid = threadIdx.x, nt = blockDim.x;
@@ -216,16 +290,28 @@ __device__ __forceinline__ bool ms_fwd_a(const FrontDev& fd, int s, int r_lo, in
     const int* pp = fd.pull_ptr + fd.pull_off[s];
     // the pivot of this thread's row of the first pass, ahead of the wait
     const float d0 = r_lo + tid < r_hi ? F[(long)(r_lo + tid) * f + r_lo + tid] : 1.0f;
+    const float* X = fd.linv + fd.linv_off[s];
+    GemvPre pre;
+    MsPull pull{0, 0, 0, 0};
+    float rv = 0.0f;
+    if (FEW) {
+        pre.load<true, false>(X, p, r_lo, r_hi, p);
+        if (tid < r_hi) {
+            pull = ms_pull_begin(fd, pp, tid);
+            rv = fd.rvec[base + tid];
+        }
+    }
     if (!wait()) return false;
-    for (int t = tid; t < r_hi; t += nt) w[t] = ms_pull(fd, pp, t) + fd.rvec[base + t];
+    if (FEW && tid < r_hi) w[tid] = ms_pull_end(fd, pull, tid) + rv;
+    for (int t = FEW ? tid + nt : tid; t < r_hi; t += nt) w[t] = ms_pull(fd, pp, t) + fd.rvec[base + t];
     __syncthreads();
-    cm_gemv<true, false>(fd.linv + fd.linv_off[s], p, r_lo, r_hi, p, w, red, [&](int i, float t) {
+    cm_gemv<true, false, FEW>(X, p, r_lo, r_hi, p, w, red, [&](int i, float t) {
         fd.yvec[base + i] = t;
         fd.zvec[base + i] = t / (i == r_lo + tid ? d0 : F[(long)i * f + i]);
-    });
+    }, &pre);
     return true;
 }
-template <class Wait>
+template <bool FEW, class Wait>
 __device__ __forceinline__ bool ms_fwd_b(const FrontDev& fd, int s, int r_lo, int r_hi, float* __restrict__ y,
                                          Wait wait) {
     const int tid = threadIdx.x, nt = blockDim.x;
@@ -234,12 +320,20 @@ __device__ __forceinline__ bool ms_fwd_b(const FrontDev& fd, int s, int r_lo, in
     float* red = w + nr;               // [GV_MAXG][GV_ROWS]
     const int* pp = fd.pull_ptr + fd.pull_off[s];
     float* acc = fd.acc + fd.acc_off[s];
+    const float* A = fd.pool + fd.off[s] + p;
+    GemvPre pre;
+    MsPull pull{0, 0, 0, 0};
+    if (FEW) {
+        pre.load<false, false>(A, f, r_lo, r_hi, p);
+        if (tid < nr) pull = ms_pull_begin(fd, pp, p + r_lo + tid);
+    }
     if (!wait()) return false;
     for (int t = tid; t < p; t += nt) y[t] = __ldcg(fd.yvec + base + t);
-    for (int t = tid; t < nr; t += nt) w[t] = ms_pull(fd, pp, p + r_lo + t);
+    if (FEW && tid < nr) w[tid] = ms_pull_end(fd, pull, p + r_lo + tid);
+    for (int t = FEW ? tid + nt : tid; t < nr; t += nt) w[t] = ms_pull(fd, pp, p + r_lo + t);
     __syncthreads();
-    cm_gemv<false, false>(fd.pool + fd.off[s] + p, f, r_lo, r_hi, p, y, red,
-                          [&](int i, float t) { acc[i] = w[i - r_lo] - t; });
+    cm_gemv<false, false, FEW>(A, f, r_lo, r_hi, p, y, red,
+                               [&](int i, float t) { acc[i] = w[i - r_lo] - t; }, &pre);
     return true;
 }
 
@@ -324,7 +418,7 @@ __device__ __forceinline__ bool ms_bwd_b(const FrontDev& fd, int s, int r_lo, in
 
 // The whole of front s on one CTA: both halves with the vectors kept in shared memory (the
 // same sums in the same order).
-template <class Wait>
+template <bool FEW, class Wait>
 __device__ __forceinline__ bool ms_fwd_whole(const FrontDev& fd, int s, float* __restrict__ w, Wait wait) {
     const int tid = threadIdx.x, nt = blockDim.x;
     const int f = fd.f[s], p = fd.p[s], base = 3 * fd.begin[s];
@@ -332,25 +426,48 @@ __device__ __forceinline__ bool ms_fwd_whole(const FrontDev& fd, int s, float* _
     float* y = w + f;
     float* red = y + p;                // [GV_MAXG][GV_ROWS]
     const int* pp = fd.pull_ptr + fd.pull_off[s];
+    const float* X = fd.linv + fd.linv_off[s];
+    GemvPre pre;
+    MsPull pull{0, 0, 0, 0};
+    float rv = 0.0f, d = 1.0f;
+    if (FEW) {
+        pre.load<true, true>(X, p, 0, p, p);
+        if (tid < f) pull = ms_pull_begin(fd, pp, tid);
+        if (tid < p) {
+            rv = fd.rvec[base + tid];
+            d = F[(long)tid * f + tid];
+        }
+    }
     if (!wait()) return false;
-    for (int t = tid; t < f; t += nt) w[t] = ms_pull(fd, pp, t) + (t < p ? fd.rvec[base + t] : 0.0f);
+    if (FEW && tid < f) w[tid] = ms_pull_end(fd, pull, tid) + rv;
+    for (int t = FEW ? tid + nt : tid; t < f; t += nt)
+        w[t] = ms_pull(fd, pp, t) + (t < p ? fd.rvec[base + t] : 0.0f);
     __syncthreads();
-    cm_gemv<true, true>(fd.linv + fd.linv_off[s], p, 0, p, p, w, red, [&](int i, float t) { y[i] = t; });
+    cm_gemv<true, true, FEW>(X, p, 0, p, p, w, red, [&](int i, float t) { y[i] = t; }, &pre,
+                             [&]() { pre.load<false, true>(F + p, f, 0, f - p, p); });
     float* acc = fd.acc + fd.acc_off[s];
-    cm_gemv<false, true>(F + p, f, 0, f - p, p, y, red, [&](int i, float t) { acc[i] = w[p + i] - t; });
-    for (int t = tid; t < p; t += nt) fd.zvec[base + t] = y[t] / F[(long)t * f + t];
+    cm_gemv<false, true, FEW>(F + p, f, 0, f - p, p, y, red, [&](int i, float t) { acc[i] = w[p + i] - t; }, &pre);
+    for (int t = tid; t < p; t += nt) fd.zvec[base + t] = y[t] / (FEW && t == tid ? d : F[(long)t * f + t]);
     return true;
 }
-template <class Wait>
+template <bool FEW, class Wait>
 __device__ __forceinline__ bool ms_bwd_whole(const FrontDev& fd, int s, float* __restrict__ w, Wait wait) {
     const int tid = threadIdx.x, nt = blockDim.x;
     const int f = fd.f[s], p = fd.p[s], nu = f - p, base = 3 * fd.begin[s];
     const float* F = fd.pool + fd.off[s];
     float* xu = w + p;
     const int* un = fd.unode + fd.uptr[s];
+    // zvec is the forward launch's
+    int src = 0;
+    if (FEW) {
+        if (tid < nu) src = un[tid / 3];
+        for (int t = tid; t < p; t += nt) w[t] = __ldcg(fd.zvec + base + t);
+    }
     if (!wait()) return false;
-    for (int t = tid; t < p; t += nt) w[t] = __ldcg(fd.zvec + base + t);
-    for (int k = tid; k < nu; k += nt) xu[k] = __ldcg(fd.xvec + 3 * un[k / 3] + k % 3);
+    if (!FEW)
+        for (int t = tid; t < p; t += nt) w[t] = __ldcg(fd.zvec + base + t);
+    if (FEW && tid < nu) xu[tid] = __ldcg(fd.xvec + 3 * src + tid % 3);
+    for (int k = FEW ? tid + nt : tid; k < nu; k += nt) xu[k] = __ldcg(fd.xvec + 3 * un[k / 3] + k % 3);
     __syncthreads();
     if (nu > 0) {
         rm_gemv<false>(F + p, f, 0, p, nu, xu, [&](int i, float t) { w[i] -= t; });
@@ -362,12 +479,12 @@ __device__ __forceinline__ bool ms_bwd_whole(const FrontDev& fd, int s, float* _
 }
 
 // A task of front s: rows of one half, or all of it (MS_AB).
-template <bool fwd, class Wait>
+template <bool fwd, bool FEW, class Wait>
 __device__ __forceinline__ bool ms_front(const FrontDev& fd, int s, int phase, int r_lo, int r_hi,
                                          float* __restrict__ sm, Wait wait) {
-    if (phase == MS_AB) return fwd ? ms_fwd_whole(fd, s, sm, wait) : ms_bwd_whole(fd, s, sm, wait);
+    if (phase == MS_AB) return fwd ? ms_fwd_whole<FEW>(fd, s, sm, wait) : ms_bwd_whole<FEW>(fd, s, sm, wait);
     if (fwd)
-        return phase == MS_A ? ms_fwd_a(fd, s, r_lo, r_hi, sm, wait) : ms_fwd_b(fd, s, r_lo, r_hi, sm, wait);
+        return phase == MS_A ? ms_fwd_a<FEW>(fd, s, r_lo, r_hi, sm, wait) : ms_fwd_b<FEW>(fd, s, r_lo, r_hi, sm, wait);
     return phase == MS_A ? ms_bwd_a(fd, s, r_lo, r_hi, sm, wait) : ms_bwd_b(fd, s, r_lo, r_hi, sm, wait);
 }
 
@@ -377,14 +494,14 @@ __global__ void __launch_bounds__(FT) k_msolve_fwd(FrontDev fd, const int* __res
     extern __shared__ float sm[];
     const int s = sn_list[blockIdx.x];
     if (mask && mask[fd.sn_inst[s]] == 0.0) return;
-    ms_front<true>(fd, s, MS_AB, 0, 0, sm, []() { return true; });
+    ms_front<true, false>(fd, s, MS_AB, 0, 0, sm, []() { return true; });
 }
 __global__ void __launch_bounds__(FT) k_msolve_bwd(FrontDev fd, const int* __restrict__ sn_list,
                                                     const double* __restrict__ mask) {
     extern __shared__ float sm[];
     const int s = sn_list[blockIdx.x];
     if (mask && mask[fd.sn_inst[s]] == 0.0) return;
-    ms_front<false>(fd, s, MS_AB, 0, 0, sm, []() { return true; });
+    ms_front<false, false>(fd, s, MS_AB, 0, 0, sm, []() { return true; });
 }
 
 // Tree-scheduled solves, one launch per sweep.  Persistent CTAs take tasks -- a front, or
@@ -401,10 +518,16 @@ __global__ void __launch_bounds__(FT) k_msolve_bwd(FrontDev fd, const int* __res
 // Threads per CTA and CTAs per SM: a front is a chain of latencies, so many CTAs share an SM
 // where there are many fronts (96 cloths, the gradient call: forward at 3 CTAs 53.3 ms,
 // at 4 51.2), and the fronts on the dependency chain are the large ones, so wide CTAs pay.
+// FEW (at most MS_FEW fronts, 24 per SM): the time is the chain of fronts, each of them a
+// chain of loads after its wait, so a thread loads its pull lists, right-hand side, pivots
+// and the first entries of its rows before the wait and the second product's during the
+// first.  That takes 64 registers, two CTAs an SM, which many fronts cannot spare.
+// Measured, without -> with (us, gradient calls): 256-node cloth 14400 -> 13500, 61 x 61 nodes
+// 21400 -> 20000, 200 x 200 nodes 49800 -> 47300; 96 cloths 47600 -> 49200.
 constexpr int MT = 512;
 
-template <bool FWD>
-__global__ void __launch_bounds__(MT, FWD ? 4 : 3) k_msolve_tree(FrontDev fd, const int* __restrict__ list, int n,
+template <bool FWD, bool FEW>
+__global__ void __launch_bounds__(MT, FEW ? 2 : FWD ? 4 : 3) k_msolve_tree(FrontDev fd, const int* __restrict__ list, int n,
                                                        const double* __restrict__ mask) {
     extern __shared__ float sm[];
     __shared__ int s_item, s_ok;
@@ -443,7 +566,7 @@ __global__ void __launch_bounds__(MT, FWD ? 4 : 3) k_msolve_tree(FrontDev fd, co
             __syncthreads();
             return s_ok != 0;
         };
-        if (!ms_front<FWD>(fd, s, phase, task.z, task.w, sm, wait)) return;
+        if (!ms_front<FWD, FEW>(fd, s, phase, task.z, task.w, sm, wait)) return;
         __syncthreads();
         if (threadIdx.x == 0) {
             const bool mid = phase == MS_A && fd.parent[s] >= 0;   // (a root's forward ends with half A)
@@ -505,8 +628,9 @@ cudaError_t frontal_configure(int max_f) {
     std::lock_guard<std::mutex> lock(mu);
     const size_t sb = frontal_solve_smem(max_f);
     if (sb > solve_bytes) {
-        for (const void* k : {(const void*)k_msolve_fwd, (const void*)k_msolve_bwd, (const void*)k_msolve_tree<true>,
-                              (const void*)k_msolve_tree<false>}) {
+        for (const void* k : {(const void*)k_msolve_fwd, (const void*)k_msolve_bwd, (const void*)k_msolve_tree<true, false>,
+                              (const void*)k_msolve_tree<false, false>, (const void*)k_msolve_tree<true, true>,
+                              (const void*)k_msolve_tree<false, true>}) {
             cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sb);
             if (e != cudaSuccess) return e;
         }
@@ -515,13 +639,14 @@ cudaError_t frontal_configure(int max_f) {
     return cudaSuccess;
 }
 
-cudaError_t frontal_tree_grid(int max_f, int* grid, size_t* smem_out) {
+cudaError_t frontal_tree_grid(int max_f, bool few, int* grid, size_t* smem_out) {
     const size_t smem = frontal_solve_smem(max_f);
     *smem_out = smem;
     int dev = 0, sms = 0, n = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_msolve_tree<true>, MT, smem);
+    if (e == cudaSuccess) e = few ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_msolve_tree<true, true>, MT, smem)
+                                 : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_msolve_tree<true, false>, MT, smem);
     if (e != cudaSuccess) return e;
     *grid = sms * (n > 0 ? n : 1);
     return cudaSuccess;
@@ -608,9 +733,9 @@ void frontal_precond(const AdjDev& ad, const FrontDev& fd, const int* lvl_ptr, i
             cudaMemsetAsync(fd.sched, 0, sizeof(int) * (4 * (size_t)fd.S + 2), s);
             if (kt) kt->begin(DC_KT_MSOLVE);
             dc_note_launch();
-            k_msolve_tree<true><<<std::min(nf, fd.tree_grid), MT, fd.tree_smem, s>>>(fd, act_f, nf, ad.mask);
+            (fd.few ? k_msolve_tree<true, true> : k_msolve_tree<true, false>)<<<std::min(nf, fd.tree_grid), MT, fd.tree_smem, s>>>(fd, act_f, nf, ad.mask);
             dc_note_launch();
-            k_msolve_tree<false><<<std::min(nb, fd.tree_grid), MT, fd.tree_smem, s>>>(fd, act_b, nb, ad.mask);
+            (fd.few ? k_msolve_tree<false, true> : k_msolve_tree<false, false>)<<<std::min(nb, fd.tree_grid), MT, fd.tree_smem, s>>>(fd, act_b, nb, ad.mask);
             if (kt) kt->end(DC_KT_MSOLVE);
         }
         dc_note_launch();

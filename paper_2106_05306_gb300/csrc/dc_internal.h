@@ -394,6 +394,7 @@ struct FrontDev {
     const int* pull_off;               // [S]
     const int* pull_ptr;
     const int* pull_idx;
+    int few;                           // host: at most MS_FEW fronts
     int n_ftask, n_btask;
     const int4* ftask;
     const int4* btask;

@@ -536,7 +536,8 @@ dc_status upload_params(dc_ctx* c, ParamPrep& pp) {
         fd.sched = d_sched;
         fd.fault = c->counters + 3;
         fd.tree = std::getenv("DC_LEVEL_SOLVES") ? 0 : 1;
-        CK(frontal_tree_grid(frm.max_f, &fd.tree_grid, &fd.tree_smem));
+        fd.few = frm.S <= MS_FEW;
+        CK(frontal_tree_grid(frm.max_f, fd.few != 0, &fd.tree_grid, &fd.tree_smem));
         // instance of every task, for the lists of the instances still iterating
         c->ms_finst_h.clear();
         c->ms_binst_h.clear();
