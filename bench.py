@@ -560,7 +560,7 @@ KERNEL_CLASSES = {
               "Signorini-Coulomb solve fused in)",
     "solve_fwd": "k_ps_fwd_tree (forward supernodal sweep, FP64, 3 columns)",
     "solve_bwd": "k_ps_bwd_tree (backward sweep + fused per-node Signorini-Coulomb solve)",
-    "front": "k_ff_* (one level of the FP32 multifrontal LDL^T of the adjoint preconditioner: extend, panels, updates, finish)",
+    "front": "k_ff_* (one level of the FP32 multifrontal LDL^T of the adjoint preconditioner: extend, panels, updates, inverse)",
     "msolve": "k_msolve_fwd_tree / k_msolve_bwd_tree (preconditioner solves)",
     "krylov": "k_bmdot / k_breduce / k_bvupdate / k_bscale (GMRES vectors)",
     "apply_h": "k_adj_elem + k_adj_gather (matrix-free adjoint operator)",
