@@ -306,23 +306,12 @@ void dc_merge_psolve(const std::vector<HostPSolve>& P, HostPSolve& out) {
 
 constexpr int SMS = 152;
 
-// From 32 small fronts per SM on, groups of four on eight 128-thread CTAs an SM: with
-// groups of eight 60% of the warps stood at their CTA's barriers (an item's warps wait for
-// its slowest, a large front's phases do not fill 256 threads).  One solve of 16, 32, 64, 96,
-// 160 cloths (23000 to 267000 nodes), groups of eight -> four: 238 -> 238, 295 -> 333, 451
-// -> 449, 526 -> 500, 676 -> 595 us; one 200 x 200 cloth, bound by its top fronts, 36.8 -> 40.1
-// ms a rollout.
-int ps_kind(int n_small) {
-    return n_small <= 8 * SMS ? PS_KIND_ALONE : n_small <= 32 * SMS ? PS_KIND_GROUPS : PS_KIND_MANY;
-}
-
 // Work items of the tree-scheduled sweeps, in a topological order (every front
 // after its children): fronts farther from their root come first, so the longest
 // remaining chains start earliest.  A front of more than DC_PS_SMALL nodes is an
-// item alone (one CTA); smaller fronts of equal depth go up to DC_PS_WARPS (half
-// of that in PS_KIND_MANY) to an item, one warp each, the larger ones first, since
-// an item's warps wait for its slowest (96 cloths: a rollout 63.6 -> 62.8 ms).  Item q is
-// tq_sn[tq_ptr[q] .. tq_ptr[q + 1]).
+// item alone; smaller fronts of equal depth follow, up to DC_PS_WARPS to an item, the
+// larger ones first, so that fronts solved together by one CTA are of similar cost (96
+// cloths: a rollout 63.6 -> 62.8 ms).  Item q is tq_sn[tq_ptr[q] .. tq_ptr[q + 1]).
 void dc_build_tree_items(const HostFronts& fr, std::vector<int>& tq_ptr, std::vector<int>& tq_sn) {
     std::vector<int> depth(fr.S, 0), order(fr.S);
     for (int s = 0; s < fr.S; ++s) {
@@ -335,9 +324,6 @@ void dc_build_tree_items(const HostFronts& fr, std::vector<int>& tq_ptr, std::ve
         if (large(a) != large(b)) return large(a);
         return !large(a) && (long)fr.f[a] * fr.p[a] > (long)fr.f[b] * fr.p[b];
     });
-    int n_small = 0;
-    for (int s = 0; s < fr.S; ++s) n_small += !large(s);
-    const int group = ps_kind(n_small) == PS_KIND_MANY ? DC_PS_WARPS / 2 : DC_PS_WARPS;
     tq_ptr.assign(1, 0);
     tq_sn.clear();
     for (size_t k = 0; k < order.size();) {
@@ -346,11 +332,22 @@ void dc_build_tree_items(const HostFronts& fr, std::vector<int>& tq_ptr, std::ve
             tq_sn.push_back(s);
             ++k;
         } else {
-            for (int n = 0; k < order.size() && n < group && !large(order[k]) && depth[order[k]] == depth[s]; ++n)
+            for (int n = 0; k < order.size() && n < DC_PS_WARPS && !large(order[k]) && depth[order[k]] == depth[s]; ++n)
                 tq_sn.push_back(order[k++]);
         }
         tq_ptr.push_back((int)tq_sn.size());
     }
+}
+
+// Kernel of the sweeps by the number of fronts.  Up to eight per SM, three CTAs of 256
+// threads an SM with 80 registers (one 45 x 45 cloth, two steps: 8.5 ms on the kernel before
+// tasks, 6.8 with 255 registers and one CTA an SM, 7.0 with 80, 7.2 with 64); then four with 64
+// (32 cloths of 40 x 40 nodes, three such batches on streams of their own: 9.4 ms with three
+// CTAs an SM, 7.3 with four); from 40 fronts per SM on, eight CTAs of 128 threads, whose
+// barriers hold fewer warps (one solve of 48 / 64 cloths of 40 x 40 nodes, four CTAs -> eight: 282
+// -> 300 / 298 -> 307 us, with three such batches 165 -> 122 / 234 -> 157).
+int ps_kind(int n_fronts) {
+    return n_fronts <= 8 * SMS ? PS_KIND_NARROW : n_fronts <= 40 * SMS ? PS_KIND_WIDE : PS_KIND_MANY;
 }
 
 // Tasks of the tree-scheduled supernodal sweeps, fronts farthest from their root
@@ -361,23 +358,28 @@ void dc_build_tree_items(const HostFronts& fr, std::vector<int>& tq_ptr, std::ve
 // each half is cut into row blocks of about that many: 32 tasks per SM and sweep,
 // within [1600, 8192] entries (1600 entries, 4800 FMAs over the three columns, take an
 // SM 1.4 us, about the cost of starting a task; 3200 measured 20% slower on one
-// 100 x 100 cloth).  Small fronts go one to a CTA while there are at most eight of
-// them per SM -- alone on a CTA a small front takes about 1 us of FP64 time instead of
-// 6 us on one of its eight warps -- and in groups of a warp each beyond that, where
-// every SM has other work (200 x 200 nodes, 12 per SM: 24.0 ms in groups, 30.5 alone).
+// 100 x 100 cloth).  The small fronts of a depth go to as few CTAs as their number asks for:
+// alone on a CTA's 256 threads a small front takes about 1 us instead of 6 us on one warp, but a
+// depth wider than the chip waits for CTAs, and other streams' launches for the SMs.  Up to 96
+// of them one to a CTA, to 192 two, to 1024 four, then a warp each (rollouts of 2 steps, all
+// alone -> by this rule -> a warp each, one context / three on streams of their own: 16 cloths of 16 x 16
+// nodes 3.3 / 2.7, 3.5 / 1.3, 5.0 / 1.7 ms; 12 cloths of 52 x 52 nodes 14.6 / 16.4, 10.4 / 5.6,
+// 11.2 / 6.4); on 128 threads, where a launch fills the chip anyway, up to 256 one and to 512 two
+// (one solve of 64 cloths of 40 x 40 nodes 340 -> 307 us).  `width` is the largest number of tasks
+// of one depth and phase.
 // No choice here changes a bit of the result.
 void dc_build_ps_tasks(const HostFronts& fr, const std::vector<int>& tq_ptr, const std::vector<int>& tq_sn,
-                       std::vector<int4>& ftask, std::vector<int4>& btask, std::vector<int4>& need, int& kind) {
+                       std::vector<int4>& ftask, std::vector<int4>& btask, std::vector<int4>& need, int& kind,
+                       int& width) {
     auto large = [&](int s) { return fr.f[s] / 3 > DC_PS_SMALL; };
     long long total = 0;
-    int n_small = 0;
     for (int s = 0; s < fr.S; ++s) {
         const long long ns = fr.p[s] / 3, nu = fr.f[s] / 3 - ns;
         total += ns * (ns + 1) / 2 + ns * nu;
-        n_small += !large(s);
     }
     const long long target = std::min<long long>(8192, std::max<long long>(1600, total / (SMS * 32)));
-    kind = ps_kind(n_small);
+    kind = ps_kind(fr.S);
+    width = 0;
     need.assign(fr.S, make_int4(1, 0, 1, 0));
     ftask.clear();
     btask.clear();
@@ -396,26 +398,28 @@ void dc_build_ps_tasks(const HostFronts& fr, const std::vector<int>& tq_ptr, con
     };
     std::vector<int> depth(fr.S, 0);
     for (int s = fr.S - 1; s >= 0; --s) depth[s] = fr.parent[s] >= 0 ? depth[fr.parent[s]] + 1 : 0;
-    const int n_items = (int)tq_ptr.size() - 1;
-    std::vector<std::pair<int, int>> span;   // items of one depth
-    for (int q = 0; q < n_items;) {
-        int e = q;
-        while (e < n_items && depth[tq_sn[tq_ptr[e]]] == depth[tq_sn[tq_ptr[q]]]) ++e;
-        span.push_back({q, e});
-        q = e;
+    // fronts of one depth: tq_sn[first .. small) large, tq_sn[small .. end) small
+    struct Span {
+        int first, small, end;
+    };
+    std::vector<Span> span;
+    for (int q = 0; q < fr.S;) {
+        Span sp{q, q, q};
+        while (sp.end < fr.S && depth[tq_sn[sp.end]] == depth[tq_sn[q]]) sp.small += large(tq_sn[sp.end++]);
+        span.push_back(sp);
+        q = sp.end;
     }
-    auto emit = [&](std::vector<int4>& out, const std::pair<int, int>& sp, bool fwd) {
-        for (int second = 0; second < 2; ++second)
-            for (int q = sp.first; q < sp.second; ++q) {
-                const int s = tq_sn[tq_ptr[q]];
+    const int threads = kind == PS_KIND_MANY ? 128 : 256;
+    auto emit = [&](std::vector<int4>& out, const Span& sp, bool fwd) {
+        const int n_small = sp.end - sp.small;
+        const int g = kind == PS_KIND_MANY ? (n_small <= 256 ? 1 : n_small <= 512 ? 2 : 4)
+                                           : (n_small <= 96 ? 1 : n_small <= 192 ? 2 : n_small <= 1024 ? 4 : 8);
+        for (int second = 0; second < 2; ++second) {
+            const size_t before = out.size();
+            for (int q = sp.first; q < sp.small; ++q) {
+                const int s = tq_sn[q];
                 const long long ns = fr.p[s] / 3, nu = fr.f[s] / 3 - ns;
-                if (!large(s)) {
-                    if (second) continue;
-                    if (kind == PS_KIND_ALONE)
-                        for (int e = tq_ptr[q]; e < tq_ptr[q + 1]; ++e) out.push_back(make_int4(tq_sn[e], PS_FRONT, 0, 0));
-                    else
-                        out.push_back(make_int4(tq_ptr[q], PS_GROUP, tq_ptr[q + 1] - tq_ptr[q], 0));
-                } else if (ns * (ns + 1) / 2 + ns * nu <= target) {
+                if (ns * (ns + 1) / 2 + ns * nu <= target) {
                     if (!second) out.push_back(make_int4(s, PS_AB, 0, 0));
                 } else if (fwd && !second) {
                     (nu > 0 ? need[s].y : need[s].x) =
@@ -428,6 +432,11 @@ void dc_build_ps_tasks(const HostFronts& fr, const std::vector<int>& tq_ptr, con
                     need[s].z = blocks(out, s, PS_B, (int)ns, [&](int i) { return ns - i; });
                 }
             }
+            for (int e = sp.small; !second && e < sp.end; e += g)
+                out.push_back(g == 1 ? make_int4(tq_sn[e], PS_FRONT, 0, 0)
+                                     : make_int4(e, PS_GROUP, std::min(g, sp.end - e), threads / g));
+            width = std::max(width, (int)(out.size() - before));
+        }
     };
     for (const auto& sp : span) emit(ftask, sp, true);
     for (size_t k = span.size(); k-- > 0;) emit(btask, span[k], false);

@@ -123,9 +123,9 @@ void dc_merge_psolve(const std::vector<HostPSolve>& P, HostPSolve& out);
 // Work items of the tree-scheduled sweeps, in topological order
 void dc_build_tree_items(const HostFronts& fr, std::vector<int>& tq_ptr, std::vector<int>& tq_sn);
 // Tasks of the tree-scheduled supernodal sweeps from those items (PSolveDev::ftask,
-// btask, need, kind)
+// btask, need, kind) and the most tasks of one depth and phase
 void dc_build_ps_tasks(const HostFronts& fr, const std::vector<int>& tq_ptr, const std::vector<int>& tq_sn,
-                       std::vector<int4>& ftask, std::vector<int4>& btask, std::vector<int4>& need, int& kind);
+                       std::vector<int4>& ftask, std::vector<int4>& btask, std::vector<int4>& need, int& kind, int& width);
 // Pull lists of the forward solves' child gather (see PSolveDev::pull_off and
 // FrontDev::pull_off): entry j of child c's update vector is aoff[c] + stride j
 void dc_build_pull_lists(const HostFronts& fr, const std::vector<int>& aoff, int stride, std::vector<int>& pull_off,
@@ -138,13 +138,12 @@ void dc_build_pull_lists(const HostFronts& fr, const std::vector<int>& aoff, int
 constexpr int DC_PS_SMALL = 64;
 // small fronts solved together by one CTA (one per warp)
 constexpr int DC_PS_WARPS = 8;
-// Kernel of the tree-scheduled sweeps: no groups, one CTA of 256 threads an SM and more
-// registers; groups of up to eight small fronts, 256 threads; groups of up to four, 128
-// threads and eight CTAs an SM.
-enum { PS_KIND_ALONE = 0, PS_KIND_GROUPS = 1, PS_KIND_MANY = 2 };
-int ps_kind(int n_small);
+// Kernel of the tree-scheduled sweeps: three CTAs of 256 threads an SM, four, or eight of
+// 128 threads.
+enum { PS_KIND_NARROW = 0, PS_KIND_WIDE = 1, PS_KIND_MANY = 2 };
+int ps_kind(int n_fronts);
 // A task (x, y, z, w) of the tree-scheduled sweeps: y says what it is, PS_GROUP the z
-// small fronts tq_sn[x ..), a warp each; PS_FRONT the small front x on a whole CTA;
+// small fronts tq_sn[x ..), w threads each; PS_FRONT the small front x on a whole CTA;
 // PS_AB the large front x; PS_A / PS_B rows [z, w) of its first / second half.
 enum { PS_A = 0, PS_B = 1, PS_AB = 2, PS_GROUP = 3, PS_FRONT = 4 };
 
@@ -196,7 +195,7 @@ struct PSolveDev {
     const int* pull_idx;
     int* sched;                        // [2][2 S + 1]: ticket counter, tasks done per front, half-A tasks done (fwd; bwd)
     unsigned long long* fault;         // sticky: set when a dependency wait gave up
-    int kind;                          // host: PS_KIND_*
+    int kind, width;                   // host: PS_KIND_*, most tasks of one depth and phase
     int tree_grid;                     // host: CTAs of a tree-scheduled launch
     size_t tree_smem;                  // host: its dynamic shared memory
     int fused;                         // host: 1: both sweeps of a global step as one launch
@@ -316,8 +315,8 @@ cudaError_t psolve_configure(int max_fs);
 // the launch (testing the bounded waits: those items never run).
 void launch_solve_fwd_skip(const DevMesh& dm, const d4* b, d4* y, int skip, cudaStream_t s);
 // Launch shape of the tree-scheduled sweeps whose largest CTA-path front has
-// max_fs nodes: the CTAs that fit on the device at once, and the dynamic shared memory
-cudaError_t psolve_tree_grid(int max_fs, int kind, int* grid, size_t* smem);
+// max_fs nodes and whose stages have at most `width` tasks: the CTAs, and the dynamic shared memory
+cudaError_t psolve_tree_grid(int max_fs, int kind, int width, int* grid, size_t* smem);
 // x_{n+1} = x_n + h v; sets *nonfinite when a state entry is not finite
 void launch_finalize(const DevMesh& dm, const DevParams& P, const d4* x_n, const d4* v,
                      d4* x_np1, unsigned long long* nonfinite, cudaStream_t s);

@@ -482,37 +482,27 @@ constexpr int PS_WARPS = DC_PS_WARPS;      // small fronts per CTA when they go 
 constexpr int PS_LD = PS_SMALL + 1;        // shared-memory column stride of a small front (no bank conflicts)
 constexpr int GV_ROWS = 128;               // rows of one pass
 constexpr int GV_MAXG = 8;
-constexpr int PS_CH = 16;                  // entries of an item loaded before a wait
 __host__ __device__ constexpr int gv_groups(int K) { return K <= 8 ? 1 : (K + 7) / 8 < GV_MAXG ? (K + 7) / 8 : GV_MAXG; }
 
 // The entries of the children's update vectors that add into position t of a front
-// (pull list pp, children in order), then b_t for a pivot (bt not null).  The list is
-// read before the CTA's dependency wait (ps_pull_begin), the vectors after it.  The sums
-// are those of a child-by-child scatter into zeroed storage, in the same order.
-struct PsPull {
-    int e0, e1, i0, i1;
-};
-__device__ __forceinline__ PsPull ps_pull_begin(const PSolveDev& ps, const int* __restrict__ pp, int t) {
-    PsPull q;
-    q.e0 = pp[t];
-    q.e1 = pp[t + 1];
-    q.i0 = q.e0 < q.e1 ? ps.pull_idx[q.e0] : 0;
-    q.i1 = q.e0 + 1 < q.e1 ? ps.pull_idx[q.e0 + 1] : 0;
-    return q;
-}
-__device__ __forceinline__ void ps_pull_end(const PSolveDev& ps, const PsPull& q, const d4* __restrict__ bt,
-                                            double* __restrict__ w, int stride) {
+// (pull list pp, children in order), then b_t for a pivot (bt not null): the three columns go
+// to w[0], w[stride], w[2 stride].  The sums are those of a child-by-child scatter into zeroed
+// storage, in the same order; the first two entries are loaded together.
+__device__ __forceinline__ void ps_pull(const PSolveDev& ps, const int* __restrict__ pp, int t,
+                                        const d4* __restrict__ bt, double* __restrict__ w, int stride) {
+    const int e0 = pp[t], e1 = pp[t + 1];
+    const int i0 = e0 < e1 ? ps.pull_idx[e0] : 0, i1 = e0 + 1 < e1 ? ps.pull_idx[e0 + 1] : 0;
     double x = 0.0, y = 0.0, z = 0.0;
     d4 b;
     if (bt) b = ld(bt);
-    if (q.e0 < q.e1) {
-        const d4 a = ld_cg(ps.acc + q.i0);
-        const bool two = q.e0 + 1 < q.e1;
+    if (e0 < e1) {
+        const d4 a = ld_cg(ps.acc + i0);
+        const bool two = e0 + 1 < e1;
         d4 c;
-        if (two) c = ld_cg(ps.acc + q.i1);
+        if (two) c = ld_cg(ps.acc + i1);
         x += a.x; y += a.y; z += a.z;
         if (two) { x += c.x; y += c.y; z += c.z; }
-        for (int e = q.e0 + 2; e < q.e1; ++e) {
+        for (int e = e0 + 2; e < e1; ++e) {
             const d4 d = ld_cg(ps.acc + ps.pull_idx[e]);
             x += d.x; y += d.y; z += d.z;
         }
@@ -528,269 +518,175 @@ __host__ __device__ constexpr int ps_pass_rows(int threads) { return threads > 1
 
 // Column-major product on one CTA with three right-hand sides: t_c,i = sum_k
 // A[k * lda + i] v[c * ldv + k] for rows r_lo <= i < r_hi and k < K (TRI 1: only
-// k <= i; TRI 2: only k >= i).  wait() blocks until the vectors are there and returns
-// false to give up; fill() then brings them to v.  Work items are (row, chunk) pairs,
-// the row fastest (coalesced loads), all three columns to a lane.  SPLIT: a lane for
-// each column too, for tasks too small to fill a CTA (a chunk is a serial chain of
-// FP64 FMAs, at least 64 cycles each, so a third of the chain per lane), and each
-// thread loads up to PS_CH entries of its first item before the wait.
-// fin(i, t0, t1, t2) stores.
-template <int TRI, bool SPLIT, class Wait, class Fill, class Fin>
-__device__ __forceinline__ bool ps_rows(const double* __restrict__ A, long lda, int r_lo, int r_hi, int K,
-                                        const double* __restrict__ v, int ldv, double* __restrict__ red, Wait wait,
-                                        Fill fill, Fin fin) {
+// k <= i; TRI 2: only k >= i).  Work items are the (row, chunk) pairs with a nonempty k range,
+// numbered chunk by chunk (the row fastest: coalesced loads), so that the empty half of a
+// triangle takes no lanes.  fin(i, t0, t1, t2) stores.
+template <int TRI, class Fin>
+__device__ __forceinline__ void ps_rows(const double* __restrict__ A, long lda, int r_lo, int r_hi, int K,
+                                        const double* __restrict__ v, int ldv, double* __restrict__ red, Fin fin) {
     const int nt = blockDim.x, tid = threadIdx.x;
     const int G = gv_groups(K), C = (K + G - 1) / G;
     const int ROWS = ps_pass_rows(nt);         // rows of a pass
     const int RS = ROWS * GV_MAXG;             // stride between the three columns' partial sums
-    auto range = [&](int i, int g, int& k0, int& k1) {
-        k0 = g * C;
-        k1 = min(K, k0 + C);
-        if (TRI == 1) k1 = min(k1, i + 1);
-        if (TRI == 2) k0 = max(k0, i);
-    };
-    // item -> (column, chunk, row)
-    auto decode = [&](int item, int R, int& c, int& g, int& r) {
-        const int q = item / R;
-        r = item - q * R;
-        g = SPLIT ? q % G : q;
-        c = SPLIT ? q / G : 0;
-    };
-    double a[SPLIT ? PS_CH : 1];
-    if (SPLIT) {
-        const int R = min(ROWS, r_hi - r_lo);
-        if (tid < 3 * R * G) {
-            int c, g, r, k0, k1;
-            decode(tid, R, c, g, r);
-            range(r_lo + r, g, k0, k1);
-            const double* col = A + (long)k0 * lda + r_lo + r;
-            const int n = k1 - k0;
-#pragma unroll
-            for (int q = 0; q < PS_CH; ++q) {
-                a[SPLIT ? q : 0] = q < n ? *col : 0.0;
-                col += lda;
-            }
-        }
-    }
-    if (!wait()) return false;
-    fill();
-    __syncthreads();
     for (int i0 = r_lo; i0 < r_hi; i0 += ROWS) {
         const int R = min(ROWS, r_hi - i0);
-        for (int item = tid; item < (SPLIT ? 3 : 1) * R * G; item += nt) {
-            int c, g, r, k0, k1;
-            decode(item, R, c, g, r);
-            range(i0 + r, g, k0, k1);
-            const double* col = A + (long)k0 * lda + i0 + r;
-            if (SPLIT) {
-                const double* vc = v + c * ldv + k0;
-                const int n = k1 - k0;
-                double s = 0.0;
-                int q0 = 0;
-                if (i0 == r_lo && item == tid) {
-#pragma unroll
-                    for (int q = 0; q < PS_CH; ++q) {
-                        if (q >= n) break;
-                        s += a[SPLIT ? q : 0] * vc[q];
-                    }
-                    q0 = PS_CH;
-                    col += (long)PS_CH * lda;
-                }
-#pragma unroll 8
-                for (int q = q0; q < n; ++q) {
-                    s += *col * vc[q];
-                    col += lda;
-                }
-                red[c * RS + g * ROWS + r] = s;
+        // rows [lo(g), hi(g)) of this pass have entries in chunk g
+        auto lo = [&](int g) { return TRI == 1 ? min(R, max(0, g * C - i0)) : 0; };
+        auto hi = [&](int g) { return TRI == 2 ? max(0, min(R, (g + 1) * C - i0)) : R; };
+        int n_items = R * G;
+        if (TRI != 0) {
+            n_items = 0;
+#pragma unroll 1
+            for (int g = 0; g < G; ++g) n_items += max(0, hi(g) - lo(g));
+        }
+        for (int item = tid; item < n_items; item += nt) {
+            int g = 0, r = item;
+            if (TRI == 0) {
+                g = item / R;
+                r = item - g * R;
             } else {
-                double a0 = 0.0, a1 = 0.0, a2 = 0.0;
-#pragma unroll 4
-                for (int k = k0; k < k1; ++k) {
-                    const double x = *col;
-                    col += lda;
-                    a0 += x * v[k];
-                    a1 += x * v[ldv + k];
-                    a2 += x * v[2 * ldv + k];
+#pragma unroll 1
+                for (;; ++g) {
+                    const int m = max(0, hi(g) - lo(g));
+                    if (r < m) break;
+                    r -= m;
                 }
-                red[g * ROWS + r] = a0;
-                red[RS + g * ROWS + r] = a1;
-                red[2 * RS + g * ROWS + r] = a2;
+                r += lo(g);
             }
+            int k0 = g * C, k1 = min(K, k0 + C);
+            if (TRI == 1) k1 = min(k1, i0 + r + 1);
+            if (TRI == 2) k0 = max(k0, i0 + r);
+            const double* col = A + (long)k0 * lda + i0 + r;
+            double a0 = 0.0, a1 = 0.0, a2 = 0.0;
+#pragma unroll 4
+            for (int k = k0; k < k1; ++k) {
+                const double x = *col;
+                col += lda;
+                a0 += x * v[k];
+                a1 += x * v[ldv + k];
+                a2 += x * v[2 * ldv + k];
+            }
+            red[g * ROWS + r] = a0;
+            red[RS + g * ROWS + r] = a1;
+            red[2 * RS + g * ROWS + r] = a2;
         }
         __syncthreads();
-        for (int e = tid; e < 3 * R; e += nt) {
-            const int c = e / R, r = e - c * R, i = i0 + r;
-            // the row's chunks with entries: [gl, gh)
-            const int gl = TRI == 2 ? i / C : 0, gh = TRI == 1 ? i / C + 1 : G;
-            double t = 0.0;
-            for (int g = gl; g < gh; ++g) t += red[c * RS + g * ROWS + r];
-            red[c * RS + r] = t;
+        if (tid < R) {                         // (ROWS <= nt) the row's chunks with entries, in order
+            const int i = i0 + tid, gl = TRI == 2 ? i / C : 0, gh = TRI == 1 ? i / C + 1 : G;
+            double t0 = 0.0, t1 = 0.0, t2 = 0.0;
+            for (int g = gl; g < gh; ++g) {
+                t0 += red[g * ROWS + tid];
+                t1 += red[RS + g * ROWS + tid];
+                t2 += red[2 * RS + g * ROWS + tid];
+            }
+            fin(i, t0, t1, t2);
         }
-        __syncthreads();
-        for (int r = tid; r < R; r += nt) fin(i0 + r, red[r], red[RS + r], red[2 * RS + r]);
         __syncthreads();
     }
-    return true;
+}
+// Nodes [lo, hi) of src, component-major with stride n, into dst (through L2: other CTAs of
+// the launch may have written them).
+__device__ __forceinline__ void ps_load(const d4* __restrict__ src, int lo, int hi, int n, double* __restrict__ dst) {
+    for (int t = lo + threadIdx.x; t < hi; t += blockDim.x) {
+        const d4 a = ld_cg(src + t);
+        dst[t] = a.x;
+        dst[n + t] = a.y;
+        dst[2 * n + t] = a.z;
+    }
+}
+__device__ __forceinline__ void ps_load_nodes(const d4* __restrict__ src, const int* __restrict__ node, int n,
+                                              double* __restrict__ dst) {
+    for (int t = threadIdx.x; t < n; t += blockDim.x) {
+        const d4 a = ld_cg(src + node[t]);
+        dst[t] = a.x;
+        dst[n + t] = a.y;
+        dst[2 * n + t] = a.z;
+    }
 }
 
-// Half A forward, rows [r_lo, r_hi).  With PRE the lookups of up to PS_PULL positions a
-// thread come before the wait.
-constexpr int PS_PULL = 2;
-template <bool PRE, class Wait>
-__device__ __forceinline__ bool ps_fwd_a(const PSolveDev& ps, int s, int r_lo, int r_hi, const d4* __restrict__ b,
-                                         d4* __restrict__ y, double* __restrict__ smd, Wait wait) {
-    const int tid = threadIdx.x, nt = blockDim.x;
-    const int begin = ps.begin[s], ns = ps.p[s] / 3;
-    double* w = smd;                       // [3][ns], positions below r_hi
-    double* red = w + 3 * ns;              // [3][GV_MAXG * GV_ROWS]
-    const int* pp = ps.pull_ptr + ps.pull_off[s];
-    constexpr int NP = PRE ? PS_PULL : 0;
-    PsPull pull[PS_PULL];
-#pragma unroll
-    for (int q = 0; q < NP; ++q)
-        if (tid + q * nt < r_hi) pull[q] = ps_pull_begin(ps, pp, tid + q * nt);
-    return ps_rows<1, PRE>(
-        ps.xinv + ps.xoff[s], ns, r_lo, r_hi, ns, w, ns, red, wait,
-        [&]() {
-#pragma unroll
-            for (int q = 0; q < NP; ++q) {
-                const int t = tid + q * nt;
-                if (t < r_hi) ps_pull_end(ps, pull[q], b + begin + t, w + t, ns);
-            }
-            for (int t = tid + NP * nt; t < r_hi; t += nt)
-                ps_pull_end(ps, ps_pull_begin(ps, pp, t), b + begin + t, w + t, ns);
-        },
-        [&](int i, double t0, double t1, double t2) { st(y + begin + i, t0, t1, t2); });
-}
-
-// Half B forward, rows [r_lo, r_hi) of the update vector.  y_s is read through L2 (other
-// CTAs of the launch may have written it).
-template <bool PRE, class Wait>
-__device__ __forceinline__ bool ps_fwd_b(const PSolveDev& ps, int s, int r_lo, int r_hi, const d4* __restrict__ y,
-                                         double* __restrict__ smd, Wait wait) {
-    const int tid = threadIdx.x, nt = blockDim.x;
-    const int begin = ps.begin[s], ns = ps.p[s] / 3, fs = ps.f[s] / 3, nr = r_hi - r_lo;
-    double* yv = smd;                      // [3][ns]
-    double* w = yv + 3 * ns;               // [3][nr]
-    double* red = w + 3 * nr;              // [3][GV_MAXG * GV_ROWS]
-    const int* pp = ps.pull_ptr + ps.pull_off[s] + ns + r_lo;
-    constexpr int NP = PRE ? 1 : 0;
-    PsPull pull{0, 0, 0, 0};
-    if (NP && tid < nr) pull = ps_pull_begin(ps, pp, tid);
-    d4* acc = ps.acc + ps.aoff[s];
-    return ps_rows<0, PRE>(
-        ps.panel + ps.poff[s] + ns, fs, r_lo, r_hi, ns, yv, ns, red, wait,
-        [&]() {
-            for (int t = tid; t < ns; t += nt) {
-                const d4 a = ld_cg(y + begin + t);
-                yv[t] = a.x;
-                yv[ns + t] = a.y;
-                yv[2 * ns + t] = a.z;
-            }
-            if (NP && tid < nr) ps_pull_end(ps, pull, nullptr, w + tid, nr);
-            for (int t = tid + NP * nt; t < nr; t += nt) ps_pull_end(ps, ps_pull_begin(ps, pp, t), nullptr, w + t, nr);
-        },
-        [&](int i, double t0, double t1, double t2) {
-            const double* q = w + i - r_lo;
-            st(acc + i, q[0] - t0, q[nr] - t1, q[2 * nr] - t2);
-        });
-}
-
-// Half A backward, rows [r_lo, r_hi) into ps.wbuf.
-template <bool PRE, class Wait>
-__device__ __forceinline__ bool ps_bwd_a(const PSolveDev& ps, int s, int r_lo, int r_hi, const d4* __restrict__ y,
-                                         double* __restrict__ smd, Wait wait) {
-    const int tid = threadIdx.x, nt = blockDim.x;
-    const int begin = ps.begin[s], ns = ps.p[s] / 3, nu = ps.f[s] / 3 - ns, nr = r_hi - r_lo;
-    double* xu = smd;                      // [3][nu]
-    double* w = xu + 3 * nu;               // [3][nr]
-    double* red = w + 3 * nr;              // [3][GV_MAXG * GV_ROWS]
-    const int* un = ps.unode + ps.uptr[s];
-    constexpr int NP = PRE ? PS_PULL : 0;
-    int src[PS_PULL];
-#pragma unroll
-    for (int q = 0; q < NP; ++q) src[q] = tid + q * nt < nu ? un[tid + q * nt] : 0;
-    auto put = [&](int k, int node) {
-        const d4 a = ld_cg(ps.xint + node);
-        xu[k] = a.x;
-        xu[nu + k] = a.y;
-        xu[2 * nu + k] = a.z;
-    };
-    return ps_rows<0, PRE>(
-        ps.pant + ps.toff[s], ns, r_lo, r_hi, nu, xu, nu, red, wait,
-        [&]() {
-            for (int t = tid; t < nr; t += nt) {
-                const d4 a = ld_cg(y + begin + r_lo + t);
-                w[t] = a.x;
-                w[nr + t] = a.y;
-                w[2 * nr + t] = a.z;
-            }
-#pragma unroll
-            for (int q = 0; q < NP; ++q)
-                if (tid + q * nt < nu) put(tid + q * nt, src[q]);
-            for (int k = tid + NP * nt; k < nu; k += nt) put(k, un[k]);
-        },
-        [&](int i, double t0, double t1, double t2) {
-            const double* q = w + i - r_lo;
-            st(ps.wbuf + begin + i, q[0] - t0, q[nr] - t1, q[2 * nr] - t2);
-        });
-}
-
-// Half B backward, rows [r_lo, r_hi), and the per-node output.  wsrc: where w_s is
-// (ps.wbuf, or y at a root, which has no half A).
-template <bool PRE, class Wait>
-__device__ __forceinline__ bool ps_bwd_b(const PSolveDev& ps, const DevParams& P, int s, int r_lo, int r_hi,
-                                         const d4* __restrict__ wsrc, d4* __restrict__ out, int mode,
-                                         const int* __restrict__ contact, const d4* __restrict__ nb,
-                                         const double* __restrict__ cc, d4* __restrict__ f, int* __restrict__ case_,
-                                         double* __restrict__ c_out, double* __restrict__ smd, Wait wait) {
-    const int tid = threadIdx.x, nt = blockDim.x;
-    const int begin = ps.begin[s], ns = ps.p[s] / 3;
-    double* w = smd;                       // [3][ns], positions from r_lo
-    double* red = w + 3 * ns;              // [3][GV_MAXG * GV_ROWS]
-    return ps_rows<2, PRE>(
-        ps.xinvt + ps.xoff[s], ns, r_lo, r_hi, ns, w, ns, red, wait,
-        [&]() {
-            for (int t = r_lo + tid; t < ns; t += nt) {
-                const d4 a = ld_cg(wsrc + begin + t);
-                w[t] = a.x;
-                w[ns + t] = a.y;
-                w[2 * ns + t] = a.z;
-            }
-        },
-        [&](int i, double t0, double t1, double t2) {
-            const int row = begin + i;
-            st(ps.xint + row, t0, t1, t2);
-            finish_row(P, row, t0, t1, t2, out, mode, contact, nb, cc, f, case_, c_out);
-        });
-}
-
-// A task of a large front: rows of one half, or all of it (PS_AB).
-template <bool PRE, class Wait>
+// A task of a large front: rows [r_lo, r_hi) of one half (PS_A, PS_B), or all of it (PS_AB),
+// with the vectors between the halves in shared memory; the same sums in the same order.
+// wait() blocks until the inputs are there and returns false to give up.
+template <class Wait>
 __device__ __forceinline__ bool ps_fwd_cta(const PSolveDev& ps, int s, int phase, int r_lo, int r_hi,
                                            const d4* __restrict__ b, d4* __restrict__ y, double* __restrict__ smd,
                                            Wait wait) {
-    const int ns = ps.p[s] / 3, nu = ps.f[s] / 3 - ns;
+    const int tid = threadIdx.x, nt = blockDim.x;
+    const int begin = ps.begin[s], ns = ps.p[s] / 3, fs = ps.f[s] / 3, nu = fs - ns;
+    const int* pp = ps.pull_ptr + ps.pull_off[s];
     const bool whole = phase == PS_AB;
-    if (phase != PS_B && !ps_fwd_a<PRE>(ps, s, whole ? 0 : r_lo, whole ? ns : r_hi, b, y, smd, wait)) return false;
-    if (phase == PS_A) return true;
-    return ps_fwd_b<PRE>(ps, s, whole ? 0 : r_lo, whole ? nu : r_hi, y, smd, [&]() { return whole || wait(); });
+    if (!wait()) return false;
+    double* yv = smd;                          // [3][ns]
+    double* w = yv + 3 * ns;                   // [3][nw] gathered right-hand side, positions from w0
+    if (phase == PS_B) {
+        const int nr = r_hi - r_lo;
+        ps_load(y + begin, 0, ns, ns, yv);
+        for (int t = tid; t < nr; t += nt) ps_pull(ps, pp + ns + r_lo, t, nullptr, w + t, nr);
+        __syncthreads();
+    } else {
+        const int n = whole ? fs : r_hi;
+        for (int t = tid; t < n; t += nt) ps_pull(ps, pp, t, t < ns ? b + begin + t : nullptr, w + t, n);
+        __syncthreads();
+        ps_rows<1>(ps.xinv + ps.xoff[s], ns, whole ? 0 : r_lo, whole ? ns : r_hi, ns, w, n, w + 3 * n,
+                   [&](int i, double t0, double t1, double t2) {
+                       yv[i] = t0;
+                       yv[ns + i] = t1;
+                       yv[2 * ns + i] = t2;
+                       st(y + begin + i, t0, t1, t2);
+                   });
+        if (!whole) return true;
+    }
+    // update vector: w_U - L_Us y_s
+    const int r0 = whole ? 0 : r_lo, r1 = whole ? nu : r_hi, ldw = whole ? fs : r_hi - r_lo;
+    const double* wu = whole ? w + ns : w - r_lo;
+    d4* acc = ps.acc + ps.aoff[s];
+    ps_rows<0>(ps.panel + ps.poff[s] + ns, fs, r0, r1, ns, yv, ns, w + 3 * ldw,
+               [&](int i, double t0, double t1, double t2) {
+                   const double* q = wu + i;
+                   st(acc + i, q[0] - t0, q[ldw] - t1, q[2 * ldw] - t2);
+               });
+    return true;
 }
-template <bool PRE, class Wait>
+
+// Backward; half A leaves w_s in ps.wbuf (a root has no half A, and reads y).
+template <class Wait>
 __device__ __forceinline__ bool ps_bwd_cta(const PSolveDev& ps, const DevParams& P, int s, int phase, int r_lo,
                                            int r_hi, const d4* __restrict__ y, d4* __restrict__ out, int mode,
                                            const int* __restrict__ contact, const d4* __restrict__ nb,
                                            const double* __restrict__ cc, d4* __restrict__ f, int* __restrict__ case_,
                                            double* __restrict__ c_out, double* __restrict__ smd, Wait wait) {
-    const int ns = ps.p[s] / 3, nu = ps.f[s] / 3 - ns;
-    const bool whole = phase == PS_AB, a = phase == PS_A || (whole && nu > 0);
-    if (a && !ps_bwd_a<PRE>(ps, s, whole ? 0 : r_lo, whole ? ns : r_hi, y, smd, wait)) return false;
+    const int begin = ps.begin[s], ns = ps.p[s] / 3, nu = ps.f[s] / 3 - ns;
+    const bool whole = phase == PS_AB;
+    if (!wait()) return false;
+    double* w = smd;                           // [3][ns]
+    double* xu = w + 3 * ns;                   // [3][nu]
+    double* red = xu + 3 * nu;                 // [3][GV_MAXG * GV_ROWS]
+    ps_load((phase == PS_B && nu > 0 ? ps.wbuf : y) + begin, whole ? 0 : r_lo, phase == PS_A ? r_hi : ns, ns, w);
+    if (phase != PS_B) ps_load_nodes(ps.xint, ps.unode + ps.uptr[s], nu, xu);
+    __syncthreads();
+    if (phase != PS_B && nu > 0)
+        ps_rows<0>(ps.pant + ps.toff[s], ns, whole ? 0 : r_lo, whole ? ns : r_hi, nu, xu, nu, red,
+                   [&](int i, double t0, double t1, double t2) {
+                       const double w0 = w[i] - t0, w1 = w[ns + i] - t1, w2 = w[2 * ns + i] - t2;
+                       if (!whole) {
+                           st(ps.wbuf + begin + i, w0, w1, w2);
+                           return;
+                       }
+                       w[i] = w0;
+                       w[ns + i] = w1;
+                       w[2 * ns + i] = w2;
+                   });
     if (phase == PS_A) return true;
-    return ps_bwd_b<PRE>(ps, P, s, whole ? 0 : r_lo, whole ? ns : r_hi, nu > 0 ? ps.wbuf : y, out, mode, contact, nb,
-                         cc, f, case_, c_out, smd, [&]() { return a || wait(); });
+    ps_rows<2>(ps.xinvt + ps.xoff[s], ns, whole ? 0 : r_lo, whole ? ns : r_hi, ns, w, ns, red,
+               [&](int i, double t0, double t1, double t2) {
+                   const int row = begin + i;
+                   st(ps.xint + row, t0, t1, t2);
+                   finish_row(P, row, t0, t1, t2, out, mode, contact, nb, cc, f, case_, c_out);
+               });
+    return true;
 }
 
-// Small fronts, on the nt lanes of a warp or of a CTA (sync: their barrier): one lane
+// Small fronts, on nt lanes (sync: their barrier): one lane
 // per (row, column) pair, so that a front of ns or nu rows keeps 3 ns or 3 nu lanes
 // busy; a pair's sum runs over k in ascending order.  w: [6][PS_LD].
 template <class Sync>
@@ -801,7 +697,7 @@ __device__ __forceinline__ void ps_fwd_small(const PSolveDev& ps, int s, const d
     double* yv = w + 3 * L;
     const int* pp = ps.pull_ptr + ps.pull_off[s];
     for (int t = lane; t < fs; t += nt)
-        ps_pull_end(ps, ps_pull_begin(ps, pp, t), t < ns ? b + begin + t : nullptr, w + t, L);
+        ps_pull(ps, pp, t, t < ns ? b + begin + t : nullptr, w + t, L);
     sync();
     // y_s = L_ss^-1 w_s (lower triangle)
     const double* X = ps.xinv + ps.xoff[s];
@@ -884,7 +780,7 @@ __global__ void __launch_bounds__(256) k_ps_fwd(PSolveDev ps, const int* __restr
     extern __shared__ double smd[];
     if ((int)blockIdx.x < n_big) {
         const int s = big[blockIdx.x];
-        ps_fwd_cta<false>(ps, s, PS_AB, 0, 0, b, y, smd, []() { return true; });
+        ps_fwd_cta(ps, s, PS_AB, 0, 0, b, y, smd, []() { return true; });
         return;
     }
     const int warp = threadIdx.x >> 5;
@@ -902,7 +798,7 @@ __global__ void __launch_bounds__(256) k_ps_bwd(PSolveDev ps, DevParams P, const
     extern __shared__ double smd[];
     if ((int)blockIdx.x < n_big) {
         const int s = big[blockIdx.x];
-        ps_bwd_cta<false>(ps, P, s, PS_AB, 0, 0, y, out, mode, contact, nb, cc, f, case_, c_out, smd,
+        ps_bwd_cta(ps, P, s, PS_AB, 0, 0, y, out, mode, contact, nb, cc, f, case_, c_out, smd,
                    []() { return true; });
         return;
     }
@@ -915,7 +811,7 @@ __global__ void __launch_bounds__(256) k_ps_bwd(PSolveDev ps, DevParams P, const
 
 // ---- tree-scheduled sweeps: one launch for both sweeps of a global step (or one
 // for each).  CTAs take tasks from a ticket counter in a topological order: a
-// group of small fronts (a warp each), one front as a whole, or some rows of one
+// group of small fronts (32 to 128 threads each), one front as a whole, or some rows of one
 // half of a large front.  Before a task a CTA waits until what it reads is complete:
 //   forward, whole or half A   every child's forward tasks
 //   backward, whole or half A  the parent's backward tasks (the parent's own wait
@@ -930,8 +826,8 @@ __global__ void __launch_bounds__(256) k_ps_bwd(PSolveDev ps, DevParams P, const
 // Every wait is bounded (dc_wait.cuh): one that gives up sets the sticky fault word,
 // and every CTA stops taking tasks once the word is set.
 //
-// Why large fronts are split by rows: an SM does one FP64 warp instruction in 19
-// cycles (measured; 64 for a warp alone), so the top fronts of one large cloth (400
+// Why large fronts are split by rows: an SM does one FP64 warp instruction in 16
+// cycles at its measured peak (a warp alone one in 64), so the top fronts of one large cloth (400
 // pivots, an 80,000-entry triangle at 200 x 200 nodes) kept one CTA busy for tens of
 // microseconds each while the rest of the chip waited for them.
 
@@ -961,26 +857,22 @@ __device__ __forceinline__ int* ps_counter(const PSolveDev& ps, bool fwd, int s,
 }
 
 constexpr int ps_tree_threads(int kind) { return kind == PS_KIND_MANY ? 128 : 256; }
-constexpr int ps_tree_ctas(int kind) { return kind == PS_KIND_ALONE ? 1 : kind == PS_KIND_GROUPS ? 4 : 8; }
+constexpr int ps_tree_ctas(int kind) { return kind == PS_KIND_NARROW ? 3 : kind == PS_KIND_WIDE ? 4 : 8; }
 // kernel instance of a kind
-#define PS_PICK(k, kind) ((kind) == PS_KIND_ALONE ? k<PS_KIND_ALONE> : (kind) == PS_KIND_GROUPS ? k<PS_KIND_GROUPS> : k<PS_KIND_MANY>)
+#define PS_PICK(k, kind) ((kind) == PS_KIND_NARROW ? k<PS_KIND_NARROW> : (kind) == PS_KIND_WIDE ? k<PS_KIND_WIDE> : k<PS_KIND_MANY>)
 
 // FWD / BWD: which sweeps this launch runs (both: the backward tasks follow the
-// forward ones in ticket order).  KIND (ps_kind): a context without groups of small fronts
-// has fewer tasks than the chip has room for, its time is the chain of waits, and the
-// kernel loads what it can before them.  The other kernels keep four CTAs of 256 or eight
-// of 128 threads on an SM instead, whose work hides one another's waits.
-template <bool FWD, bool BWD, int KIND>
+// forward ones in ticket order).
+template <bool FWD, bool BWD>
 __device__ __forceinline__ void ps_run(const PSolveDev& ps, const DevParams& P, const d4* __restrict__ b,
                                        d4* __restrict__ y, d4* __restrict__ out, int mode,
                                        const int* __restrict__ contact, const d4* __restrict__ nb,
                                        const double* __restrict__ cc, d4* __restrict__ f, int* __restrict__ case_,
                                        double* __restrict__ c_out, double* __restrict__ smd) {
-    constexpr bool ALONE = KIND == PS_KIND_ALONE;
-    __shared__ int s_item, s_ok;
+    __shared__ int s_item, s_ok, s_grp[PS_WARPS];
     int* ticket = FWD ? ps.sched : ps.sched + 2 * ps.S + 1;
     const int nf = FWD ? ps.n_ftask : 0, n = nf + (BWD ? ps.n_btask : 0);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x;
     for (;;) {
         if (tid == 0) s_item = dc_fault_set(ps.fault) ? n : atomicAdd(ticket, 1);
         __syncthreads();
@@ -988,41 +880,47 @@ __device__ __forceinline__ void ps_run(const PSolveDev& ps, const DevParams& P, 
         if (t >= n) return;
         const bool fwd = FWD && (!BWD || t < nf);
         const int4 task = fwd ? ps.ftask[t] : ps.btask[t - nf];
-        if (ALONE || task.y != PS_GROUP) {
+        if (task.y != PS_GROUP) {
             const int s = task.x;
             auto wait = [&]() {
                 if (tid == 0) s_ok = ps_wait(ps, fwd, FWD, s, task.y);
                 __syncthreads();
                 return s_ok != 0;
             };
-            if (ALONE && task.y == PS_FRONT) {
+            if (task.y == PS_FRONT) {
                 if (!wait()) return;
                 auto sync = []() { __syncthreads(); };
                 if (fwd) ps_fwd_small(ps, s, b, y, smd, tid, blockDim.x, sync);
                 else ps_bwd_small(ps, P, s, y, out, mode, contact, nb, cc, f, case_, c_out, smd, tid, blockDim.x, sync);
             } else if (fwd) {
-                if (!ps_fwd_cta<ALONE>(ps, s, task.y, task.z, task.w, b, y, smd, wait)) return;
+                if (!ps_fwd_cta(ps, s, task.y, task.z, task.w, b, y, smd, wait)) return;
             } else {
-                if (!ps_bwd_cta<ALONE>(ps, P, s, task.y, task.z, task.w, y, out, mode, contact, nb, cc, f, case_, c_out,
-                                       smd, wait))
+                if (!ps_bwd_cta(ps, P, s, task.y, task.z, task.w, y, out, mode, contact, nb, cc, f, case_, c_out, smd,
+                                wait))
                     return;
             }
             __syncthreads();
             if (tid == 0) dc_add_release(ps_counter(ps, fwd, s, task.y), 1);
         } else {
-            if (warp < task.z) {
-                const int s = ps.tq_sn[task.x + warp];
-                int ok = 1;
-                if (lane == 0) ok = ps_wait(ps, fwd, FWD, s, PS_AB);
-                ok = __shfl_sync(0xffffffffu, ok, 0);
-                __syncwarp();              // lane 0's acquire orders every lane's reads
-                if (ok) {
-                    auto sync = []() { __syncwarp(); };
-                    double* w = smd + warp * 6 * PS_LD;
-                    if (fwd) ps_fwd_small(ps, s, b, y, w, lane, 32, sync);
-                    else ps_bwd_small(ps, P, s, y, out, mode, contact, nb, cc, f, case_, c_out, w, lane, 32, sync);
-                    __syncwarp();
-                    if (lane == 0) dc_add_release(ps_counter(ps, fwd, s, PS_AB), 1);
+            const int nt = task.w, sub = tid / nt, ln = tid - sub * nt;   // (whole warps)
+            if (sub < task.z) {
+                const int s = ps.tq_sn[task.x + sub];
+                // barrier of a front's threads: nt >= 64 leaves at most four fronts to the CTA
+                auto sync = [&]() {
+                    if (nt == 32) __syncwarp();
+                    else if (sub == 0) asm volatile("bar.sync 1, %0;" ::"r"(nt) : "memory");
+                    else if (sub == 1) asm volatile("bar.sync 2, %0;" ::"r"(nt) : "memory");
+                    else if (sub == 2) asm volatile("bar.sync 3, %0;" ::"r"(nt) : "memory");
+                    else asm volatile("bar.sync 4, %0;" ::"r"(nt) : "memory");
+                };
+                if (ln == 0) s_grp[sub] = ps_wait(ps, fwd, FWD, s, PS_AB);
+                sync();                    // the leader's acquire orders every lane's reads
+                if (s_grp[sub]) {
+                    double* w = smd + sub * 6 * PS_LD;
+                    if (fwd) ps_fwd_small(ps, s, b, y, w, ln, nt, sync);
+                    else ps_bwd_small(ps, P, s, y, out, mode, contact, nb, cc, f, case_, c_out, w, ln, nt, sync);
+                    sync();
+                    if (ln == 0) dc_add_release(ps_counter(ps, fwd, s, PS_AB), 1);
                 }
             }
             __syncthreads();   // every warp has read s_item before it is rewritten
@@ -1035,7 +933,7 @@ __global__ void __launch_bounds__(ps_tree_threads(KIND), ps_tree_ctas(KIND)) k_p
                                                                     d4* __restrict__ y) {
     extern __shared__ double smd[];
     const DevParams none{};
-    ps_run<true, false, KIND>(ps, none, b, y, nullptr, 0, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, smd);
+    ps_run<true, false>(ps, none, b, y, nullptr, 0, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, smd);
 }
 
 template <int KIND>
@@ -1044,7 +942,7 @@ __global__ void __launch_bounds__(ps_tree_threads(KIND), ps_tree_ctas(KIND))
                   const int* __restrict__ contact, const d4* __restrict__ nb, const double* __restrict__ cc,
                   d4* __restrict__ f, int* __restrict__ case_, double* __restrict__ c_out) {
     extern __shared__ double smd[];
-    ps_run<false, true, KIND>(ps, P, nullptr, y, out, mode, contact, nb, cc, f, case_, c_out, smd);
+    ps_run<false, true>(ps, P, nullptr, y, out, mode, contact, nb, cc, f, case_, c_out, smd);
 }
 
 // Both sweeps of one global step as one launch: the backward work of small trees
@@ -1056,7 +954,7 @@ __global__ void __launch_bounds__(ps_tree_threads(KIND), ps_tree_ctas(KIND))
                      const double* __restrict__ cc, d4* __restrict__ f, int* __restrict__ case_,
                      double* __restrict__ c_out) {
     extern __shared__ double smd[];
-    ps_run<true, true, KIND>(ps, P, b, y, out, mode, contact, nb, cc, f, case_, c_out, smd);
+    ps_run<true, true>(ps, P, b, y, out, mode, contact, nb, cc, f, case_, c_out, smd);
 }
 
 __global__ void k_finalize(int m, double h, const d4* __restrict__ x_n, const d4* __restrict__ v,
@@ -1174,17 +1072,23 @@ cudaError_t psolve_configure(int max_fs) {
     if (need <= configured) return cudaSuccess;
     cudaError_t e = cudaSuccess;
     for (const void* k :
-         {(const void*)k_ps_fwd, (const void*)k_ps_bwd, (const void*)k_ps_fwd_tree<PS_KIND_ALONE>,
-          (const void*)k_ps_fwd_tree<PS_KIND_GROUPS>, (const void*)k_ps_fwd_tree<PS_KIND_MANY>,
-          (const void*)k_ps_bwd_tree<PS_KIND_ALONE>, (const void*)k_ps_bwd_tree<PS_KIND_GROUPS>,
-          (const void*)k_ps_bwd_tree<PS_KIND_MANY>, (const void*)k_ps_sweeps_tree<PS_KIND_ALONE>,
-          (const void*)k_ps_sweeps_tree<PS_KIND_GROUPS>, (const void*)k_ps_sweeps_tree<PS_KIND_MANY>})
+         {(const void*)k_ps_fwd, (const void*)k_ps_bwd, (const void*)k_ps_fwd_tree<PS_KIND_NARROW>,
+          (const void*)k_ps_fwd_tree<PS_KIND_WIDE>, (const void*)k_ps_fwd_tree<PS_KIND_MANY>,
+          (const void*)k_ps_bwd_tree<PS_KIND_NARROW>, (const void*)k_ps_bwd_tree<PS_KIND_WIDE>,
+          (const void*)k_ps_bwd_tree<PS_KIND_MANY>, (const void*)k_ps_sweeps_tree<PS_KIND_NARROW>,
+          (const void*)k_ps_sweeps_tree<PS_KIND_WIDE>, (const void*)k_ps_sweeps_tree<PS_KIND_MANY>})
         if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
     if (e == cudaSuccess) configured = need;
     return e;
 }
 
-cudaError_t psolve_tree_grid(int max_fs, int kind, int* grid, size_t* smem_out) {
+// CTAs of a launch: as many as the widest stage of the tree has tasks for (`width`), beyond 128
+// three quarters of that, and of the places on the chip where there are more.  A CTA without a
+// ready task polls and keeps its part of an SM from other streams' kernels.  Measured against
+// every CTA that fits: three 45 x 45 cloths on streams of their own (a stage has at most 48
+// fronts), two steps 5.28 -> 2.44 ms each, one of them alone 6.8 -> 7.0; three batches of 64 cloths
+// of 40 x 40 nodes 13.7 -> 9.8, one of them 15.3 -> 15.5.
+cudaError_t psolve_tree_grid(int max_fs, int kind, int width, int* grid, size_t* smem_out) {
     const int nt = ps_tree_threads(kind);
     const size_t smem = std::max((6 * (size_t)max_fs + 3 * (size_t)ps_pass_rows(nt) * GV_MAXG) * sizeof(double),
                                  (size_t)(nt / 32) * 6 * PS_LD * sizeof(double));
@@ -1195,7 +1099,8 @@ cudaError_t psolve_tree_grid(int max_fs, int kind, int* grid, size_t* smem_out) 
     if (e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, PS_PICK(k_ps_sweeps_tree, kind), nt, smem);
     if (e != cudaSuccess) return e;
-    *grid = sms * std::max(1, n);
+    const int fit = sms * std::max(1, n), wide = kind == PS_KIND_NARROW ? fit : fit / 4 * 3;
+    *grid = std::max(1, std::min(wide, width <= 128 ? width : std::max(128, width / 4 * 3)));
     return cudaSuccess;
 }
 

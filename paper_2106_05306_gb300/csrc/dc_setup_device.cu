@@ -603,8 +603,8 @@ dc_status upload_params(dc_ctx* c, ParamPrep& pp) {
         std::vector<int> pull_off, pull_ptr, pull_idx;
         dc_build_pull_lists(frm, pp.ps.aoff, 1, pull_off, pull_ptr, pull_idx);
         std::vector<int4> ftask, btask, need;
-        int kind = 0;
-        dc_build_ps_tasks(frm, tq_ptr, tq_sn, ftask, btask, need, kind);
+        int kind = 0, width = 0;
+        dc_build_ps_tasks(frm, tq_ptr, tq_sn, ftask, btask, need, kind, width);
         int *d_tq_sn, *d_sched, *d_pull_off, *d_pull_ptr, *d_pull_idx;
         int4 *d_ftask, *d_btask, *d_need;
         d4* d_wbuf;
@@ -623,6 +623,7 @@ dc_status upload_params(dc_ctx* c, ParamPrep& pp) {
         ps.need = d_need;
         ps.wbuf = d_wbuf;
         ps.kind = kind;
+        ps.width = width;
         ps.parent = fd.parent;
         ps.tq_sn = d_tq_sn;
         ps.sched = d_sched;
@@ -683,7 +684,7 @@ dc_status upload_params(dc_ctx* c, ParamPrep& pp) {
         int mx = 0;
         for (int v : c->ps_maxbig) mx = std::max(mx, v);
         CK(psolve_configure(mx));
-        CK(psolve_tree_grid(mx, dm.ps.kind, &dm.ps.tree_grid, &dm.ps.tree_smem));
+        CK(psolve_tree_grid(mx, dm.ps.kind, dm.ps.width, &dm.ps.tree_grid, &dm.ps.tree_smem));
     }
     {
         // per level, where each instance's fronts start in lvl_sn (an instance's
@@ -789,9 +790,9 @@ size_t estimate_device_bytes(const dc_ctx* c, const MeshPrep& mp, const ParamPre
         {
             std::vector<int> tq_ptr, tq_sn;
             std::vector<int4> ftask, btask, need;
-            int kind = 0;
+            int kind = 0, width = 0;
             dc_build_tree_items(r, tq_ptr, tq_sn);
-            dc_build_ps_tasks(r, tq_ptr, tq_sn, ftask, btask, need, kind);
+            dc_build_ps_tasks(r, tq_ptr, tq_sn, ftask, btask, need, kind, width);
             add(vbytes(ftask)); add(vbytes(btask)); add(vbytes(need));
         }
         add(4 * (size_t)r.S); add(8 * (2 * (size_t)r.S + 1)); add(MF * d4b);
