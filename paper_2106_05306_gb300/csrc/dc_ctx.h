@@ -8,6 +8,7 @@
 
 #include <algorithm>
 #include <functional>
+#include <cstring>
 #include <string>
 #include <vector>
 
@@ -229,6 +230,25 @@ dc_status upload(dc_ctx* c, Pool& pool, T** p, const std::vector<T>& h) {
     }
     return DC_OK;
 }
+
+// Several arrays in one allocation and one copy: each of them on its own costs a call to
+// the driver and, on a context with a stream-ordered pool, a wait for its copy.
+struct PackedUpload {
+    std::vector<char> host;
+    char* dev = nullptr;
+    template <class T>
+    size_t put(const std::vector<T>& v) {
+        const size_t at = (host.size() + 127) / 128 * 128;
+        host.resize(at + std::max<size_t>(v.size() * sizeof(T), 32));
+        if (!v.empty()) std::memcpy(host.data() + at, v.data(), v.size() * sizeof(T));
+        return at;
+    }
+    dc_status send(dc_ctx* c, Pool& pool) { return upload(c, pool, &dev, host); }
+    template <class T>
+    const T* get(size_t at) const {
+        return reinterpret_cast<const T*>(dev + at);
+    }
+};
 
 inline void free_pool(dc_ctx* c, Pool& pool) {
     for (void* p : pool.ptrs) {

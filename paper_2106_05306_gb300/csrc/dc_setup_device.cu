@@ -493,14 +493,7 @@ dc_status upload_params(dc_ctx* c, ParamPrep& pp) {
     fd.pr_coef = d_pcoef;
     fd.tau = d_tau;
     fd.sn_inst = d_sninst;
-    int2* d_tasks;
-    {
-        std::vector<int2> tasks;
-        ff_plan(frm, c->fplan, tasks);
-        if ((s = upload(c, F, &d_tasks, tasks))) return s;
-    }
-    fd.tasks = d_tasks;
-    // tree-scheduled solves: the fronts in a topological order (children first);
+    // tile lists of the factorisation, and the tree-scheduled solves: the fronts in a topological order (children first);
     // DC_LEVEL_SOLVES=1 in the environment selects one launch per tree level
     // instead (same results)
     {
@@ -514,26 +507,26 @@ dc_status upload_params(dc_ctx* c, ParamPrep& pp) {
         ms_plan(frm, tq_sn, ftask, btask, need);
         std::vector<int> cneed;
         for (int ch : frm.child) cneed.push_back(need[ch].x);
-        int *d_parent, *d_sched, *d_pull_off, *d_pull_ptr, *d_pull_idx, *d_cneed;
-        int4 *d_ftask, *d_btask, *d_need;
-        if ((s = upload(c, F, &d_cneed, cneed))) return s;
-        if ((s = upload(c, F, &d_ftask, ftask)) || (s = upload(c, F, &d_btask, btask)) ||
-            (s = upload(c, F, &d_need, need)) || (s = upload(c, F, &d_parent, frm.parent)) ||
-            (s = dalloc(c, F, &d_sched, 4 * (size_t)frm.S + 2)) || (s = dalloc(c, F, &fd.yvec, n3)) ||
-            (s = upload(c, F, &d_pull_off, pull_off)) ||
-            (s = upload(c, F, &d_pull_ptr, pull_ptr)) || (s = upload(c, F, &d_pull_idx, pull_idx)))
+        std::vector<int2> tasks;
+        ff_plan(frm, c->fplan, tasks);
+        PackedUpload up;
+        const size_t a_tasks = up.put(tasks), a_ftask = up.put(ftask), a_btask = up.put(btask), a_need = up.put(need),
+                     a_cneed = up.put(cneed), a_parent = up.put(frm.parent), a_off = up.put(pull_off),
+                     a_ptr = up.put(pull_ptr), a_idx = up.put(pull_idx);
+        if ((s = up.send(c, F)) || (s = dalloc(c, F, &fd.sched, 4 * (size_t)frm.S + 2)) ||
+            (s = dalloc(c, F, &fd.yvec, n3)))
             return s;
-        fd.pull_off = d_pull_off;
-        fd.pull_ptr = d_pull_ptr;
-        fd.pull_idx = d_pull_idx;
+        fd.tasks = up.get<int2>(a_tasks);
+        fd.pull_off = up.get<int>(a_off);
+        fd.pull_ptr = up.get<int>(a_ptr);
+        fd.pull_idx = up.get<int>(a_idx);
         fd.n_ftask = (int)ftask.size();
         fd.n_btask = (int)btask.size();
-        fd.ftask = d_ftask;
-        fd.btask = d_btask;
-        fd.need = d_need;
-        fd.cneed = d_cneed;
-        fd.parent = d_parent;
-        fd.sched = d_sched;
+        fd.ftask = up.get<int4>(a_ftask);
+        fd.btask = up.get<int4>(a_btask);
+        fd.need = up.get<int4>(a_need);
+        fd.cneed = up.get<int>(a_cneed);
+        fd.parent = up.get<int>(a_parent);
         fd.fault = c->counters + 3;
         fd.tree = std::getenv("DC_LEVEL_SOLVES") ? 0 : 1;
         fd.few = frm.S <= MS_FEW;
@@ -596,8 +589,6 @@ dc_status upload_params(dc_ctx* c, ParamPrep& pp) {
             c->ps_nsmall[l] = pos - c->ps_lvl_ptr[l] - c->ps_nbig[l];
         }
         c->ps_lvl_ptr[nl] = pos;
-        int* d_psn;
-        if ((s = upload(c, F, &d_psn, psn))) return s;
         std::vector<int> tq_ptr, tq_sn;
         dc_build_tree_items(frm, tq_ptr, tq_sn);
         std::vector<int> pull_off, pull_ptr, pull_idx;
@@ -605,37 +596,32 @@ dc_status upload_params(dc_ctx* c, ParamPrep& pp) {
         std::vector<int4> ftask, btask, need;
         int kind = 0, width = 0;
         dc_build_ps_tasks(frm, tq_ptr, tq_sn, ftask, btask, need, kind, width);
-        int *d_tq_sn, *d_sched, *d_pull_off, *d_pull_ptr, *d_pull_idx;
-        int4 *d_ftask, *d_btask, *d_need;
-        d4* d_wbuf;
-        if ((s = upload(c, F, &d_ftask, ftask)) || (s = upload(c, F, &d_btask, btask)) ||
-            (s = upload(c, F, &d_need, need)) || (s = upload(c, F, &d_tq_sn, tq_sn)) ||
-            (s = dalloc(c, F, &d_wbuf, (size_t)std::max(MF, 1))) ||
-            (s = dalloc(c, F, &d_sched, 2 * (2 * (size_t)frm.S + 1))) || (s = upload(c, F, &d_pull_off, pull_off)) ||
-            (s = upload(c, F, &d_pull_ptr, pull_ptr)) || (s = upload(c, F, &d_pull_idx, pull_idx)))
-            return s;
         PSolveDev& ps = dm.ps;
+        PackedUpload up;
+        const size_t a_ftask = up.put(ftask), a_btask = up.put(btask), a_need = up.put(need), a_tq = up.put(tq_sn),
+                     a_sn = up.put(psn), a_off = up.put(pull_off), a_ptr = up.put(pull_ptr), a_idx = up.put(pull_idx);
+        if ((s = up.send(c, F)) || (s = dalloc(c, F, &ps.wbuf, (size_t)std::max(MF, 1))) ||
+            (s = dalloc(c, F, &ps.sched, 2 * (2 * (size_t)frm.S + 1))))
+            return s;
         ps.S = frm.S;
         ps.n_ftask = (int)ftask.size();
         ps.n_btask = (int)btask.size();
-        ps.ftask = d_ftask;
-        ps.btask = d_btask;
-        ps.need = d_need;
-        ps.wbuf = d_wbuf;
+        ps.ftask = up.get<int4>(a_ftask);
+        ps.btask = up.get<int4>(a_btask);
+        ps.need = up.get<int4>(a_need);
         ps.kind = kind;
         ps.width = width;
         ps.parent = fd.parent;
-        ps.tq_sn = d_tq_sn;
-        ps.sched = d_sched;
-        ps.pull_off = d_pull_off;
-        ps.pull_ptr = d_pull_ptr;
-        ps.pull_idx = d_pull_idx;
+        ps.tq_sn = up.get<int>(a_tq);
+        ps.pull_off = up.get<int>(a_off);
+        ps.pull_ptr = up.get<int>(a_ptr);
+        ps.pull_idx = up.get<int>(a_idx);
         ps.fault = c->counters + 3;
         ps.tree = fd.tree;
         // both sweeps of a global step in one launch (DC_SEPARATE_SWEEPS=1 in the
         // environment: two launches, for comparison; the same results)
         ps.fused = std::getenv("DC_SEPARATE_SWEEPS") ? 0 : 1;
-        ps.sn = d_psn;
+        ps.sn = up.get<int>(a_sn);
         ps.begin = d_begin;
         ps.f = d_f;
         ps.p = d_p;
