@@ -396,11 +396,12 @@ dc_status dc_debug_sweep_wait_timeout(dc_ctx* ctx, int32_t skip_items);
  * complement A22 - L21 D L21^T.  linv_out (host, p x p column-major, nullable)
  * receives the inverse of L's unit-lower pivot block.  use_tc: 1 updates trailing
  * blocks of 64 rows or more on the tensor cores (TF32 split in three passes, FP32
- * accumulation), 0 by FP32 FMA tiles.  threads (128, 256 or 512) and use_gscr named
- * variants of an earlier one-CTA kernel; they are checked as before and change
- * nothing else.  Synchronous; allocates its own device memory.  DC_ERR_INVALID
- * unless 1 <= p <= n <= 4096 (without use_gscr a front must also fit the 227 KB that
- * one CTA's panel took), DC_ERR_TIMEOUT if a tensor-core completion wait gave up,
+ * accumulation), 0 by FP32 FMA tiles.  threads (512, 256 or 128): the inverse of the
+ * pivot block in tasks of at most 32, 16 or 8 columns; use_gscr: 1 forms it in global
+ * memory (as for pivot blocks of more than 6144 unknowns).  The results are the same
+ * bits.  Synchronous; allocates its own device memory.  DC_ERR_INVALID
+ * unless 1 <= p <= n <= 4096 (without use_gscr a front's panel and 64 columns of the
+ * inverse must also fit 227 KB), DC_ERR_TIMEOUT if a tensor-core completion wait gave up,
  * DC_ERR_CUDA on a CUDA error; dc_last_error(NULL) has the message. */
 dc_status dc_debug_front_factor(int32_t n, int32_t p, const float* A, float* out, float* linv_out,
                                 int32_t threads, int32_t use_tc, int32_t use_gscr);

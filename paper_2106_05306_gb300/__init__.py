@@ -462,7 +462,9 @@ def fma_peak(precision=64, n_iter=None):
 
 def front_factor(A, p, threads=512, use_tc=True, use_gscr=False):
     """One dense front through the adjoint preconditioner's factorisation (a test
-    hook; threads and use_gscr are checked and change nothing): A is a symmetric (n, n) array, p the pivot count.  Returns (F, Linv):
+    hook): A is a symmetric (n, n) array, p the pivot count; threads (512, 256, 128) and
+    use_gscr choose how the pivot block's inverse is split (32, 16 or 8 columns a task, or
+    in global memory; the same bits).  Returns (F, Linv):
     F holds D and the unit-lower L in its first p columns and the Schur complement
     in its trailing lower triangle (float32, (n, n)); Linv is the inverse of L's
     pivot block ((p, p))."""

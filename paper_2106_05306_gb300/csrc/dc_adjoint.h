@@ -65,10 +65,11 @@ void adj_add_ext(d4* g, const double* ext, const int* int2ext, int m, int layout
 // Per-step multifrontal LDL^T preconditioner (dc_frontal.cu).
 // Numeric factorisation of the fronts (dc_front_factor.cu): the tile lists of its
 // launches, laid out once per front structure, and one factorisation.
-void ff_plan(const HostFronts& fr, FrontPlan& plan, std::vector<int2>& tasks, int tc = -1);
+void ff_plan(const HostFronts& fr, FrontPlan& plan, std::vector<int2>& tasks, int tc = -1, int cols = 32);
 cudaError_t ff_configure();
 void ff_factorize(const FrontDev& fd, const FrontPlan& plan, cudaStream_t s, KTimer* kt);
-dc_status ff_debug_factor(int n, int p, const float* A, float* out, float* linv_out, int tc, std::string* err);
+dc_status ff_debug_factor(int n, int p, const float* A, float* out, float* linv_out, int tc, int cols,
+                          std::string* err);
 size_t frontal_solve_smem(int max_f);
 // Raises the shared-memory limits of the solve kernels (fronts of up to max_f unknowns).
 cudaError_t frontal_configure(int max_f);

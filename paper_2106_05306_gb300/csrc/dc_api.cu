@@ -582,6 +582,8 @@ dc_status dc_get_instance_nonconverged(dc_ctx* c, int64_t* counts) {
     return DC_OK;
 }
 
+// The fronts the hook takes without use_gscr: a 32-column panel of the front, or 64 columns
+// of its inverse, and the update's operands in one CTA's shared memory.
 static size_t one_cta_front_bytes(int n, int p, bool tc) {
     const size_t panel = 2 * 32 * 33 + 32 + 32 * (((size_t)n + 7) / 8 * 8), inverse = 64 * ((size_t)p + 1) + 1024;
     return ((tc ? 12288 : 0) + std::max(panel, inverse)) * sizeof(float) + 64;
@@ -596,7 +598,7 @@ dc_status dc_debug_front_factor(int32_t n, int32_t p, const float* A, float* out
     else if (!use_gscr && one_cta_front_bytes(n, p, use_tc != 0) > 227 * 1024)
         err = "dc_debug_front_factor: front too large for shared memory; set use_gscr";
     else
-        st = ff_debug_factor(n, p, A, out, linv_out, use_tc, &err);
+        st = ff_debug_factor(n, p, A, out, linv_out, use_tc, use_gscr ? 0 : threads / 16, &err);
     if (st != DC_OK) g_create_err = err;
     return st;
 }

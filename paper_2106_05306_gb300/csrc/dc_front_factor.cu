@@ -434,6 +434,8 @@ __global__ void __launch_bounds__(256) k_ff_inverse(FrontDev fd, const int2* __r
             if (r >= ch + c) {
                 F[(long)(k1 + ch + c) * f + k1 + r] = *w;
                 *w = b;
+            } else if (!SX) {
+                *w = 0.0f;                 // (read back with the column's other rows)
             }
             if (SX) xsm[r * CW + c] = b;
         } else if (SX && r < jb) {
@@ -507,10 +509,10 @@ inline int cdiv(int a, int b) { return (a + b - 1) / b; }
 
 }  // namespace
 
-// The columns of X a k_ff_inverse CTA takes for a pivot block of p unknowns: 32, 16 or 8
-// while they fit its shared memory, else 8 without (returns 0).
-static int ff_inverse_cols(int p) {
-    for (int cw = 32; cw >= 8; cw /= 2)
+// The columns of X a k_ff_inverse CTA takes for a pivot block of p unknowns: 32, 16 or 8 (at
+// most `most`) while they fit its shared memory, else 8 without (returns 0).
+static int ff_inverse_cols(int p, int most) {
+    for (int cw = most; cw >= 8; cw /= 2)
         if ((size_t)cw * p * sizeof(float) <= 192 * 1024) return cw;
     return 0;
 }
@@ -526,8 +528,9 @@ static bool ff_level_tc(int max_f) {
 }
 
 // Tile lists of every level's launches, in launch order.  tc: -1 by the level's largest
-// front, 0 / 1 forced (tests).
-void ff_plan(const HostFronts& fr, FrontPlan& pl, std::vector<int2>& tasks, int tc) {
+// front, 0 / 1 forced; cols: the most columns of an inverse task, 0 for its form without
+// shared memory (both for tests).
+void ff_plan(const HostFronts& fr, FrontPlan& pl, std::vector<int2>& tasks, int tc, int cols) {
     pl = FrontPlan();
     tasks.clear();
     const int nl = (int)fr.lvl_ptr.size() - 1;
@@ -576,7 +579,7 @@ void ff_plan(const HostFronts& fr, FrontPlan& pl, std::vector<int2>& tasks, int 
         for (int cw : {32, 16, 8, 0}) {
             for (int q = q0; q < q1; ++q) {
                 const int s = fr.lvl_sn[q], p = fr.p[s];
-                if (ff_inverse_cols(p) != cw) continue;
+                if (ff_inverse_cols(p, cols) != cw) continue;
                 const int w = std::max(cw, 8);
                 for (int J = 0; J * PB < p; ++J)
                     for (int c = 0; c * w < std::min(PB, p - J * PB); ++c) tasks.push_back(make_int2(s, (J << 8) | c));
@@ -586,7 +589,7 @@ void ff_plan(const HostFronts& fr, FrontPlan& pl, std::vector<int2>& tasks, int 
                 pl.launches.back().k == cw) {
                 int p = 0;
                 for (int q = q0; q < q1; ++q)
-                    if (ff_inverse_cols(fr.p[fr.lvl_sn[q]]) == cw) p = std::max(p, fr.p[fr.lvl_sn[q]]);
+                    if (ff_inverse_cols(fr.p[fr.lvl_sn[q]], cols) == cw) p = std::max(p, fr.p[fr.lvl_sn[q]]);
                 pl.launches.back().smem = cw * p * (int)sizeof(float);
             }
         }
@@ -633,7 +636,8 @@ void ff_factorize(const FrontDev& fd, const FrontPlan& pl, cudaStream_t s, KTime
 
 // One dense front through the factorisation: the test hook behind
 // dc_debug_front_factor (synchronous; allocates and frees its own buffers).
-dc_status ff_debug_factor(int n, int p, const float* A, float* out, float* linv_out, int tc, std::string* err) {
+dc_status ff_debug_factor(int n, int p, const float* A, float* out, float* linv_out, int tc, int cols,
+                          std::string* err) {
     if (!A || !out) {
         *err = "dc_debug_front_factor: null A or out";
         return DC_ERR_INVALID;
@@ -647,7 +651,7 @@ dc_status ff_debug_factor(int n, int p, const float* A, float* out, float* linv_
     fr.lvl_sn = {0};
     FrontPlan pl;
     std::vector<int2> tasks;
-    ff_plan(fr, pl, tasks, tc != 0);
+    ff_plan(fr, pl, tasks, tc != 0, cols);
     const int nbk = cdiv(p, PB);
     // device image: ints [f, p, cptr0, cptr1], long longs [off, binv_off, linv_off]
     int hi[4] = {n, p, 0, 0};
@@ -670,7 +674,7 @@ dc_status ff_debug_factor(int n, int p, const float* A, float* out, float* linv_
             (e = cudaMemcpy(dt, tasks.data(), sizeof(int2) * tasks.size(), cudaMemcpyHostToDevice)) ||
             (e = cudaMemcpy(dtau, &tau, sizeof(float), cudaMemcpyHostToDevice)) ||
             (e = cudaMemcpy(pool, A, sizeof(float) * (size_t)n * n, cudaMemcpyHostToDevice)) ||
-            (e = cudaMemset(linv, 0, sizeof(float) * (size_t)p * p)))
+            (e = cudaMemset(linv, 0xff, sizeof(float) * (size_t)p * p)))   // NaNs: nothing there may be read
             break;
         FrontDev fd{};
         fd.S = 1;
@@ -692,7 +696,10 @@ dc_status ff_debug_factor(int n, int p, const float* A, float* out, float* linv_
         if ((e = cudaMemcpy(&fl, fault, sizeof(fl), cudaMemcpyDeviceToHost)) ||
             (e = cudaMemcpy(out, pool, sizeof(float) * (size_t)n * n, cudaMemcpyDeviceToHost)))
             break;
-        if (linv_out) e = cudaMemcpy(linv_out, linv, sizeof(float) * (size_t)p * p, cudaMemcpyDeviceToHost);
+        if (linv_out) {
+            e = cudaMemcpy(linv_out, linv, sizeof(float) * (size_t)p * p, cudaMemcpyDeviceToHost);
+            for (int c = 0; c < p; ++c) std::fill(linv_out + (size_t)c * p, linv_out + (size_t)c * p + c, 0.0f);
+        }
     } while (false);
     cudaFree(di);
     cudaFree(dl);
