@@ -76,23 +76,11 @@ FP32_DERIVED_TFLOPS = SMS * FP32_LANES * 2 * SM_MAX_MHZ * 1e6 / 1e12
 FP64_DERIVED_TFLOPS = 1.25
 HBM_FALLBACK_GBS = 6800.0
 
-# DRAM read + write bytes per launch measured by ncu on this workload (the
-# kernel-traffic profile; null once the kernel's source file has changed).
-# DRAM read + write per full-size launch from one ncu capture of the 256-cloth batch
-# (profiles/kernel_traffic_batched_256cloths.md), valid while the kernel's source
-# file is the one measured (its hash).
-TRAFFIC = {
-    "front": {"source": "dc_front_factor.cu", "source_sha": "d56e13ad7997eba6", "bytes_per_launch": 945.14e6,
-              "note": "ncu dram__bytes_read.sum + dram__bytes_write.sum, mean of the 9 levels of one "
-                      "factorisation, 256 cloths (profiles/kernel_traffic_batched_256cloths.md)"},
-    "sweeps": {"source": "dc_kernels.cu", "source_sha": "232ea24582784521", "bytes_per_launch": 747.46e6,
-               "note": "ncu dram__bytes_read.sum + dram__bytes_write.sum per launch, 256 cloths "
-                       "(profiles/kernel_traffic_batched_256cloths.md)"},
-    "local": {"source": "dc_kernels.cu", "source_sha": "232ea24582784521", "bytes_per_launch": 182.29e6,
-              "note": "ncu, 256 cloths (profiles/kernel_traffic_batched_256cloths.md)"},
-    "gather": {"source": "dc_kernels.cu", "source_sha": "232ea24582784521", "bytes_per_launch": 149.42e6,
-               "note": "ncu, 256 cloths (profiles/kernel_traffic_batched_256cloths.md)"},
-}
+# DRAM read + write bytes per launch from an ncu capture of this workload, by kernel class:
+# {"source": file under csrc/, "source_sha": first 16 digits of its SHA-256 when captured,
+# "bytes_per_launch", "note"}.  Null once the source file has changed; the captures in
+# profiles/kernel_traffic_batched_256cloths.md are of earlier kernels.
+TRAFFIC = {}
 
 
 def parse_args(argv=None):
@@ -561,7 +549,7 @@ KERNEL_CLASSES = {
     "solve_fwd": "k_ps_fwd_tree (forward supernodal sweep, FP64, 3 columns)",
     "solve_bwd": "k_ps_bwd_tree (backward sweep + fused per-node Signorini-Coulomb solve)",
     "front": "k_ff_* (one level of the FP32 multifrontal LDL^T of the adjoint preconditioner: extend, panels, updates, inverse)",
-    "msolve": "k_msolve_fwd_tree / k_msolve_bwd_tree (preconditioner solves)",
+    "msolve": "k_msolve_tree (preconditioner solves, forward and backward)",
     "krylov": "k_bmdot / k_breduce / k_bvupdate / k_bscale (GMRES vectors)",
     "apply_h": "k_adj_elem + k_adj_gather (matrix-free adjoint operator)",
     "assemble": "adjoint per-step setup and front assembly",

@@ -75,7 +75,7 @@ size_t frontal_solve_smem(int max_f);
 cudaError_t frontal_configure(int max_f);
 // Launch shape of the tree-scheduled solve for fronts of at most max_f unknowns: the
 // CTAs that fit on the device at once, and the dynamic shared memory.
-constexpr int MS_FEW = 24 * 152;   // fronts of a context whose solves load ahead (dc_frontal.cu)
+constexpr int MS_FEW = 24 * DC_SMS;   // fronts of a context whose solves load ahead (dc_frontal.cu)
 cudaError_t frontal_tree_grid(int max_f, bool few, int* grid, size_t* smem);
 // Its tasks; order: the fronts in topological order, farthest from their root first.
 void ms_plan(const HostFronts& fr, const std::vector<int>& order, std::vector<int4>& ftask, std::vector<int4>& btask,

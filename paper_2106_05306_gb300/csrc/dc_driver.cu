@@ -760,7 +760,7 @@ dc_status adjoint_step(dc_ctx* c, const d4* x_n, const d4* x1, const d4* v1, int
 // Block-size autotuner: times the local-step, gather, per-node and adjoint
 // element kernels at 64..512 threads per block on this context's mesh (rest
 // state, zero velocity) and keeps the fastest of each.  The launch shape of
-// these kernels changes no result (one thread per element or node).
+// these kernels changes no result (an element's or node's threads are one warp's).
 dc_status autotune(dc_ctx* c) {
     RET(ensure_adjoint(c));
     cudaStream_t s = c->stream;

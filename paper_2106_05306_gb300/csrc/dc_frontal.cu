@@ -523,7 +523,9 @@ __global__ void __launch_bounds__(FT) k_msolve_bwd(FrontDev fd, const int* __res
 // and the first entries of its rows before the wait and the second product's during the
 // first.  That takes 64 registers, two CTAs an SM, which many fronts cannot spare.
 // Measured, without -> with (us, gradient calls): 256-node cloth 14400 -> 13500, 61 x 61 nodes
-// 21400 -> 20000, 200 x 200 nodes 49800 -> 47300; 96 cloths 47600 -> 49200.
+// 21400 -> 20000, 200 x 200 nodes 49800 -> 47300; batches of 8 cloths of 16 x 16 nodes 6255 ->
+// 6090, 4 of 32 x 32 9720 -> 9330, 16 of 24 x 24 9210 -> 9130, 12 of 40 x 40 15450 both; 96 cloths
+// 47600 -> 49200.
 constexpr int MT = 512;
 
 template <bool FWD, bool FEW>
@@ -664,7 +666,7 @@ void ms_plan(const HostFronts& fr, const std::vector<int>& order, std::vector<in
              std::vector<int4>& need) {
     long long total = 0;
     for (int s = 0; s < fr.S; ++s) total += (long long)fr.p[s] * (fr.p[s] + 1) / 2 + (long long)fr.p[s] * (fr.f[s] - fr.p[s]);
-    const long long target = std::min<long long>(65536, std::max<long long>(4096, total / (152 * 16)));
+    const long long target = std::min<long long>(65536, std::max<long long>(4096, total / (DC_SMS * 16)));
     need.assign(fr.S, make_int4(1, 0, 1, 0));
     ftask.clear();
     btask.clear();

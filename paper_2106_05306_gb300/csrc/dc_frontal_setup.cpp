@@ -304,8 +304,6 @@ void dc_merge_psolve(const std::vector<HostPSolve>& P, HostPSolve& out) {
     out.n_pant = to;
 }
 
-constexpr int SMS = 152;
-
 // Work items of the tree-scheduled sweeps, in a topological order (every front
 // after its children): fronts farther from their root come first, so the longest
 // remaining chains start earliest.  A front of more than DC_PS_SMALL nodes is an
@@ -347,7 +345,7 @@ void dc_build_tree_items(const HostFronts& fr, std::vector<int>& tq_ptr, std::ve
 // barriers hold fewer warps (one solve of 48 / 64 cloths of 40 x 40 nodes, four CTAs -> eight: 282
 // -> 300 / 298 -> 307 us, with three such batches 165 -> 122 / 234 -> 157).
 int ps_kind(int n_fronts) {
-    return n_fronts <= 8 * SMS ? PS_KIND_NARROW : n_fronts <= 40 * SMS ? PS_KIND_WIDE : PS_KIND_MANY;
+    return n_fronts <= 8 * DC_SMS ? PS_KIND_NARROW : n_fronts <= 40 * DC_SMS ? PS_KIND_WIDE : PS_KIND_MANY;
 }
 
 // Tasks of the tree-scheduled supernodal sweeps, fronts farthest from their root
@@ -377,7 +375,7 @@ void dc_build_ps_tasks(const HostFronts& fr, const std::vector<int>& tq_ptr, con
         const long long ns = fr.p[s] / 3, nu = fr.f[s] / 3 - ns;
         total += ns * (ns + 1) / 2 + ns * nu;
     }
-    const long long target = std::min<long long>(8192, std::max<long long>(1600, total / (SMS * 32)));
+    const long long target = std::min<long long>(8192, std::max<long long>(1600, total / (DC_SMS * 32)));
     kind = ps_kind(fr.S);
     width = 0;
     need.assign(fr.S, make_int4(1, 0, 1, 0));

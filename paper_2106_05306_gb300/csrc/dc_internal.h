@@ -136,8 +136,10 @@ void dc_build_pull_lists(const HostFronts& fr, const std::vector<int>& aoff, int
 // Supernodal substitution: fronts of at most this many nodes are solved by one
 // warp each, larger ones by a whole CTA.
 constexpr int DC_PS_SMALL = 64;
-// small fronts solved together by one CTA (one per warp)
+// small fronts solved together by one CTA at most (one per warp)
 constexpr int DC_PS_WARPS = 8;
+// SMs of a GB300, for the task sizes laid out on the host (the grids ask the device)
+constexpr int DC_SMS = 152;
 // Kernel of the tree-scheduled sweeps: three CTAs of 256 threads an SM, four, or eight of
 // 128 threads.
 enum { PS_KIND_NARROW = 0, PS_KIND_WIDE = 1, PS_KIND_MANY = 2 };

@@ -1,6 +1,6 @@
-// Dependency waits between CTAs of one launch (tree-scheduled sweeps).  A flag
-// is published with a release store after the producer's data, read with an
-// acquire load, and every wait is bounded: after DC_SPIN_LIMIT polls it sets the
+// Dependency waits between CTAs of one launch (tree-scheduled sweeps).  A counter of
+// finished tasks is added to with a release reduction after the producer's data and read
+// with an acquire load, and every wait is bounded: after DC_SPIN_LIMIT polls it sets the
 // launch's sticky fault word and gives up, so that no kernel can hang the GPU.
 #pragma once
 
@@ -10,9 +10,6 @@ static __device__ __forceinline__ int dc_ld_acquire(const int* p) {
     int v;
     asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
-}
-static __device__ __forceinline__ void dc_st_release(int* p, int v) {
-    asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 static __device__ __forceinline__ bool dc_fault_set(const unsigned long long* fault) {
     return *reinterpret_cast<const volatile unsigned long long*>(fault) != 0ull;
@@ -31,8 +28,4 @@ static __device__ bool dc_wait_count(const int* count, int target, unsigned long
     }
     atomicExch(fault, 1ull);
     return false;
-}
-// Waits until *flag is nonzero.
-static __device__ __forceinline__ bool dc_wait_flag(const int* flag, unsigned long long* fault) {
-    return dc_wait_count(flag, 1, fault);
 }
