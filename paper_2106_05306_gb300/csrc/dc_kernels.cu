@@ -1087,7 +1087,9 @@ cudaError_t psolve_configure(int max_fs) {
 // ready task polls and keeps its part of an SM from other streams' kernels.  Measured against
 // every CTA that fits: three 45 x 45 cloths on streams of their own (a stage has at most 48
 // fronts), two steps 5.28 -> 2.44 ms each, one of them alone 6.8 -> 7.0; three batches of 64 cloths
-// of 40 x 40 nodes 13.7 -> 9.8, one of them 15.3 -> 15.5.
+// of 40 x 40 nodes 13.7 -> 9.8, one of them 15.3 -> 15.5.  A stage of twice the places or more
+// takes them all: 256 cloths of 40 x 40 nodes, three quarters -> all, one batch 39.1 -> 36.1 ms, three
+// 33.2 -> 34.6 ms each.
 cudaError_t psolve_tree_grid(int max_fs, int kind, int width, int* grid, size_t* smem_out) {
     const int nt = ps_tree_threads(kind);
     const size_t smem = std::max((6 * (size_t)max_fs + 3 * (size_t)ps_pass_rows(nt) * GV_MAXG) * sizeof(double),
@@ -1099,7 +1101,8 @@ cudaError_t psolve_tree_grid(int max_fs, int kind, int width, int* grid, size_t*
     if (e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, PS_PICK(k_ps_sweeps_tree, kind), nt, smem);
     if (e != cudaSuccess) return e;
-    const int fit = sms * std::max(1, n), wide = kind == PS_KIND_NARROW ? fit : fit / 4 * 3;
+    const int fit = sms * std::max(1, n);
+    const int wide = kind == PS_KIND_NARROW || width >= 2 * fit ? fit : fit / 4 * 3;
     *grid = std::max(1, std::min(wide, width <= 128 ? width : std::max(128, width / 4 * 3)));
     return cudaSuccess;
 }
