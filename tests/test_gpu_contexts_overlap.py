@@ -1,8 +1,8 @@
 """Contexts on streams of their own share the GPU: three cloths' rollouts replayed as graphs, none
 of which fills the chip, take together less than three in turn would (as every launch takes only
 the CTAs its tree has tasks for), and give each cloth's own bits.  A context that takes every
-SM for its waiting CTAs makes the three nearly as slow as in turn (0.78 of it on 45 x 45
-nodes, where sharing gives 0.34)."""
+SM for its waiting CTAs makes the three nearly as slow as in turn (0.88 of it on 45 x 45
+nodes; with the CTAs a tree has use for it is 0.35)."""
 import time
 
 import pytest
